@@ -164,6 +164,7 @@ struct DeviceTables {
   size_t esz;
   void *K;
   void *Kperm;  // K[m1][k2(p2)][k3(p3)]: axes 2 and 3 in the plane passes' output positions
+  void *Klp;    // FP32: the table in the line-pair chain's layout (null without a plan for the grid)
   void *tw[3];
 };
 std::mutex g_tab_mu;
@@ -213,6 +214,16 @@ cudaError_t get_tables(int dev, const ace_desc &d, cudaStream_t st, const Device
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(t.Kperm, Kp.data(), sizeof(T) * Kp.size(), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return e;
+  if constexpr (sizeof(T) == 4) {
+    ace::PlaneOps<float> lp{};
+    if (ace::line_pair_ops(d.n[0], d.n[1], d.n[2], &lp)) {
+      e = cudaMalloc(&t.Klp, 2 * sizeof(float) * (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2));
+      if (e != cudaSuccess) return e;
+      e = ace::launch_line_pair_table(static_cast<const float *>(t.K), d.n[0], d.n[1], d.n[2],
+                                      static_cast<float *>(t.Klp), st);
+      if (e != cudaSuccess) return e;
+    }
+  }
   std::vector<cpx<T>> twh[3];
   for (int a = 0; a < 3; ++a) {
     const int L = d.n[a];
@@ -467,15 +478,16 @@ bool find_persist_ops<double>(int, int, int, ace::PersistOps<double> *) {
   return false;
 }
 
+// Plane-chain passes of a grid (false: the grid takes the five pencil passes).
 template <typename T>
-bool find_plane_ops(int n2, int n3, ace::PlaneOps<T> *out);
+bool find_plane_ops(const ace_desc &d, ace::PlaneOps<T> *out);
 template <>
-bool find_plane_ops<float>(int n2, int n3, ace::PlaneOps<float> *out) {
-  return ace::plane_ops_f32_small(n2, n3, out) || ace::plane_ops_f32_large(n2, n3, out);
+bool find_plane_ops<float>(const ace_desc &d, ace::PlaneOps<float> *out) {
+  return ace::line_pair_ops(d.n[0], d.n[1], d.n[2], out);
 }
 template <>
-bool find_plane_ops<double>(int n2, int n3, ace::PlaneOps<double> *out) {
-  return ace::plane_ops_f64(n2, n3, out);
+bool find_plane_ops<double>(const ace_desc &d, ace::PlaneOps<double> *out) {
+  return ace::conv_length_supported(d.n[0]) && ace::plane_ops_f64(d.n[1], d.n[2], out);
 }
 
 // Run-time parameters of the plane chain: packs per CTA group (G), packs per batch (B), side
@@ -545,6 +557,15 @@ void tune_store(const TuneKey &k, const ChainParams &c) {
 
 ChainParams chain_params(const ace_desc &d, bool fp64) {
   ChainParams c;
+  if (!fp64) {
+    // Mixed form: packs per batch such that the scratch of all side streams takes about 60 MB (half
+    // the L2; what the sweep of batch sizes and streams picked on every grid from 32^3 to
+    // 160x144x128, within 3%), at most 16; three streams for packs above 18 MB.  Against the fixed 2
+    // packs on 4 streams: 32^3 0.23 -> 0.08 ms per chain, 64^3 2.9 -> 1.6 ms, 128^3 40.0 -> 36.4 ms.
+    const double pack = 8.0 * d.n[0] * d.n[1] * d.n[2];
+    c.streams = pack > 18e6 ? 3 : 4;
+    c.B = std::min(16, std::max(1, (int)std::lround(60e6 / (c.streams * pack))));
+  }
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_file_load_locked();
@@ -840,8 +861,9 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
   const long long N = op->N;
   cudaStream_t st = op->stream;
   const int G = cp.G;
-  const int B = std::max(G, cp.B);
   const int nstreams = std::min(kSide, std::max(1, cp.streams));
+  // few packs: smaller batches, so that every side stream has one
+  const int B = std::max(G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams));
   const bool acc = pops.acc_fits && G > 1;
   std::vector<int4> packs;
   std::vector<int4> groups;
@@ -895,7 +917,10 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
   std::vector<int4> up(packs);
   up.insert(up.end(), groups.begin(), groups.end());
   ACE_CUDA(host_upload(op, packs_d, up.data(), sizeof(int4) * up.size(), st), "pack upload");
-  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<T>) * (size_t)N * B * nstreams, st), "alloc scratch");
+  // complex values of one pack in the scratch (FP32: 16-byte units of two lines of axis 2)
+  const size_t pack_elems =
+      sizeof(T) == 4 ? (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2) * 2 : (size_t)N;
+  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<T>) * pack_elems * B * nstreams, st), "alloc scratch");
   temps.push_back(tmp);
   cpx<T> *scratch_all = static_cast<cpx<T> *>(tmp);
   // plane maxima for the plane skip (mixed form), on st before the side streams fork from it
@@ -925,8 +950,8 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
   const int persist_mb = cp.persist_mb;
   if (persist_mb > 0 && nstreams > 1) {
     for (int k = 0; k < nstreams; ++k)
-      l2_window(side[k], op->dev, scratch_all + (size_t)k * B * N,
-                std::min<size_t>(((size_t)persist_mb << 20) / (size_t)nstreams, sizeof(cpx<T>) * (size_t)B * (size_t)N),
+      l2_window(side[k], op->dev, scratch_all + (size_t)k * B * pack_elems,
+                std::min<size_t>(((size_t)persist_mb << 20) / (size_t)nstreams, sizeof(cpx<T>) * (size_t)B * pack_elems),
                 persist_mb);
   }
 
@@ -940,6 +965,8 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
   pa.tw3 = static_cast<const cpx<T> *>(tab->tw[2]);
   pa.N = N;
   pa.n1 = d.n[0];
+  pa.n2 = d.n[1];
+  pa.n3 = d.n[2];
   pa.hints = env_int("ACE_L2_HINTS", 1);
   pa.pmax = skip_rel > 0.f ? op->pmax : nullptr;
   pa.gmax = skip_rel > 0.f ? op->gmax : nullptr;
@@ -949,7 +976,7 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
   ca.W = static_cast<T *>(op->W);
   ca.scratch = scratch_all;
   ca.packs = packs_d;
-  ca.kernel = static_cast<const T *>(tab->Kperm);
+  ca.kernel = static_cast<const T *>(sizeof(T) == 4 ? tab->Klp : tab->Kperm);
   ca.tw = static_cast<const cpx<T> *>(tab->tw[0]);
   ca.N = N;
   ca.n1 = d.n[0];
@@ -962,15 +989,20 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
     const int k = (int)(bi % nstreams);
     const int p0 = groups[b.x].x;
     const int p1 = groups[b.y - 1].x + groups[b.y - 1].y;
-    pa.scratch = scratch_all + (size_t)k * B * N;
+    pa.scratch = scratch_all + (size_t)k * B * pack_elems;
     ca.scratch = pa.scratch;
     pa.pack0 = p0;
     pa.batch0 = p0;
     pa.group0 = b.x;
     ca.pack0 = p0;
     ACE_CUDA(pops.fwd(pa, p1 - p0, side[k]), "plane forward");
-    ACE_CUDA(ace::launch_conv_pass<T>(ca, p1 - p0, side[k]), "pencil pass");
-    ACE_CUDA(pops.inv(pa, b.y - b.x, acc_on, side[k]), "plane inverse");
+    if constexpr (sizeof(T) == 4) {
+      ACE_CUDA(ace::launch_line_pair_conv(ca, p1 - p0, side[k]), "pencil pass");
+      ACE_CUDA(pops.inv(pa, p1 - p0, false, side[k]), "plane inverse");
+    } else {
+      ACE_CUDA(ace::launch_conv_pass<T>(ca, p1 - p0, side[k]), "pencil pass");
+      ACE_CUDA(pops.inv(pa, b.y - b.x, acc_on, side[k]), "plane inverse");
+    }
     op->launches += 3;
     if (rounds_on && nstreams > 1 && round_end[bi]) {
       // every stream waits for every other one: the next round starts after this one ends
@@ -1241,8 +1273,7 @@ ace_status run_chain(ace_op *op, const T *phi, int count) {
   ACE_CUDA(cudaMemsetAsync(op->W, 0, op->esz * (size_t)op->n * op->N, op->stream), "zero W");
   ace::PlaneOps<T> pops{};
   ace::PersistOps<T> qops{};
-  const bool plane = find_plane_ops<T>(d.n[1], d.n[2], &pops) && ace::conv_length_supported(d.n[0]) &&
-                     env_int("ACE_FORCE_PENCIL", 0) == 0;
+  const bool plane = find_plane_ops<T>(d, &pops) && env_int("ACE_FORCE_PENCIL", 0) == 0;
   const ChainParams cp = chain_params(d, op->fp64);
   const bool persistent = plane && cp.persistent && find_persist_ops<T>(d.n[0], d.n[1], d.n[2], &qops);
   if (count > 0 && persistent) {
@@ -2200,8 +2231,7 @@ ace_status ace_autotune(const ace_desc *desc, const void *phi, ace_dtype dtype, 
   auto run = [&](auto tag) -> ace_status {
     using T = decltype(tag);
     ace::PlaneOps<T> pops{};
-    if (count == 0 || !find_plane_ops<T>(desc->n[1], desc->n[2], &pops) || !ace::conv_length_supported(desc->n[0]))
-      return ACE_OK;  // nothing to tune
+    if (count == 0 || !find_plane_ops<T>(*desc, &pops)) return ACE_OK;  // nothing to tune
     ACE_CUDA(op_alloc(op, &op->W, op->esz * (size_t)op->n * op->N), "alloc W");
     const T *phi_w = static_cast<const T *>(op->phi_work);
     // a sample long enough (about 40% of a 128-orbital build on 96^3) for the L2 reuse of the

@@ -33,8 +33,8 @@ struct PairPassArgs {
   const cpx<T> *tw;         // [L] e^{-2 pi i e / L} for the axis of this pass
   long long N;              // N1 N2 N3
   int n1, n2, n3;
-  int conv_tile;            // axis-1 pencil pass of the plane chain, FP32: 0 (32 columns, default
-                            // threads), 1 (32 columns, the other thread count), 2 (16 columns, 128)
+  int conv_tile;            // axis-1 pass of the FP32 plane chain: 0 (two warps of 8 line pairs a CTA), 1 (four
+                            // warps), 2 (two warps of 4 line pairs)
 };
 
 // Arguments of the three-pass (plane, pencil, plane) chain.
@@ -51,7 +51,7 @@ struct PlaneArgs {
   const cpx<T> *tw2;   // [N2] e^{-2 pi i e / N2}
   const cpx<T> *tw3;   // [N3] e^{-2 pi i e / N3}
   long long N;
-  int n1;
+  int n1, n2, n3;
   int hints;           // bit 0: drop each consumed scratch plane from L2 without writing it back
   const float *pmax;   // plane maxima [norb][n1] and orbital maxima [norb] for the plane skip
   const float *gmax;
@@ -62,12 +62,19 @@ struct PlaneArgs {
 template <typename T>
 struct PlaneOps {
   cudaError_t (*fwd)(const PlaneArgs<T> &, int npacks, cudaStream_t);
-  cudaError_t (*inv)(const PlaneArgs<T> &, int ngroups, bool acc, cudaStream_t);
+  // FP64: over groups [group0, group0 + count); FP32: over packs [pack0, pack0 + count)
+  cudaError_t (*inv)(const PlaneArgs<T> &, int count, bool acc, cudaStream_t);
   bool acc_fits;  // the inverse pass can keep a plane of W_i partial sums in shared memory
 };
-bool plane_ops_f32_small(int n2, int n3, PlaneOps<float> *out);
-bool plane_ops_f32_large(int n2, int n3, PlaneOps<float> *out);
 bool plane_ops_f64(int n2, int n3, PlaneOps<double> *out);
+
+// FP32 plane chain, two lines per thread (line_pair.cuh): the plane passes of one grid, false without a
+// plan.  A pack's scratch holds n1 n3 ceil(n2/2) 16-byte units, and the axis-1 pass reads the Coulomb
+// table in that layout (launch_line_pair_table: n1 n3 ceil(n2/2) float pairs, from the natural-order
+// table).
+bool line_pair_ops(int n1, int n2, int n3, PlaneOps<float> *out);
+cudaError_t launch_line_pair_table(const float *K, int n1, int n2, int n3, float *out, cudaStream_t st);
+cudaError_t launch_line_pair_conv(const PairPassArgs<float> &a, int npacks, cudaStream_t st);
 
 // Persistent pair chain (persistent_chain.cuh): one launch walks every pack of one or more builds
 // on one grid through a device-side task queue.

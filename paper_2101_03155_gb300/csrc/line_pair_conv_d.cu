@@ -1,0 +1,6 @@
+// Axis-1 pass of the line-pair chain for the axis lengths of group D (pair_chain.cuh).
+#include "line_pair_kernels.cuh"
+
+namespace ace {
+ACE_DEFINE_LP_CONV(d, ACE_LENGTHS_D)
+}  // namespace ace

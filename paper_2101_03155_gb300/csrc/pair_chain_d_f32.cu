@@ -1,4 +1,4 @@
-// Pencil-pass and axis-1 kernels (float) for the axis lengths of group D (pair_chain.cuh).
+// Pencil-pass kernels (float) for the axis lengths of group D (pair_chain.cuh).
 #include "pair_chain.cuh"
 
 namespace ace {

@@ -3,8 +3,7 @@
 
 namespace ace {
 #define ACE_DECLARE_GROUP(G)                                                                             \
-  bool pass_##G##_f32(int L, int mode, const PairPassArgs<float> &a, int npacks, cudaStream_t st, cudaError_t *e); \
-  bool conv_##G##_f32(int L, const PairPassArgs<float> &a, int npacks, cudaStream_t st, cudaError_t *e);
+  bool pass_##G##_f32(int L, int mode, const PairPassArgs<float> &a, int npacks, cudaStream_t st, cudaError_t *e);
 ACE_DECLARE_GROUP(a)
 ACE_DECLARE_GROUP(b)
 ACE_DECLARE_GROUP(c)
@@ -17,15 +16,6 @@ cudaError_t launch_pair_pass<float>(int mode, const PairPassArgs<float> &a, int 
   cudaError_t e = cudaErrorInvalidValue;
   if (pass_a_f32(L, mode, a, npacks, st, &e) || pass_b_f32(L, mode, a, npacks, st, &e) ||
       pass_c_f32(L, mode, a, npacks, st, &e) || pass_d_f32(L, mode, a, npacks, st, &e))
-    return e;
-  return cudaErrorInvalidValue;
-}
-
-template <>
-cudaError_t launch_conv_pass<float>(const PairPassArgs<float> &a, int npacks, cudaStream_t st) {
-  cudaError_t e = cudaErrorInvalidValue;
-  if (conv_a_f32(a.n1, a, npacks, st, &e) || conv_b_f32(a.n1, a, npacks, st, &e) ||
-      conv_c_f32(a.n1, a, npacks, st, &e) || conv_d_f32(a.n1, a, npacks, st, &e))
     return e;
   return cudaErrorInvalidValue;
 }
