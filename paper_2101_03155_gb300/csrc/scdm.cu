@@ -20,44 +20,100 @@
 namespace ace {
 namespace {
 
-constexpr int kSelNT = 256;  // threads of the one-CTA reduction kernel
 constexpr int kUpdNT = 256;  // threads of the streaming selection kernels
 constexpr int kUpdBlocks = 1024;  // most blocks of a selection pass (sizes the block-maximum arrays)
 constexpr int kNsMax = 64;          // Newton-Schulz iterations at most
 constexpr int kNsChunk = 16;        // iterations launched between host checks of convergence
 constexpr double kNsStop = 1e-12;   // max |T - I| below which the following iterations are skipped
+constexpr int kBlk = 8;             // points of a block of the FP32 selection
+constexpr int kSeedLag = 16;        // most vectors a threshold block may be behind
 constexpr int kChunk = 8;           // products summed in the working type before the FP64 add
 constexpr double kDependent = 1e-24;    // |residual|^2 / |psi(c)|^2 below which a column is dependent
 constexpr double kDependent32 = 1e-10;  // the same with FP32 Gram-Schmidt
 
-// (value, index) maximum, the smaller index winning ties
-__device__ __forceinline__ void amax(double &v, long long &i, double v2, long long i2) {
-  if (v2 > v || (v2 == v && i2 < i)) {
+// Order key of an FP64 residual norm: the bits of a double compare like the values for non-negative ones,
+// with chosen points (-1) below them and NaN (never chosen) at kNone.  Comparisons of FP64 values would run
+// on the FP64 pipe, which issues one warp instruction per 64 cycles.
+constexpr long long kNone = (long long)0x8000000000000000ull;
+__device__ __forceinline__ long long res_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? kNone : b;
+}
+
+// The FP32 selection keeps its residual norms as 64-bit fixed-point numbers in units of 2^(E - 60), E the
+// exponent of the largest |psi(r)|^2: exact sums of exact squares down to 2^-60 of the largest norm (an FP64
+// sum rounds to 2^-53 of each residual), with integer adds of a few cycles where a chain of dependent FP64
+// updates took 200 cycles a step.  -1 marks chosen points, kNone a norm that is not a number.  Until a
+// block is first updated its norms are the FP32 values of the start, as their bits with kRaw set (E is not
+// known before every norm is); they are ordered like the numbers.
+constexpr long long kRaw = 1ll << 62;
+__device__ __forceinline__ long long raw_norm(float v) {
+  return v >= 0.f ? kRaw | (long long)__float_as_uint(v) : kNone;  // a sum of squares: never negative
+}
+__device__ __forceinline__ int float_exp(unsigned b) { return max((int)(b >> 23 & 255), 1) - 150; }  // of the last bit
+__device__ __forceinline__ unsigned float_mant(unsigned b) { return (b & 0x7fffff) | (b >> 23 & 255 ? 0x800000u : 0u); }
+__device__ __forceinline__ long long shift_to(unsigned long long m, int t) {
+  return t >= 0 ? (long long)(m << min(t, 63)) : (t > -64 ? (long long)(m >> -t) : 0);
+}
+// the value of a stored norm (raw or fixed) in fixed point; unit exponent e0 = E - 60
+__device__ __forceinline__ long long to_fixed(long long v, int e0) {
+  if (v < kRaw) return v;
+  const unsigned b = (unsigned)v;
+  return shift_to(float_mant(b), float_exp(b) - e0);
+}
+// v - p^2, not below 0 (0 when p is not finite), for v >= 0
+__device__ __forceinline__ long long downdate(long long v, float p, int e0) {
+  const unsigned b = __float_as_uint(p) & 0x7fffffff;
+  const unsigned long long m = float_mant(b);
+  const long long t = v - shift_to(m * m, 2 * float_exp(b) - e0);
+  return v < 0 ? v : (t < 0 || b >= 0x7f800000u ? 0 : t);
+}
+
+// (key, index) maximum, the smaller index winning ties
+__device__ __forceinline__ void amax(long long &v, long long &i, long long v2, long long i2) {
+  if (v2 > v || (v2 == v && v2 != kNone && i2 < i)) {
     v = v2;
     i = i2;
   }
 }
 
-__device__ __forceinline__ void warp_amax(double &v, long long &i) {
+// over the lanes of a warp (in lane 0)
+__device__ __forceinline__ void warp_amax(long long &v, long long &i) {
   for (int o = 16; o > 0; o >>= 1) {
-    const double v2 = __shfl_down_sync(0xffffffffu, v, o);
+    const long long v2 = __shfl_down_sync(0xffffffffu, v, o);
     const long long i2 = __shfl_down_sync(0xffffffffu, i, o);
     amax(v, i, v2, i2);
   }
+}
+// over the points of a block (lane >> 2; in every lane)
+__device__ __forceinline__ long long blk_max(long long v) {
+  for (int o = 16; o > 2; o >>= 1) {
+    const long long v2 = __shfl_xor_sync(0xffffffffu, v, o);
+    v = v2 > v ? v2 : v;
+  }
+  return v;
 }
 
 // State of the greedy selection passed to the streaming kernels.  Each pass publishes one
 // (maximum, index) per block; the block that publishes last takes the pivot step of the pass, so
 // that no separate launch (and no waiting) sits between the passes.
 struct SelArgs {
-  double *bval;          // [gridDim.x] block maxima of the residual norms
+  long long *bval;       // [gridDim.x] keys of the block maxima of the residual norms
   long long *bidx;       // [gridDim.x] their grid indices
   unsigned int *count;   // blocks of the current pass that have published (the last one resets it)
-  void *Ub;              // [n][ldu] of the working type, row j = u_j, ldu = n rounded up to even
-                         // (pad column zero)
+  void *Ub;              // [n][ldu] of the working type, row j = u_j, row stride ldu
+                         // (basis_ld; the padding is zero)
   int *piv;              // [n]
   int *dependent;        // set when a chosen column lies in the span of the earlier ones
   int k;                 // step whose pivot this pass selects
+  // FP32 selection: per block of kBlk points, an upper bound of its residual norms and the number of
+  // basis vectors its residuals account for; per step, the largest up-to-date residual seen so far
+  // and per CTA of a pass the largest bound over its blocks (as they stand at its end), with its block
+  long long *tval, *tidx;   // [gridDim.x]
+  long long *bmax;       // [blocks]
+  int *bcnt;             // [blocks]
+  long long *thr;        // [n + 1], from 0
+  int *unit;             // exponent of the fixed-point unit, set by the first pivot step
 };
 
 template <typename T>
@@ -71,6 +127,12 @@ struct Vec2<double> {
   using type = double2;
 };
 
+// Row stride of the basis u_j: whole float4 rows for FP32, even for FP64 (the padding is zero)
+template <typename T>
+__host__ __device__ constexpr int basis_ld(int n) {
+  return sizeof(T) == 4 ? (n + 3) & ~3 : (n + 1) & ~1;
+}
+
 // Shared memory of a streaming block: u_{k-1} while streaming, the pivot step's vectors afterwards.
 template <typename T>
 struct __align__(16) ScdmSmem {
@@ -79,9 +141,202 @@ struct __align__(16) ScdmSmem {
   } sel;
   T us[1024];
   double rv[kUpdNT / 32], rv0[kUpdNT / 32];
-  long long ri[kUpdNT / 32];
-  long long chosen;
-  int last;
+  long long rk[kUpdNT / 32], ri[kUpdNT / 32], tk[kUpdNT / 32], ti[kUpdNT / 32];
+  long long chosen, top;
+  int last, unit;
+};
+
+__device__ __forceinline__ float dot4(float4 a, float4 b) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
+}
+
+// A block's 8 points as a warp holds them: lane 4 p + c has point p and the orbital quads l = c, c + 4, ...,
+// c + 28 (orbitals 4 l .. 4 l + 3), x[4 i + t] orbital 4 (c + 4 i) + t (+ 128 f0 with more than 128 orbitals).
+__device__ __forceinline__ void load_block(const float *__restrict__ psi, int n, long long N, long long r0, int lim,
+                                           int f0, float (&x)[32]) {
+  const int lane = threadIdx.x & 31, p = lane >> 2, c = lane & 3;
+  const float *q = psi + (long long)(4 * (f0 + c)) * N + r0 + p;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int orb = 4 * (f0 + c + 4 * i) + t;
+      x[4 * i + t] = orb < n && p < lim ? __ldg(q + (long long)(16 * i + t) * N) : 0.f;
+    }
+}
+
+// pm[q] = u_{j+q} . psi(point lane >> 2) for q < 4 (from the row k - 1 on: any value).  The quads' sums are
+// added in FP32 by a pairwise tree over l (l ^ 16, 8, 4 inside the lane, then l ^ 2, 1 over the four lanes of
+// a point): two shuffles per vector for 8 points, where a lane per quad needed 23.
+__device__ __forceinline__ void project4(const float *__restrict__ psi, int n, long long N, const float *Ub, long long r0,
+                                         int lim, int j, int k, float (&x)[32], float (&pm)[4]) {
+  const int c = threadIdx.x & 3, nf = (n + 3) / 4;
+  const unsigned full = 0xffffffffu;
+  const float4 *u4 = reinterpret_cast<const float4 *>(Ub);
+  float acc[4][8];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[q][i] = 0.f;
+  for (int f0 = 0; f0 < nf; f0 += 32) {
+    if (nf > 32) load_block(psi, n, N, r0, lim, f0, x);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float4 *u = u4 + (long long)min(j + q, k - 1) * nf + f0 + c;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float4 w = f0 + c + 4 * i < nf ? u[4 * i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        acc[q][i] += dot4(w, make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]));
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+      for (int i = 0; i < o; ++i) acc[q][i] += acc[q][i + o];
+    float t = acc[q][0];
+    t += __shfl_xor_sync(full, t, 2);
+    t += __shfl_xor_sync(full, t, 1);
+    pm[q] = t;
+  }
+}
+
+// End of a block's update (a warp): residuals dr of point lane & 7, up to date with j of k vectors.
+__device__ __forceinline__ void store_block(long long *d, const SelArgs &s, long long blk, long long r0, int lim, int j_in,
+                                            int j, int k, long long dr, long long mx, long long &best, long long &bi) {
+  const int lane = threadIdx.x & 31, p = lane >> 2;
+  const bool mine = (lane & 3) == 0 && p < lim;
+  if (j != j_in && mine) d[r0 + p] = dr;
+  if (lane == 0) {
+    s.bmax[blk] = mx;
+    s.bcnt[blk] = j;
+  }
+  if (j == k) {
+    if (mine) amax(best, bi, dr, r0 + p);
+    if (lane == 0 && mx > 0) atomicMax(s.thr + k, mx);
+  }
+}
+
+// A block's residuals (point lane >> 2, as stored), count and points, for refresh_loaded.  Residuals and
+// counts are read through L2: in the pivot step other CTAs of the pass wrote them.
+__device__ __forceinline__ void load_state(const float *__restrict__ psi, int n, long long N, const long long *d,
+                                           const SelArgs &s, long long blk, long long &r0, int &lim, int &j,
+                                           long long &dr, float (&x)[32]) {
+  const int p = (threadIdx.x & 31) >> 2;
+  r0 = blk * kBlk;
+  lim = (int)min((long long)kBlk, N - r0);
+  dr = p < lim ? __ldcg(d + r0 + p) : -1;
+  j = __ldcg(s.bcnt + blk);
+  if (n <= 128) load_block(psi, n, N, r0, lim, 0, x);
+}
+
+// Basis rows j .. j + 7 (rows past `upto` repeat the last one) into a warp's staging buffer, asynchronously;
+// quads past the orbitals are zero.
+constexpr int kRows = 8;                                  // rows of a buffer
+constexpr int kStage = 2 * kRows * 32;                    // float4 per warp: two buffers
+constexpr int kStageBytes = 16 * kStage * (kUpdNT / 32);
+__device__ __forceinline__ void stage_rows(const float *Ub, int nf, int j, int upto, float4 *buf) {
+  const int lane = threadIdx.x & 31;
+  const float4 *u4 = reinterpret_cast<const float4 *>(Ub);
+#pragma unroll
+  for (int q = 0; q < kRows; ++q) {
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(buf + q * 32 + lane);
+    const float4 *src = u4 + (long long)min(j + q, upto - 1) * nf + (lane < nf ? lane : 0);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(lane < nf ? 16 : 0) : "memory");
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Applies the basis vectors j .. upto - 1 (upto <= k) to one block (a warp): its residuals lose
+// (u_j . psi(r))^2 in order of j.  With `stop` it ends early once every residual is below the largest
+// up-to-date one: the residuals only fall, so the block cannot hold the pivot.  A block that gets to k adds
+// its maximum to (best, bi) and to the threshold.  Returns the block's new bound.
+//   Up to 128 orbitals the rows of the basis come through the warp's staging buffers, eight ahead of their
+// use (loads from L2 one vector at a time took most of a long catch-up).
+__device__ __forceinline__ long long refresh_loaded(const float *__restrict__ psi, int n, long long N, long long *d,
+                                                    const SelArgs &s, long long blk, long long r0, int lim, int j, int k,
+                                                    int upto, bool stop, int e0, long long dr, float (&x)[32],
+                                                    float4 *stage,
+                                                    long long &best, long long &bi) {
+  const int j_in = j;
+  const long long thr = stop ? __ldcg(s.thr + k) : kNone;
+  const float *Ub = static_cast<const float *>(s.Ub);
+  dr = to_fixed(dr, e0);
+  long long mx = blk_max(dr);
+  if (n <= 128) {
+    const int c = threadIdx.x & 3, nf = (n + 3) / 4;
+    int buf = 0;
+    if (j < upto) stage_rows(Ub, nf, j, upto, stage);
+    while (j < upto && mx >= thr) {
+      if (j + kRows < upto) {
+        stage_rows(Ub, nf, j + kRows, upto, stage + (buf ^ 1) * (kRows * 32));
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      __syncwarp();
+      const int m = min(kRows, upto - j);
+      float pm[kRows];
+#pragma unroll
+      for (int q = 0; q < kRows; ++q) {
+        const float4 *u = stage + (buf * kRows + q) * 32 + c;
+        float acc[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          acc[i] = dot4(u[4 * i], make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]));
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+          for (int i = 0; i < o; ++i) acc[i] += acc[i + o];
+        float t = acc[0];
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        pm[q] = t + __shfl_xor_sync(0xffffffffu, t, 1);
+      }
+#pragma unroll
+      for (int q = 0; q < kRows; ++q)
+        if (q < m) dr = downdate(dr, pm[q], e0);
+      j += m;
+      mx = blk_max(dr);
+      buf ^= 1;
+      __syncwarp();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+  } else {
+    while (j < upto && mx >= thr) {
+      float pm[4];
+      project4(psi, n, N, Ub, r0, lim, j, upto, x, pm);
+      const int m = min(4, upto - j);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < m) dr = downdate(dr, pm[q], e0);
+      j += m;
+      mx = blk_max(dr);
+    }
+  }
+  store_block(d, s, blk, r0, lim, j_in, j, k, dr, mx, best, bi);
+  return mx;
+}
+__device__ long long refresh_block(const float *__restrict__ psi, int n, long long N, long long *d, const SelArgs &s,
+                                   long long blk, int k, int upto, bool stop, int e0, float4 *stage,
+                                   long long &best, long long &bi) {
+  long long r0, dr;
+  int lim, j;
+  float x[32];
+  load_state(psi, n, N, d, s, blk, r0, lim, j, dr, x);
+  return refresh_loaded(psi, n, N, d, s, blk, r0, lim, j, k, upto, stop, e0, dr, x, stage, best, bi);
+}
+
+// Stored residuals: FP64 values, or the fixed-point numbers of the FP32 selection
+template <typename T>
+struct Resid {
+  using type = double;
+};
+template <>
+struct Resid<float> {
+  using type = long long;
 };
 
 // Pivot step k, run by the whole last block of a pass: the pivot c_k from the block maxima (it
@@ -92,31 +347,66 @@ struct __align__(16) ScdmSmem {
 // u_k = 0 and sets *dependent.
 template <typename T>
 __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr, int n, long long N, int nblk,
-                           double *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm) {
+                           typename Resid<T>::type *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm,
+                           float4 *stage) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int kWarps = kUpdNT / 32;
   using V2 = typename Vec2<T>::type;
   T *u = sm.sel.u, *c = sm.sel.c;
   const T *Ub = static_cast<const T *>(s.Ub);
   const int k = s.k;
-  double best = -2.0;
-  long long bi = N;
+  long long best = kNone, bi = N;
   for (int b = tid; b < nblk; b += kUpdNT) amax(best, bi, __ldcg(s.bval + b), __ldcg(s.bidx + b));
   warp_amax(best, bi);
   if (lane == 0) {
-    sm.rv[warp] = best;
+    sm.rk[warp] = best;
     sm.ri[warp] = bi;
   }
   __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < kWarps; ++w) amax(best, bi, sm.rv[w], sm.ri[w]);
-    sm.chosen = bi < N ? bi : 0;
-    s.piv[k] = (int)sm.chosen;
-    d[sm.chosen] = -1.0;
+  if (warp == 0) {
+    best = lane < kWarps ? sm.rk[lane] : kNone;
+    bi = lane < kWarps ? sm.ri[lane] : N;
+    warp_amax(best, bi);
+    if (lane == 0) {
+      sm.chosen = bi < N ? bi : 0;
+      s.piv[k] = (int)sm.chosen;
+      d[sm.chosen] = -1;
+      if constexpr (sizeof(T) == 4) {
+        // the largest norm of all gives the fixed-point unit (an infinite one: any)
+        if (k == 0) *s.unit = float_exp((unsigned)best) + 23 - 60;
+        sm.unit = k == 0 ? float_exp((unsigned)best) + 23 - 60 : *s.unit;
+      }
+    }
   }
   __syncthreads();
   const long long cr = sm.chosen;
-  const int ldu = (n + 1) & ~1, np = ldu / 2;  // Ub row stride (even; the pad column is zero)
+  // FP32: the next step's threshold comes from the blocks with the largest bounds, one per warp from its
+  // share of the CTAs, brought up to date with u_k at the end of this step.  Away from c_k bounds near the
+  // top hardly change, so one of these is the next pivot's block, or close to it in value.  Their points are
+  // loaded here, ahead of the basis vector.
+  long long seed = N, sr0 = 0;
+  int slim = 0, sj = 0;
+  long long seed_d = -1;
+  float sv[32];
+  if constexpr (sizeof(T) == 4) {
+    if (k + 1 < n) {
+      long long tb = kNone, tbi = N;
+      for (int b = warp + kWarps * lane; b < nblk; b += kWarps * 32) amax(tb, tbi, __ldcg(s.tval + b), __ldcg(s.tidx + b));
+      warp_amax(tb, tbi);
+      seed = __shfl_sync(0xffffffffu, tbi, 0);
+      if (seed < N && k + 1 - __ldcg(s.bcnt + seed) > kSeedLag) {
+        // too far behind: the best point of the share that this pass brought up to date instead
+        tb = kNone;
+        tbi = N;
+        for (int b = warp + kWarps * lane; b < nblk; b += kWarps * 32) amax(tb, tbi, __ldcg(s.bval + b), __ldcg(s.bidx + b));
+        warp_amax(tb, tbi);
+        tbi = __shfl_sync(0xffffffffu, tbi, 0);
+        seed = tbi < N ? tbi / kBlk : N;
+      }
+      if (seed < N) load_state(psi, n, N, d, s, seed, sr0, slim, sj, seed_d, sv);
+    }
+  }
+  const int ldu = basis_ld<T>(n), np = ldu / 2;
   T part0 = (T)0;
   for (int i = tid; i < ldu; i += kUpdNT) {
     u[i] = i < n ? psi[(long long)i * si + cr * sr] : (T)0;
@@ -203,35 +493,65 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
   const T inv = c[0];
   T *Uw = static_cast<T *>(s.Ub);
   for (int i = tid; i < ldu; i += kUpdNT) Uw[(long long)k * ldu + i] = i < n ? u[i] * inv : (T)0;
+  if constexpr (sizeof(T) == 4) {
+    if (k + 1 < n) {
+      __threadfence();
+      __syncthreads();  // u_k for the CTA, in L2
+      if (seed < N) {
+        if (sr0 + (lane >> 2) == cr) seed_d = -1;
+        refresh_loaded(psi, n, N, d, s, seed, sr0, slim, sj, k + 1, k + 1, true, sm.unit, seed_d, sv, stage + warp * kStage, best, bi);
+      }
+    }
+  }
 }
 
 // End of a pass for one block: publish the block maximum; the last block to publish takes the
-// pivot step and resets the counter for the next pass.  Orbital i at point r is psi[i si + r sr].
+// pivot step and resets the counter for the next pass (true for that block).  Orbital i at point r is psi[i si + r sr].
 template <typename T>
-__device__ void finish_pass(double best, long long bi, const T *__restrict__ psi, long long si, long long sr, int n,
-                            long long N, double *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm) {
+__device__ bool finish_pass(long long best, long long bi, long long top, long long ti, const T *__restrict__ psi, long long si, long long sr, int n,
+                            long long N, typename Resid<T>::type *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm,
+                           float4 *stage) {
   const int tid = threadIdx.x;
+  constexpr int kWarps = kUpdNT / 32;
   warp_amax(best, bi);
+  if constexpr (sizeof(T) == 4) warp_amax(top, ti);
   if ((tid & 31) == 0) {
-    sm.rv[tid >> 5] = best;
+    sm.rk[tid >> 5] = best;
     sm.ri[tid >> 5] = bi;
+    sm.tk[tid >> 5] = top;
+    sm.ti[tid >> 5] = ti;
   }
   __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < kUpdNT / 32; ++w) amax(best, bi, sm.rv[w], sm.ri[w]);
-    s.bval[blockIdx.x] = best;
-    s.bidx[blockIdx.x] = bi;
-    __threadfence();  // the maximum (and this block's residual norms) before the count
-    sm.last = atomicAdd(s.count, 1u) == gridDim.x - 1;
+  if (tid < 32) {
+    best = tid < kWarps ? sm.rk[tid] : kNone;
+    bi = tid < kWarps ? sm.ri[tid] : N;
+    warp_amax(best, bi);
+    if constexpr (sizeof(T) == 4) {
+      top = tid < kWarps ? sm.tk[tid] : kNone;
+      ti = tid < kWarps ? sm.ti[tid] : N;
+      warp_amax(top, ti);
+      if (tid == 0) {
+        s.tval[blockIdx.x] = top;
+        s.tidx[blockIdx.x] = ti;
+        sm.top = ti;
+      }
+    }
+    if (tid == 0) {
+      s.bval[blockIdx.x] = best;
+      s.bidx[blockIdx.x] = bi;
+      __threadfence();  // the maximum (and this block's residual norms) before the count
+      sm.last = atomicAdd(s.count, 1u) == gridDim.x - 1;
+    }
   }
   __syncthreads();
-  if (!sm.last) return;
+  if (!sm.last) return false;
   __threadfence();
-  pivot_step<T>(psi, si, sr, n, N, gridDim.x, d, s, sm);
+  pivot_step<T>(psi, si, sr, n, N, gridDim.x, d, s, sm, stage);
   if (tid == 0) *s.count = 0u;
+  return true;
 }
 
-// One selection pass, any T and any N (one point per thread per iteration):
+// One selection pass of the FP64 form (one point per thread per iteration):
 //   NORM: d[r] = |psi(r)|^2 (the start);
 //   else: d[r] -= (u_{k-1} . psi(r))^2 for every column still a candidate (d[r] >= 0), u_{k-1} = row
 //         k-1 of Ub.
@@ -242,10 +562,9 @@ __global__ void __launch_bounds__(kUpdNT) scdm_pass_kernel(const T *__restrict__
   __shared__ ScdmSmem<T> sm;
   if (!NORM)
     for (int i = threadIdx.x; i < n; i += kUpdNT)
-      sm.us[i] = static_cast<const T *>(s.Ub)[(long long)(s.k - 1) * ((n + 1) & ~1) + i];
+      sm.us[i] = static_cast<const T *>(s.Ub)[(long long)(s.k - 1) * basis_ld<T>(n) + i];
   __syncthreads();
-  double best = -2.0;
-  long long bi = N;
+  long long best = kNone, bi = N;
   for (long long r = blockIdx.x * (long long)kUpdNT + threadIdx.x; r < N; r += (long long)gridDim.x * kUpdNT) {
     double dr = NORM ? 0.0 : d[r];
     if (NORM || dr >= 0.0) {
@@ -262,125 +581,134 @@ __global__ void __launch_bounds__(kUpdNT) scdm_pass_kernel(const T *__restrict__
       dr = NORM ? p : fmax(dr - p * p, 0.0);
       d[r] = dr;
     }
-    amax(best, bi, dr, r);
+    amax(best, bi, res_key(dr), r);
   }
-  finish_pass<T>(best, bi, psi, N, 1, n, N, d, s, sm);
+  finish_pass<T>(best, bi, kNone, N, psi, N, 1, n, N, d, s, sm, nullptr);
 }
 
-// Point-major copy of FP32 orbitals for the streaming passes: pt[r][i] = psi[i][r] for i < n, zero for
-// n <= i < ldt (ldt = n rounded up to a multiple of 4, so that every row starts on 16 bytes).
-__global__ void scdm_transpose_kernel(const float *__restrict__ psi, int n, long long N, int ldt,
-                                      float *__restrict__ pt) {
-  __shared__ float tile[32][33];
-  const long long r0 = (long long)blockIdx.x * 32;
-  const int i0 = blockIdx.y * 32;
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const int i = i0 + y;
-    const long long r = r0 + threadIdx.x;
-    tile[y][threadIdx.x] = (i < n && r < N) ? psi[(long long)i * N + r] : 0.f;
-  }
-  __syncthreads();
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const long long r = r0 + y;
-    const int i = i0 + threadIdx.x;
-    if (r < N && i < ldt) pt[r * ldt + i] = tile[threadIdx.x][y];
-  }
-}
+// The FP32 selection.  The residual norms only fall from step to step, so the residual a point had when
+// it was last brought up to date bounds its present one: a step has to look only at the blocks whose
+// bound reaches the largest up-to-date residual.  For 128 orbitals on 96^3 that is 27,000 block visits in
+// all 128 steps, a quarter of the blocks once, where passes over every point (the plain greedy selection)
+// read Psi 128 times: 11.4 ms per call, bound by HBM at 0.8 of its bandwidth; now 5.0 ms, of which the
+// chain of the 127 steps (launch, look at the bounds, visits, pivot step: about 30 us each) is 3.9 ms.
+//   Every residual goes through the same operations in the same order as when all points are updated in
+// every step, so the pivots are the same.
 
-__device__ __forceinline__ float dot4(float4 a, float4 b) {
-  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
-}
-
-// The selection pass for FP32 orbitals in the point-major copy pt [N][ldt].  Every warp takes an
-// equal share of the points, 32 at a time in four groups of 8: lane l loads the float4 of orbitals
-// 4l..4l+3 (and 4l + 128 m) of the 8 points of a group, so that each warp load reads a whole orbital
-// row of one point.  The lanes' partial sums are added over the lanes in FP32 by a pairwise tree (two
-// all-reduce levels, then three butterfly levels that leave point l & 7 of the group on lane l), and
-// lane l keeps point l of the 32.  Only the residual update itself is FP64 (this GPU's FP64 rate is a
-// small fraction of its FP32 rate).
-template <bool NORM>
-__global__ void __launch_bounds__(kUpdNT, 3) scdm_pass_pt_kernel(const float *__restrict__ pt, int n, int ldt,
-                                                                long long N, double *__restrict__ d, SelArgs s) {
+// d[r] = |psi(r)|^2 (FP32), one point per thread; the sum has the order of refresh_block's (32 partial sums over
+// orbitals 4 l .. 4 l + 3 (+ 128 f), then the pairwise tree).
+__global__ void __launch_bounds__(kUpdNT) scdm_norm_kernel(const float *__restrict__ psi, int n, long long N,
+                                                           long long *__restrict__ d, SelArgs s) {
   __shared__ __align__(16) ScdmSmem<float> sm;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int nf = ldt / 4;  // float4 per point row
-  if (!NORM)
-    for (int i = tid; i < ldt; i += kUpdNT)
-      sm.us[i] = i < n ? static_cast<const float *>(s.Ub)[(long long)(s.k - 1) * ((n + 1) & ~1) + i] : 0.f;
-  __syncthreads();
-  const float4 *pt4 = reinterpret_cast<const float4 *>(pt);
-  const float4 *u4 = reinterpret_cast<const float4 *>(sm.us);
-  const long long nwarps = (long long)gridDim.x * (kUpdNT / 32);
-  const long long wg = (long long)blockIdx.x * (kUpdNT / 32) + (tid >> 5);
-  const long long ra = N * wg / nwarps, rb = N * (wg + 1) / nwarps;
-  const unsigned full = 0xffffffffu;
-  double best = -2.0;
-  long long bi = N;
-  for (long long r0 = ra; r0 < rb; r0 += 32) {  // same trip count for the whole warp
-    const long long rme = r0 + lane;
-    double dr = (!NORM && rme < rb) ? d[rme] : 0.0;  // the residual this lane updates, early
-    float mine = 0.f;
-#pragma unroll 1
-    for (int grp = 0; grp < 4; ++grp) {
-      const long long rg = r0 + 8 * grp;
-      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-      for (int f0 = 0; f0 < nf; f0 += 32) {
-        const int f = f0 + lane;
-        const bool fv = f < nf;
-        const float4 uu = (NORM || !fv) ? make_float4(0.f, 0.f, 0.f, 0.f) : u4[f];
-        float4 v[8];
-        const float4 *base = pt4 + rg * nf + f;
-        const int lim = fv ? (int)min(8LL, rb - rg) : 0;  // points of the group inside this warp's share
+  extern __shared__ float4 stage_all[];  // kStage per warp
+  const int nf = (n + 3) / 4;
+  long long best = kNone, bi = N;
+  const long long step = (long long)gridDim.x * kUpdNT;
+  for (long long r0 = blockIdx.x * (long long)kUpdNT; r0 < N; r0 += step) {  // same trip count for the CTA
+    const long long r = r0 + threadIdx.x;
+    float acc[32];
 #pragma unroll
-        for (int p = 0; p < 8; ++p)
-          v[p] = p < lim ? __ldcs(base + p * nf) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int l = 0; l < 32; ++l) acc[l] = 0.f;
+    for (int f0 = 0; f0 < nf; f0 += 32) {
 #pragma unroll
-        for (int p = 0; p < 8; ++p) acc[p] += NORM ? dot4(v[p], v[p]) : dot4(uu, v[p]);
-      }
+      for (int l = 0; l < 32; ++l) {
+        float x[4];
 #pragma unroll
-      for (int p = 0; p < 8; ++p) {
-        acc[p] += __shfl_xor_sync(full, acc[p], 16);
-        acc[p] += __shfl_xor_sync(full, acc[p], 8);
-      }
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int j = 0; j < o; ++j) {
-          const float send = up ? acc[j] : acc[j + o];
-          const float keep = up ? acc[j + o] : acc[j];
-          acc[j] = keep + __shfl_xor_sync(full, send, o);
+        for (int t = 0; t < 4; ++t) {
+          const int i = 4 * (f0 + l) + t;
+          x[t] = (i < n && r < N) ? __ldcs(psi + (long long)i * N + r) : 0.f;
         }
+        const float4 v = make_float4(x[0], x[1], x[2], x[3]);
+        acc[l] += dot4(v, v);
       }
-      if ((lane >> 3) == grp) mine = acc[0];  // point rg + (lane & 7) = r0 + lane
     }
-    if (rme < rb) {
-      const double pm = (double)mine;
-      if (NORM)
-        dr = pm;
-      else if (dr >= 0.0)
-        dr = fmax(fma(-pm, pm, dr), 0.0);
-      d[rme] = dr;
-      amax(best, bi, dr, rme);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int l = 0; l < o; ++l) acc[l] += acc[l + o];
+    const long long dr = r < N ? raw_norm(acc[0]) : -1;
+    long long mx = dr;  // over the 8 lanes of a block
+    for (int o = kBlk / 2; o > 0; o >>= 1) {
+      const long long v = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = v > mx ? v : mx;
+    }
+    if (r < N) {
+      d[r] = dr;
+      amax(best, bi, dr, r);
+    }
+    if (r < N && r % kBlk == 0) {
+      s.bmax[r / kBlk] = mx;
+      s.bcnt[r / kBlk] = 0;
     }
   }
-  finish_pass<float>(best, bi, pt, 1, ldt, n, N, d, s, sm);
+  finish_pass<float>(best, bi, best, bi < N ? bi / kBlk : N, psi, N, 1, n, N, d, s, sm, stage_all);
 }
 
-// sum_l a[l sa] b[l sb] over l < n, in four interleaved partial sums (independent loads in flight)
+// Step k >= 1: the warps look through the blocks' bounds, 32 at a time (neighbouring blocks belong to
+// different warps), and bring those that reach the threshold up to date.
+//   While the last CTA takes the pivot step, the others move blocks forward whose bound is not far below the
+// threshold and which a later step will need: without it the longest catch-up of a step was 57 vectors on
+// average (128 orbitals on 96^3), a chain of dependent FP64 updates (8.0 ms per call).  A CTA leaves out the
+// block with its largest bound, which the pivot step may be working on.
+constexpr int kSoonFrac = 5;   // bounds from 1 - 1 / kSoonFrac of the threshold on
+constexpr int kAhead = 8;      // vectors per step and block
+constexpr int kAheadMost = 2;  // blocks per warp and step
+__global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__restrict__ psi, int n, long long N,
+                                                              long long *__restrict__ d, SelArgs s) {
+  __shared__ __align__(16) ScdmSmem<float> sm;
+  extern __shared__ float4 stage_all[];  // kStage per warp
+  float4 *stage = stage_all + (threadIdx.x >> 5) * kStage;
+  const int lane = threadIdx.x & 31;
+  const unsigned full = 0xffffffffu;
+  const long long nb = (N + kBlk - 1) / kBlk;
+  const long long nwarps = (long long)gridDim.x * (kUpdNT / 32);
+  const long long w = (long long)blockIdx.x * (kUpdNT / 32) + (threadIdx.x >> 5);
+  const int e0 = *s.unit;
+  long long thr = __ldcg(s.thr + s.k);
+  const long long soon = thr - thr / kSoonFrac;
+  long long best = kNone, bi = N, top = kNone, ti = N;
+  for (long long b0 = w; b0 < nb; b0 += 32 * nwarps) {
+    const long long b = b0 + lane * nwarps;
+    long long bound = b < nb ? to_fixed(s.bmax[b], e0) : kNone;
+    unsigned left = __ballot_sync(full, bound >= 0 && bound >= thr);
+    while (left) {
+      const int src = __ffs(left) - 1;
+      left &= left - 1;
+      const long long mx = refresh_block(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, s.k, true, e0, stage, best, bi);
+      if (lane == src) bound = mx;
+      if (left) {
+        thr = __ldcg(s.thr + s.k);
+        left &= __ballot_sync(full, bound >= thr);
+      }
+    }
+    amax(top, ti, bound, b);
+  }
+  if (finish_pass<float>(best, bi, top, ti, psi, N, 1, n, N, d, s, sm, stage_all)) return;
+  int most = kAheadMost;
+  for (long long b0 = w; b0 < nb && most > 0; b0 += 32 * nwarps) {
+    const long long b = b0 + lane * nwarps;
+    const long long bound = b < nb ? to_fixed(s.bmax[b], e0) : kNone;
+    const int cnt = bound >= 0 && bound >= soon && b != sm.top ? s.bcnt[b] : s.k;
+    for (unsigned ahead = __ballot_sync(full, cnt < s.k); ahead && most > 0; ahead &= ahead - 1, --most) {
+      const int src = __ffs(ahead) - 1;
+      refresh_block(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, min(s.k, __shfl_sync(full, cnt, src) + kAhead), false,
+                    e0, stage, best, bi);
+    }
+  }
+}
+
+// sum_l a[l sa] b[l sb] over l < n, in eight interleaved partial sums: with one output per thread these
+// products wait for the FP64 pipe's latency (four sums: 18 us per 128 x 128 product, its issue rate is 4 us)
 __device__ __forceinline__ double strided_dot(const double *__restrict__ a, long long sa, const double *__restrict__ b,
                                               long long sb, int n) {
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   int l = 0;
-  for (; l + 4 <= n; l += 4) {
-    s0 += a[l * sa] * b[l * sb];
-    s1 += a[(l + 1) * sa] * b[(l + 1) * sb];
-    s2 += a[(l + 2) * sa] * b[(l + 2) * sb];
-    s3 += a[(l + 3) * sa] * b[(l + 3) * sb];
+  for (; l + 8 <= n; l += 8) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s[q] += a[(l + q) * sa] * b[(l + q) * sb];
   }
-  for (; l < n; ++l) s0 += a[l * sa] * b[l * sb];
-  return (s0 + s1) + (s2 + s3);
+  for (; l < n; ++l) s[0] += a[l * sa] * b[l * sb];
+  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
 }
 
 // M[i][j] = psi_i(c_j)
@@ -402,18 +730,22 @@ __global__ void gram_t_kernel(const double *__restrict__ M, int n, double *__res
   S[e] = s;
 }
 
-// f = |S|_F (one CTA)
-__global__ void frob_kernel(const double *__restrict__ S, int n, double *__restrict__ f) {
-  __shared__ double rv[kSelNT / 32];
-  double part = 0.0;
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) part += S[e] * S[e];
+// f = |S|_F (one CTA of 1024 threads)
+__global__ void __launch_bounds__(1024) frob_kernel(const double *__restrict__ S, int n, double *__restrict__ f) {
+  __shared__ double rv[32];
+  double p0 = 0.0, p1 = 0.0;
+  for (int e = threadIdx.x; e < n * n; e += 2048) {
+    p0 += S[e] * S[e];
+    if (e + 1024 < n * n) p1 += S[e + 1024] * S[e + 1024];
+  }
+  double part = p0 + p1;
   for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
   if ((threadIdx.x & 31) == 0) rv[threadIdx.x >> 5] = part;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < kSelNT / 32; ++w) s += rv[w];
-    *f = sqrt(s);
+  if (threadIdx.x < 32) {
+    double s = rv[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *f = sqrt(s);
   }
 }
 
@@ -494,7 +826,7 @@ __global__ void scdm_factor_kernel(const double *__restrict__ M, const double *_
 }
 
 struct Layout {
-  size_t d, bval, bidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count, pt, total;
+  size_t d, bval, bidx, tval, tidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count, bmax, bcnt, thr, unit, total;
 };
 
 Layout layout(int n, long long N, size_t elem) {
@@ -507,9 +839,11 @@ Layout layout(int n, long long N, size_t elem) {
   };
   const size_t nn = (size_t)n * n;
   L.d = take(sizeof(double) * (size_t)N);
-  L.bval = take(sizeof(double) * kUpdBlocks);
+  L.bval = take(sizeof(long long) * kUpdBlocks);
   L.bidx = take(sizeof(long long) * kUpdBlocks);
-  L.Ub = take(elem * (size_t)n * (n + 1));
+  L.tval = take(sizeof(long long) * kUpdBlocks);
+  L.tidx = take(sizeof(long long) * kUpdBlocks);
+  L.Ub = take(elem * (size_t)n * (n + 3));
   L.M = take(sizeof(double) * nn);
   L.S = take(sizeof(double) * nn);
   L.Y0 = take(sizeof(double) * nn);
@@ -524,8 +858,12 @@ Layout layout(int n, long long N, size_t elem) {
   L.piv = take(sizeof(int) * (size_t)n);
   L.dependent = take(sizeof(int));
   L.count = take(sizeof(unsigned int));
-  // FP32 working type: the point-major copy [N][n rounded up to a multiple of 4]
-  L.pt = take(elem == 4 ? sizeof(float) * (size_t)N * ((n + 3) & ~3) : 0);
+  // FP32: the block bounds and the steps' thresholds
+  const size_t nb = elem == 4 ? ((size_t)N + kBlk - 1) / kBlk : 0;
+  L.bmax = take(sizeof(long long) * nb);
+  L.bcnt = take(sizeof(int) * nb);
+  L.thr = take(sizeof(long long) * (n + 1));
+  L.unit = take(sizeof(int));
   L.total = off;
   return L;
 }
@@ -540,8 +878,8 @@ template <typename T>
 cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t st, long *launches, ScdmResult *res) {
   const Layout L = layout(n, N, sizeof(T));
   char *w = static_cast<char *>(ws);
-  double *d = reinterpret_cast<double *>(w + L.d);
-  double *bval = reinterpret_cast<double *>(w + L.bval);
+  auto *d = reinterpret_cast<typename Resid<T>::type *>(w + L.d);
+  long long *bval = reinterpret_cast<long long *>(w + L.bval);
   long long *bidx = reinterpret_cast<long long *>(w + L.bidx);
   void *Ub = w + L.Ub;
   double *M = reinterpret_cast<double *>(w + L.M);
@@ -559,37 +897,42 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
   cudaError_t e = cudaMemsetAsync(res->dev, 0, sizeof(double) * kNsMax, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(res->dependent, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  // column selection: n streaming passes over Psi; the last block of each pass takes the pivot step
-  SelArgs sa{bval, bidx, count, Ub, res->piv, res->dependent, 0};
-  // FP32: the passes stream the point-major copy (whole orbital rows of points per warp load)
-  constexpr bool kPointMajor = sizeof(T) == 4;
-  const int ldt = (n + 3) & ~3;
-  float *pt = reinterpret_cast<float *>(w + L.pt);
-  // one resident wave of persistent blocks
+  // column selection: n passes; the last block of each pass takes the pivot step
+  SelArgs sa{bval, bidx, count, Ub, res->piv, res->dependent, 0, reinterpret_cast<long long *>(w + L.tval),
+             reinterpret_cast<long long *>(w + L.tidx), reinterpret_cast<long long *>(w + L.bmax),
+             reinterpret_cast<int *>(w + L.bcnt), reinterpret_cast<long long *>(w + L.thr), reinterpret_cast<int *>(w + L.unit)};
+  constexpr bool kLazy = sizeof(T) == 4;  // FP32: block bounds, see scdm_step_kernel
+  // one resident wave of blocks
   int dev = 0, sms = 0, per_sm = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = kPointMajor ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scdm_pass_pt_kernel<false>, kUpdNT, 0)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scdm_pass_kernel<T, false>, kUpdNT, 0);
-  if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)std::max<long long>(1, std::min<long long>((long long)std::max(per_sm, 1) * sms,
-                                                                            std::min<long long>(kUpdBlocks,
-                                                                                                (N + 255) / 256)));
-  e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st);
-  if (e != cudaSuccess) return e;
-  if constexpr (kPointMajor) {
-    const dim3 tg((unsigned)((N + 31) / 32), (unsigned)((ldt + 31) / 32)), tb(32, 8);
-    scdm_transpose_kernel<<<tg, tb, 0, st>>>(reinterpret_cast<const float *>(psi), n, N, ldt, pt);
-    *launches += 1;
+  if (e == cudaSuccess) {
+    if constexpr (kLazy) {
+      // shared memory above 48 KB, asked for once per call (a driver call of a microsecond)
+      e = cudaFuncSetAttribute(scdm_norm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(scdm_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
+      if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scdm_norm_kernel, kUpdNT, kStageBytes);
+    } else
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scdm_pass_kernel<T, false>, kUpdNT, 0);
   }
+  if (e != cudaSuccess) return e;
+  auto blocks = [&](int per, long long most) {
+    return (unsigned)std::max<long long>(1, std::min({(long long)std::max(per, 1) * sms, (long long)kUpdBlocks, most}));
+  };
+  const unsigned grid = blocks(per_sm, (N + 255) / 256);
+  e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(sa.thr, 0, sizeof(long long) * (n + 1), st);
+  if (e != cudaSuccess) return e;
   for (int k = 0; k < n; ++k) {
     sa.k = k;
-    if constexpr (kPointMajor) {
+    if constexpr (kLazy) {
+      const unsigned steps = blocks(2, (N + kBlk * kUpdNT - 1) / (kBlk * kUpdNT));  // a block per lane
       if (k == 0)
-        scdm_pass_pt_kernel<true><<<grid, kUpdNT, 0, st>>>(pt, n, ldt, N, d, sa);
+        scdm_norm_kernel<<<grid, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
       else
-        scdm_pass_pt_kernel<false><<<grid, kUpdNT, 0, st>>>(pt, n, ldt, N, d, sa);
+        scdm_step_kernel<<<steps, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
     } else {
       if (k == 0)
         scdm_pass_kernel<T, true><<<grid, kUpdNT, 0, st>>>(psi, n, N, d, sa);
@@ -605,7 +948,7 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
   const unsigned g1 = (unsigned)((nn + kSmallNT - 1) / kSmallNT), g2 = (unsigned)((2 * nn + kSmallNT - 1) / kSmallNT);
   scdm_gather_kernel<T><<<g1, kSmallNT, 0, st>>>(psi, n, N, res->piv, M);
   gram_t_kernel<<<g1, kSmallNT, 0, st>>>(M, n, S);
-  frob_kernel<<<1, kSelNT, 0, st>>>(S, n, f);
+  frob_kernel<<<1, 1024, 0, st>>>(S, n, f);
   ns_start_kernel<<<g1, kSmallNT, 0, st>>>(S, n, f, Y[0], Z[0]);
   *launches += 4;
   // Newton-Schulz in chunks of kNsChunk iterations; between chunks the host reads the last two
