@@ -565,6 +565,10 @@ ChainParams chain_params(const ace_desc &d, bool fp64) {
     const double pack = 8.0 * d.n[0] * d.n[1] * d.n[2];
     c.streams = pack > 18e6 ? 3 : 4;
     c.B = std::min(16, std::max(1, (int)std::lround(60e6 / (c.streams * pack))));
+  } else {
+    // FP64 form: bound by the FP64 pipe wherever the scratch lies; batches of about 128 MB in all fill the
+    // GPU on small grids
+    c.B = std::min(16, std::max(1, (int)std::lround(128e6 / (c.streams * 16.0 * d.n[0] * d.n[1] * d.n[2]))));
   }
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -587,57 +591,42 @@ ChainParams chain_params(const ace_desc &d, bool fp64) {
 
 // Five pencil passes per batch of packs (any compiled grid).
 int form_packs(const std::vector<int2> &pr, int RB, std::vector<int4> &packs);
-std::vector<int> form_rounds(std::vector<int4> &packs, int norb);
 
-// Five pencil passes per batch of packs, one stream.  The FP64 form takes its packs in rounds on
-// disjoint orbitals (batches never span two rounds), so that W repeats bit for bit.
-template <typename T>
-ace_status run_chain_pencil(ace_op *op, const T *phi, const T *Kd, const cpx<T> *const *twd, int count,
+// Five pencil passes per batch of packs, one stream (FP32; the FP64 form runs run_chain_f64).
+ace_status run_chain_pencil(ace_op *op, const float *phi, const float *Kd, const cpx<float> *const *twd, int count,
                             std::vector<void *> &temps) {
   const ace_desc &d = op->desc;
   const long long N = op->N;
   cudaStream_t st = op->stream;
   const int npacks = (count + 1) / 2;
   const double scratch_budget = (double)env_int("ACE_SCRATCH_MB", 64) * 1048576.0;
-  int batch = (int)std::max(1.0, std::floor(scratch_budget / (double)(sizeof(cpx<T>) * N)));
+  int batch = (int)std::max(1.0, std::floor(scratch_budget / (double)(sizeof(cpx<float>) * N)));
   batch = std::min(batch, std::max(npacks, 1));
   batch = std::min(batch, 65535);
   void *tmp = nullptr;
-  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<T>) * (size_t)N * batch, st), "alloc scratch");
+  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<float>) * (size_t)N * batch, st), "alloc scratch");
   temps.push_back(tmp);
-  ace::PairPassArgs<T> a{};
+  ace::PairPassArgs<float> a{};
   a.phi = phi;
-  a.W = static_cast<T *>(op->W);
-  a.scratch = static_cast<cpx<T> *>(tmp);
+  a.W = static_cast<float *>(op->W);
+  a.scratch = static_cast<cpx<float> *>(tmp);
   a.packs = op->packs;
   a.kernel = Kd;
   a.N = N;
   a.n1 = d.n[0];
   a.n2 = d.n[1];
   a.n3 = d.n[2];
-  std::vector<int> rb = {0, npacks};
-  if (op->fp64) {
-    std::vector<int4> packs;
-    form_packs(op->pairs_h, 1, packs);
-    rb = form_rounds(packs, op->n);
-    ACE_CUDA(cudaMallocAsync(&tmp, sizeof(int4) * packs.size(), st), "alloc packs");
-    temps.push_back(tmp);
-    ACE_CUDA(host_upload(op, tmp, packs.data(), sizeof(int4) * packs.size(), st), "pack upload");
-    a.packs = static_cast<const int4 *>(tmp);
-  }
-  for (size_t r = 0; r + 1 < rb.size(); ++r)
-    for (int p0 = rb[r]; p0 < rb[r + 1]; p0 += batch) {
-      const int nb = std::min(batch, rb[r + 1] - p0);
-      a.pack0 = p0;
-      const int modes[5] = {ace::PASS_FWD3_PAIR, ace::PASS_FWD2, ace::PASS_CONV1, ace::PASS_INV2,
-                            ace::PASS_INV3_ACC};
-      const int axis[5] = {2, 1, 0, 1, 2};
-      for (int k = 0; k < 5; ++k) {
-        a.tw = twd[axis[k]];
-        ACE_CUDA(ace::launch_pair_pass<T>(modes[k], a, nb, st), "pair pass");
-        ++op->launches;
-      }
+  for (int p0 = 0; p0 < npacks; p0 += batch) {
+    const int nb = std::min(batch, npacks - p0);
+    a.pack0 = p0;
+    const int modes[5] = {ace::PASS_FWD3_PAIR, ace::PASS_FWD2, ace::PASS_CONV1, ace::PASS_INV2, ace::PASS_INV3_ACC};
+    const int axis[5] = {2, 1, 0, 1, 2};
+    for (int k = 0; k < 5; ++k) {
+      a.tw = twd[axis[k]];
+      ACE_CUDA(ace::launch_pair_pass<float>(modes[k], a, nb, st), "pair pass");
+      ++op->launches;
     }
+  }
   return ACE_OK;
 }
 
@@ -730,40 +719,6 @@ int form_packs(const std::vector<int2> &pr, int RB, std::vector<int4> &packs) {
   return nshared;
 }
 
-// Reorders packs into rounds whose packs touch disjoint orbitals (first fit in pack order) and
-// returns the start of every round in the new order, followed by the end.  Inside a round each W
-// element receives at most one addition, so a chain run round after round adds the terms of every
-// element in one fixed order: the FP64 form repeats bit for bit.
-std::vector<int> form_rounds(std::vector<int4> &packs, int norb) {
-  std::vector<std::vector<int4>> rounds;
-  std::vector<std::vector<unsigned char>> used;
-  for (const int4 &p : packs) {
-    const int rows[4] = {p.x, p.y, p.z, p.w};
-    size_t r = 0;
-    for (; r < rounds.size(); ++r) {
-      bool free_ = true;
-      for (int k = 0; k < 4 && free_; ++k)
-        if (rows[k] >= 0 && used[r][rows[k]]) free_ = false;
-      if (free_) break;
-    }
-    if (r == rounds.size()) {
-      rounds.emplace_back();
-      used.emplace_back((size_t)norb, (unsigned char)0);
-    }
-    for (int k = 0; k < 4; ++k)
-      if (rows[k] >= 0) used[r][rows[k]] = 1;
-    rounds[r].push_back(p);
-  }
-  std::vector<int> bounds;
-  packs.clear();
-  for (const auto &rd : rounds) {
-    bounds.push_back((int)packs.size());
-    packs.insert(packs.end(), rd.begin(), rd.end());
-  }
-  bounds.push_back((int)packs.size());
-  return bounds;
-}
-
 // Persistent chain of one or more builds on one grid: every pack of every build in one launch
 // (persistent_chain.cuh) on stream st.  The packs are either on the host (packs, with pack_build the
 // build of each pack, empty for one build), or, with packs empty, the builds' device lists `dev`,
@@ -853,116 +808,66 @@ ace_status run_chain_persistent(ace_op *op, cudaStream_t st, const DeviceTables 
   return ACE_OK;
 }
 
-// Plane, pencil, plane per batch; packs grouped by their shared first orbital.
-template <typename T>
-ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, const ace::PlaneOps<T> &pops,
+// Side streams of a chain on op's lane, forked from op->stream.
+ace_status fork_side(ace_op *op, int nstreams, cudaStream_t *side, cudaEvent_t *ev) {
+  for (int k = 0; k < kSide; ++k) side[k] = op->stream;
+  if (nstreams < 2) return ACE_OK;
+  ACE_CUDA(cudaEventCreateWithFlags(ev, cudaEventDisableTiming), "event");
+  ACE_CUDA(cudaEventRecord(*ev, op->stream), "event");
+  for (int k = 0; k < nstreams; ++k) {
+    ACE_CUDA(get_side_stream(op->dev, kSide * op->lane + k, &side[k]), "side stream");
+    ACE_CUDA(cudaStreamWaitEvent(side[k], *ev, 0), "wait");
+  }
+  return ACE_OK;
+}
+
+// Mixed form: plane, pencil, plane per batch of packs (line_pair.cuh).
+ace_status run_chain_plane(ace_op *op, const float *phi, const DeviceTables *tab, const ace::PlaneOps<float> &pops,
                            int count, std::vector<void *> &temps, const ChainParams &cp, int max_packs = -1) {
   const ace_desc &d = op->desc;
   const long long N = op->N;
   cudaStream_t st = op->stream;
-  const int G = cp.G;
   const int nstreams = std::min(kSide, std::max(1, cp.streams));
   // few packs: smaller batches, so that every side stream has one
-  const int B = std::max(G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams));
-  const bool acc = pops.acc_fits && G > 1;
+  const int B = std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams));
   std::vector<int4> packs;
-  std::vector<int4> groups;
-  int nshared = form_packs(op->pairs_h, cp.RB, packs);
-  // FP64 form: rounds of packs on disjoint orbitals, one pack per group, the side streams joined
-  // between rounds (deterministic W)
-  const bool rounds_on = op->fp64;
-  std::vector<int> rb;
-  if (rounds_on) {
-    rb = form_rounds(packs, op->n);
-    nshared = 0;
-  }
-  const bool acc_on = acc && !rounds_on;
-  // groups: runs of at most G consecutive packs with the same shared orbital (accumulated in
-  // shared memory by the inverse pass when acc); mixed packs are groups of their own
-  for (int k = 0; k < (int)packs.size();) {
-    int k1 = k + 1;
-    if (k < nshared)
-      while (k1 < nshared && k1 - k < G && packs[k1].x == packs[k].x) ++k1;
-    groups.push_back(make_int4(k, k1 - k, (acc_on && k < nshared) ? packs[k].x : -1, 0));
-    k = k1;
-  }
-  // batches of whole groups holding at most B packs (never across a round boundary); round_end[b]
-  // marks the last batch of a round
-  std::vector<int2> batches;  // (first group, end group)
-  std::vector<char> round_end;
-  {
-    size_t ri = 1;
-    int gb = 0, cnt = 0;
-    for (int g = 0; g < (int)groups.size(); ++g) {
-      const bool new_round = rounds_on && ri < rb.size() && groups[g].x == rb[ri];
-      if ((cnt + groups[g].y > B || new_round) && g > gb) {
-        batches.push_back(make_int2(gb, g));
-        round_end.push_back(new_round ? 1 : 0);
-        gb = g;
-        cnt = 0;
-      }
-      if (new_round) ++ri;
-      cnt += groups[g].y;
-    }
-    if (gb < (int)groups.size()) {
-      batches.push_back(make_int2(gb, (int)groups.size()));
-      round_end.push_back(1);
-    }
-  }
+  form_packs(op->pairs_h, cp.RB, packs);
   void *tmp = nullptr;
-  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(int4) * (packs.size() + groups.size()), st), "alloc packs");
+  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(int4) * packs.size(), st), "alloc packs");
   temps.push_back(tmp);
   int4 *packs_d = static_cast<int4 *>(tmp);
-  int4 *groups_d = packs_d + packs.size();
-  std::vector<int4> up(packs);
-  up.insert(up.end(), groups.begin(), groups.end());
-  ACE_CUDA(host_upload(op, packs_d, up.data(), sizeof(int4) * up.size(), st), "pack upload");
-  // complex values of one pack in the scratch (FP32: 16-byte units of two lines of axis 2)
-  const size_t pack_elems =
-      sizeof(T) == 4 ? (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2) * 2 : (size_t)N;
-  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<T>) * pack_elems * B * nstreams, st), "alloc scratch");
+  ACE_CUDA(host_upload(op, packs_d, packs.data(), sizeof(int4) * packs.size(), st), "pack upload");
+  // complex values of one pack in the scratch (16-byte units of two lines of axis 2)
+  const size_t pack_elems = (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2) * 2;
+  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<float>) * pack_elems * B * nstreams, st), "alloc scratch");
   temps.push_back(tmp);
-  cpx<T> *scratch_all = static_cast<cpx<T> *>(tmp);
-  // plane maxima for the plane skip (mixed form), on st before the side streams fork from it
-  float skip_rel = 0.f;
-  if constexpr (sizeof(T) == 4) {
-    skip_rel = plane_skip_rel(false);
-    if (skip_rel > 0.f) ACE_CUDA(plane_max_table(op, phi, st), "plane maxima");
-  }
+  cpx<float> *scratch_all = static_cast<cpx<float> *>(tmp);
+  // plane maxima for the plane skip, on st before the side streams fork from it
+  const float skip_rel = plane_skip_rel(false);
+  if (skip_rel > 0.f) ACE_CUDA(plane_max_table(op, phi, st), "plane maxima");
   // consecutive batches alternate between side streams (own scratch each) so that one batch's
   // kernels fill the tail of the previous one; W is only touched by atomic adds
   cudaStream_t side[kSide];
-  for (int k = 0; k < kSide; ++k) side[k] = st;
   cudaEvent_t fork = nullptr;
-  cudaEvent_t rev[kSide] = {};
-  if (nstreams > 1 && rounds_on)
-    for (int k = 0; k < nstreams; ++k) ACE_CUDA(cudaEventCreateWithFlags(&rev[k], cudaEventDisableTiming), "event");
-  if (nstreams > 1) {
-    ACE_CUDA(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming), "event");
-    ACE_CUDA(cudaEventRecord(fork, st), "event");
-    for (int k = 0; k < nstreams; ++k) {
-      ACE_CUDA(get_side_stream(op->dev, kSide * op->lane + k, &side[k]), "side stream");
-      ACE_CUDA(cudaStreamWaitEvent(side[k], fork, 0), "wait");
-    }
-  }
+  const ace_status fs = fork_side(op, nstreams, side, &fork);
+  if (fs != ACE_OK) return fs;
   // ask L2 to keep each stream's FFT scratch resident between the three passes (a per-context
   // set-aside of the L2 for persisting lines; ACE_L2_PERSIST_MB=0 turns it off)
   const int persist_mb = cp.persist_mb;
   if (persist_mb > 0 && nstreams > 1) {
     for (int k = 0; k < nstreams; ++k)
       l2_window(side[k], op->dev, scratch_all + (size_t)k * B * pack_elems,
-                std::min<size_t>(((size_t)persist_mb << 20) / (size_t)nstreams, sizeof(cpx<T>) * (size_t)B * pack_elems),
+                std::min<size_t>(((size_t)persist_mb << 20) / (size_t)nstreams, sizeof(cpx<float>) * (size_t)B * pack_elems),
                 persist_mb);
   }
 
-  ace::PlaneArgs<T> pa;
+  ace::PlaneArgs<float> pa;
   pa.phi = phi;
-  pa.W = static_cast<T *>(op->W);
+  pa.W = static_cast<float *>(op->W);
   pa.scratch = scratch_all;
   pa.packs = packs_d;
-  pa.groups = groups_d;
-  pa.tw2 = static_cast<const cpx<T> *>(tab->tw[1]);
-  pa.tw3 = static_cast<const cpx<T> *>(tab->tw[2]);
+  pa.tw2 = static_cast<const cpx<float> *>(tab->tw[1]);
+  pa.tw3 = static_cast<const cpx<float> *>(tab->tw[2]);
   pa.N = N;
   pa.n1 = d.n[0];
   pa.n2 = d.n[1];
@@ -971,46 +876,29 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
   pa.pmax = skip_rel > 0.f ? op->pmax : nullptr;
   pa.gmax = skip_rel > 0.f ? op->gmax : nullptr;
   pa.skip_rel = skip_rel;
-  ace::PairPassArgs<T> ca;
+  ace::PairPassArgs<float> ca;
   ca.phi = phi;
-  ca.W = static_cast<T *>(op->W);
+  ca.W = static_cast<float *>(op->W);
   ca.scratch = scratch_all;
   ca.packs = packs_d;
-  ca.kernel = static_cast<const T *>(sizeof(T) == 4 ? tab->Klp : tab->Kperm);
-  ca.tw = static_cast<const cpx<T> *>(tab->tw[0]);
+  ca.kernel = static_cast<const float *>(tab->Klp);
+  ca.tw = static_cast<const cpx<float> *>(tab->tw[0]);
   ca.N = N;
   ca.n1 = d.n[0];
   ca.n2 = d.n[1];
   ca.n3 = d.n[2];
   ca.conv_tile = cp.conv;
-  for (size_t bi = 0; bi < batches.size(); ++bi) {
-    const int2 b = batches[bi];
-    if (max_packs >= 0 && groups[b.x].x >= max_packs) break;  // autotuning sample
-    const int k = (int)(bi % nstreams);
-    const int p0 = groups[b.x].x;
-    const int p1 = groups[b.y - 1].x + groups[b.y - 1].y;
+  const int np = (int)packs.size();
+  for (int p0 = 0, bi = 0; p0 < np; p0 += B, ++bi) {
+    if (max_packs >= 0 && p0 >= max_packs) break;  // autotuning sample
+    const int k = bi % nstreams, nb = std::min(B, np - p0);
     pa.scratch = scratch_all + (size_t)k * B * pack_elems;
     ca.scratch = pa.scratch;
-    pa.pack0 = p0;
-    pa.batch0 = p0;
-    pa.group0 = b.x;
-    ca.pack0 = p0;
-    ACE_CUDA(pops.fwd(pa, p1 - p0, side[k]), "plane forward");
-    if constexpr (sizeof(T) == 4) {
-      ACE_CUDA(ace::launch_line_pair_conv(ca, p1 - p0, side[k]), "pencil pass");
-      ACE_CUDA(pops.inv(pa, p1 - p0, false, side[k]), "plane inverse");
-    } else {
-      ACE_CUDA(ace::launch_conv_pass<T>(ca, p1 - p0, side[k]), "pencil pass");
-      ACE_CUDA(pops.inv(pa, b.y - b.x, acc_on, side[k]), "plane inverse");
-    }
+    pa.pack0 = pa.batch0 = ca.pack0 = p0;
+    ACE_CUDA(pops.fwd(pa, nb, side[k]), "plane forward");
+    ACE_CUDA(ace::launch_line_pair_conv(ca, nb, side[k]), "pencil pass");
+    ACE_CUDA(pops.inv(pa, nb, side[k]), "plane inverse");
     op->launches += 3;
-    if (rounds_on && nstreams > 1 && round_end[bi]) {
-      // every stream waits for every other one: the next round starts after this one ends
-      for (int j = 0; j < nstreams; ++j) ACE_CUDA(cudaEventRecord(rev[j], side[j]), "event");
-      for (int j = 0; j < nstreams; ++j)
-        for (int q = 0; q < nstreams; ++q)
-          if (q != j) ACE_CUDA(cudaStreamWaitEvent(side[j], rev[q], 0), "round join");
-    }
   }
   if (nstreams > 1) {
     for (int k = 0; k < nstreams; ++k) {
@@ -1019,9 +907,91 @@ ace_status run_chain_plane(ace_op *op, const T *phi, const DeviceTables *tab, co
       ACE_CUDA(cudaStreamWaitEvent(st, fork, 0), "join");
     }
     cudaEventDestroy(fork);
-    for (int k = 0; k < nstreams; ++k)
-      if (rev[k]) cudaEventDestroy(rev[k]);
   }
+  return ACE_OK;
+}
+
+// FP64 form: the transforms of each batch of packs on a side stream (plane, pencil, plane where the plane
+// shape is compiled, pops non-null; else five pencil passes) leave the potentials in the batch's scratch;
+// op->stream adds them into W batch after batch, in pack order, so that W repeats bit for bit.
+ace_status run_chain_f64(ace_op *op, const double *phi, const DeviceTables *tab, const ace::PlaneOps<double> *pops,
+                         int count, std::vector<void *> &temps, const ChainParams &cp, int max_packs = -1) {
+  const ace_desc &d = op->desc;
+  const long long N = op->N;
+  cudaStream_t st = op->stream;
+  const int nstreams = std::min(kSide, std::max(1, cp.streams));
+  const int B = std::min(65535, std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams)));
+  std::vector<int4> packs;
+  form_packs(op->pairs_h, cp.RB, packs);
+  void *tmp = nullptr;
+  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(int4) * packs.size(), st), "alloc packs");
+  temps.push_back(tmp);
+  int4 *packs_d = static_cast<int4 *>(tmp);
+  ACE_CUDA(host_upload(op, packs_d, packs.data(), sizeof(int4) * packs.size(), st), "pack upload");
+  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<double>) * (size_t)N * B * nstreams, st), "alloc scratch");
+  temps.push_back(tmp);
+  cpx<double> *scratch_all = static_cast<cpx<double> *>(tmp);
+  cudaStream_t side[kSide];
+  cudaEvent_t ev = nullptr;
+  const ace_status fs = fork_side(op, nstreams, side, &ev);
+  if (fs != ACE_OK) return fs;
+  struct Events {
+    cudaEvent_t ev[kSide] = {};
+    ~Events() {
+      for (cudaEvent_t e : ev)
+        if (e) cudaEventDestroy(e);
+    }
+  } added;  // per side stream: its last batch has been added into W
+  if (nstreams > 1)
+    for (int k = 0; k < nstreams; ++k) ACE_CUDA(cudaEventCreateWithFlags(&added.ev[k], cudaEventDisableTiming), "event");
+  ace::PlaneArgs<double> pa{};
+  pa.phi = phi;
+  pa.packs = packs_d;
+  pa.tw2 = static_cast<const cpx<double> *>(tab->tw[1]);
+  pa.tw3 = static_cast<const cpx<double> *>(tab->tw[2]);
+  pa.N = N;
+  pa.n1 = d.n[0];
+  ace::PairPassArgs<double> ca{};
+  ca.phi = phi;
+  ca.packs = packs_d;
+  ca.kernel = static_cast<const double *>(pops ? tab->Kperm : tab->K);
+  ca.N = N;
+  ca.n1 = d.n[0];
+  ca.n2 = d.n[1];
+  ca.n3 = d.n[2];
+  const int np = (int)packs.size();
+  for (int p0 = 0, bi = 0; p0 < np; p0 += B, ++bi) {
+    if (max_packs >= 0 && p0 >= max_packs) break;  // autotuning sample
+    const int k = bi % nstreams, nb = std::min(B, np - p0);
+    pa.scratch = ca.scratch = scratch_all + (size_t)k * B * (size_t)N;
+    pa.pack0 = pa.batch0 = ca.pack0 = p0;
+    // the scratch's previous batch has been added
+    if (nstreams > 1 && bi >= nstreams) ACE_CUDA(cudaStreamWaitEvent(side[k], added.ev[k], 0), "wait");
+    if (pops) {
+      ca.tw = static_cast<const cpx<double> *>(tab->tw[0]);
+      ACE_CUDA(pops->fwd(pa, nb, side[k]), "plane forward");
+      ACE_CUDA(ace::launch_conv_pass<double>(ca, nb, side[k]), "pencil pass");
+      ACE_CUDA(pops->inv(pa, nb, side[k]), "plane inverse");
+      op->launches += 3;
+    } else {
+      const int modes[5] = {ace::PASS_FWD3_PAIR, ace::PASS_FWD2, ace::PASS_CONV1, ace::PASS_INV2, ace::PASS_INV3};
+      const int axis[5] = {2, 1, 0, 1, 2};
+      for (int m = 0; m < 5; ++m) {
+        ca.tw = static_cast<const cpx<double> *>(tab->tw[axis[m]]);
+        ACE_CUDA(ace::launch_pair_pass<double>(modes[m], ca, nb, side[k]), "pair pass");
+        ++op->launches;
+      }
+    }
+    if (nstreams > 1) {
+      ACE_CUDA(cudaEventRecord(ev, side[k]), "event");
+      ACE_CUDA(cudaStreamWaitEvent(st, ev, 0), "wait");
+    }
+    ACE_CUDA(ace::launch_pair_accumulate<double>(phi, static_cast<double *>(op->W), pa.scratch, packs_d + p0, nb, N, st),
+             "accumulation");
+    ++op->launches;
+    if (nstreams > 1) ACE_CUDA(cudaEventRecord(added.ev[k], st), "event");
+  }
+  if (ev) cudaEventDestroy(ev);
   return ACE_OK;
 }
 
@@ -1289,11 +1259,14 @@ ace_status run_chain(ace_op *op, const T *phi, int count) {
         {phi, static_cast<T *>(op->W), static_cast<const T *>(tab->Kperm), pm, gm}};
     return run_chain_persistent<T>(op, op->stream, tab, qops, packs, {}, {}, 0, one, temps, cp);
   }
-  if (count > 0 && plane) return run_chain_plane<T>(op, phi, tab, pops, count, temps, cp);
   if (count > 0) {
-    const cpx<T> *twd[3] = {static_cast<const cpx<T> *>(tab->tw[0]), static_cast<const cpx<T> *>(tab->tw[1]),
-                            static_cast<const cpx<T> *>(tab->tw[2])};
-    return run_chain_pencil<T>(op, phi, static_cast<const T *>(tab->K), twd, count, temps);
+    if constexpr (sizeof(T) == 8) return run_chain_f64(op, phi, tab, plane ? &pops : nullptr, count, temps, cp);
+    else if (plane) return run_chain_plane(op, phi, tab, pops, count, temps, cp);
+    else {
+      const cpx<T> *twd[3] = {static_cast<const cpx<T> *>(tab->tw[0]), static_cast<const cpx<T> *>(tab->tw[1]),
+                              static_cast<const cpx<T> *>(tab->tw[2])};
+      return run_chain_pencil(op, phi, static_cast<const T *>(tab->K), twd, count, temps);
+    }
   }
   return ACE_OK;
 }
@@ -2237,6 +2210,10 @@ ace_status ace_autotune(const ace_desc *desc, const void *phi, ace_dtype dtype, 
     // a sample long enough (about 40% of a 128-orbital build on 96^3) for the L2 reuse of the
     // blocked pack order and of the persisting scratch window to show in the timing
     const int sample = std::min((count + 1) / 2, 480);
+    auto run_sample = [&](const ChainParams &c, std::vector<void *> &tmp) {
+      if constexpr (sizeof(T) == 8) return run_chain_f64(op, phi_w, op->tab, &pops, count, tmp, c, sample);
+      else return run_chain_plane(op, phi_w, op->tab, pops, count, tmp, c, sample);
+    };
     cudaEvent_t e0, e1;
     ACE_CUDA(cudaEventCreate(&e0), "event");
     ACE_CUDA(cudaEventCreate(&e1), "event");
@@ -2256,7 +2233,7 @@ ace_status ace_autotune(const ace_desc *desc, const void *phi, ace_dtype dtype, 
           for (int rep = 0; rep < 2; ++rep) {
             std::vector<void *> tmp;
             ACE_CUDA(cudaEventRecord(e0, op->stream), "event");
-            ace_status r = run_chain_plane<T>(op, phi_w, op->tab, pops, count, tmp, c, sample);
+            ace_status r = run_sample(c, tmp);
             ACE_CUDA(cudaEventRecord(e1, op->stream), "event");
             for (void *q : tmp) cudaFreeAsync(q, op->stream);
             if (r != ACE_OK) return r;
@@ -2279,7 +2256,7 @@ ace_status ace_autotune(const ace_desc *desc, const void *phi, ace_dtype dtype, 
         for (int rep = 0; rep < 2; ++rep) {
           std::vector<void *> tmp;
           ACE_CUDA(cudaEventRecord(e0, op->stream), "event");
-          ace_status r = run_chain_plane<T>(op, phi_w, op->tab, pops, count, tmp, c, sample);
+          ace_status r = run_sample(c, tmp);
           ACE_CUDA(cudaEventRecord(e1, op->stream), "event");
           for (void *q : tmp) cudaFreeAsync(q, op->stream);
           if (r != ACE_OK) return r;

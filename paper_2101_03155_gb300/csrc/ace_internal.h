@@ -16,7 +16,8 @@ enum PassMode : int {
   PASS_FWD2 = 1,       // axis 2 forward
   PASS_CONV1 = 2,      // axis 1 forward, multiply by 4 pi/(N |G|^2), axis 1 inverse
   PASS_INV2 = 3,       // axis 2 inverse
-  PASS_INV3_ACC = 4    // axis 3 inverse; epilogue W_a += v_ab phi_b, W_b += v_ab phi_a, ...
+  PASS_INV3_ACC = 4,   // axis 3 inverse; epilogue W_a += v_ab phi_b, W_b += v_ab phi_a, ... (atomic)
+  PASS_INV3 = 5        // axis 3 inverse; the potentials stay in the scratch (FP64)
 };
 
 // A pack holds two pairs (a,b) and (c,d) transformed together as z = rho_ab + i rho_cd; the
@@ -44,9 +45,7 @@ struct PlaneArgs {
   T *W;                // [norb][N]
   cpx<T> *scratch;     // [batch][N], pack p of the launch at p - batch0
   const int4 *packs;   // all packs of the build
-  const int4 *groups;  // (first pack, pack count, shared first orbital or -1, 0)
-  int pack0;           // forward pass: first pack of this launch
-  int group0;          // inverse pass: first group of this launch
+  int pack0;           // first pack of this launch
   int batch0;          // first pack of the batch held in the scratch
   const cpx<T> *tw2;   // [N2] e^{-2 pi i e / N2}
   const cpx<T> *tw3;   // [N3] e^{-2 pi i e / N3}
@@ -62,9 +61,8 @@ struct PlaneArgs {
 template <typename T>
 struct PlaneOps {
   cudaError_t (*fwd)(const PlaneArgs<T> &, int npacks, cudaStream_t);
-  // FP64: over groups [group0, group0 + count); FP32: over packs [pack0, pack0 + count)
-  cudaError_t (*inv)(const PlaneArgs<T> &, int count, bool acc, cudaStream_t);
-  bool acc_fits;  // the inverse pass can keep a plane of W_i partial sums in shared memory
+  // FP32: adds W; FP64: leaves the potentials in the scratch
+  cudaError_t (*inv)(const PlaneArgs<T> &, int npacks, cudaStream_t);
 };
 bool plane_ops_f64(int n2, int n3, PlaneOps<double> *out);
 
@@ -133,6 +131,12 @@ cudaError_t launch_flag_fanout(const int *src, int *const *dst, int n, cudaStrea
 cudaError_t launch_queue_assemble(const QueueSrc *src, int nb, int4 *packs_out, int *pack_build, int *np_out,
                                   cudaStream_t st);
 bool persist_ops_f32_large(int n1, int n2, int n3, PersistOps<float> *out);
+
+// W of `npacks` packs (Eq. vx) from their potentials z = v_ab + i v_cd [npacks][N] in natural order, added in
+// pack order by one thread per point: no atomics, the same bits on every run.
+template <typename T>
+cudaError_t launch_pair_accumulate(const T *phi, T *W, const cpx<T> *z, const int4 *packs, int npacks, long long N,
+                                   cudaStream_t st);
 
 // Launch one pass over `npacks` packs (grid.y); returns cudaErrorInvalidValue if the axis
 // length has no compiled plan.

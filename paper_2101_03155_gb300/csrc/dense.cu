@@ -23,19 +23,60 @@
 namespace ace {
 
 // ----------------------------------------------------------------------------------------
-// Gram: 64 x 64 output tile per CTA, 256 threads with 4 x 4 register tiles, K chunk per CTA.
+// General Gram (the FP64 form, and FP32 point counts off the 16-byte grid): BM x BM output tile per CTA
+// (BM 16 or 32), 16 x 16 threads with (BM / 16)^2 outputs each, one chunk of K per CTA.
+//   Bound by the FP64 pipe (2 multiply-adds per cycle and SM), so what counts is that no output of a tile
+// is padding and that every SM has the same number of chunks: 64 x 64 tiles of 4096-point chunks left 12
+// orbitals at 28 times the work on 21 SMs (4.8 ms for 86,400 points), and 64 orbitals on 72^3 on 91 of
+// 152 SMs (5.3 ms).  Small tiles cost loads (each row is read once per tile of the other operand), which
+// stay below 2% of the FP64 time.
 // ----------------------------------------------------------------------------------------
-constexpr int GR_BM = 64, GR_BK = 32, GR_CHUNK = 4096, GR_NT = 256;
+constexpr int GR_BK = 32, GR_NT = 256;
+constexpr long long GR_LONGEST = 1ll << 17;  // FP64 (FP32 sums go to FP64 every 4096 points)
+
+struct GramPlan {
+  int bm, nbx, tiles;
+  long long chunk, chunks;
+};
+// Chunks of K, at most `longest` points, such that tiles x chunks CTAs spread evenly over the SMs (four to
+// sixteen per SM).
+static GramPlan gram_plan(int nx, int ny, long long K, bool upper_only, long long longest) {
+  GramPlan p;
+  p.bm = nx <= 16 && ny <= 16 ? 16 : 32;
+  p.nbx = (nx + p.bm - 1) / p.bm;
+  const int nby = (ny + p.bm - 1) / p.bm;
+  p.tiles = upper_only ? p.nbx * (p.nbx + 1) / 2 : p.nbx * nby;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      sms < 1)
+    sms = 152;
+  const long long least = std::max(1ll, (4ll * sms + p.tiles - 1) / p.tiles);
+  const long long most = std::max(1ll, std::min(65535ll, (K + 2 * GR_BK - 1) / (2 * GR_BK)));
+  long long best = std::min(least, most);
+  double fill = 0.0;
+  for (long long c = best; c <= std::min(most, 4 * least); ++c) {
+    const long long ctas = c * p.tiles, waves = (ctas + sms - 1) / sms;
+    const double f = (double)ctas / (double)(waves * sms);
+    if (f > fill + 0.01) {
+      fill = f;
+      best = c;
+    }
+  }
+  p.chunk = std::min(longest, ((K + best - 1) / best + GR_BK - 1) / GR_BK * GR_BK);
+  p.chunks = (K + p.chunk - 1) / p.chunk;
+  return p;
+}
 
 // With `partial` non-null the CTA of chunk c writes its scaled tile sums to partial[c] (no
 // atomics) and gram_chunks_reduce_kernel adds the chunks in a fixed order: the result is then
 // the same bit for bit on every run.
-template <typename T, bool ABS>
+template <typename T, bool ABS, int BM>
 __global__ void __launch_bounds__(GR_NT) gram_kernel(const T *__restrict__ X, int nx, const T *__restrict__ Y, int ny,
-                                                     long long K, double scale, bool upper_only, int nbx,
+                                                     long long K, long long chunk, double scale, bool upper_only, int nbx,
                                                      double *__restrict__ G, double *__restrict__ partial) {
-  __shared__ T xs[GR_BK][GR_BM + 1];
-  __shared__ T ys[GR_BK][GR_BM + 1];
+  constexpr int RT = BM / 16;
+  __shared__ T xs[GR_BK][BM + 1];
+  __shared__ T ys[GR_BK][BM + 1];
   int bi, bj;
   if (upper_only) {
     // blockIdx.x enumerates tile pairs (bi <= bj) row by row
@@ -50,22 +91,25 @@ __global__ void __launch_bounds__(GR_NT) gram_kernel(const T *__restrict__ X, in
     bi = blockIdx.x % nbx;
     bj = blockIdx.x / nbx;
   }
-  const int i0 = bi * GR_BM, j0 = bj * GR_BM;
-  const long long k0 = (long long)blockIdx.y * GR_CHUNK;
-  const long long k1 = min(K, k0 + GR_CHUNK);
+  const int i0 = bi * BM, j0 = bj * BM;
+  const long long k0 = (long long)blockIdx.y * chunk;
+  const long long k1 = min(K, k0 + chunk);
   const int tid = threadIdx.x;
   const int ty = tid / 16, tx = tid % 16;
   // acc + comp is a compensated (Kahan) running sum of the 32-point partial sums of each tile
-  T acc[4][4], comp[4][4];
+  T acc[RT][RT], comp[RT][RT];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < RT; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = comp[a][b] = (T)0;
+    for (int b = 0; b < RT; ++b) acc[a][b] = comp[a][b] = (T)0;
 
-  for (long long kk = k0; kk < k1; kk += GR_BK) {
-    // load 64 rows x 32 k of X and of Y (coalesced along k)
-    for (int e = tid; e < GR_BM * GR_BK; e += GR_NT) {
-      const int r = e / GR_BK, c = e % GR_BK;
+  // the next step's rows are loaded into registers while this step multiplies (coalesced along k)
+  constexpr int NE = BM * GR_BK / GR_NT;
+  T xn[NE], yn[NE];
+  auto fetch = [&](long long kk) {
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      const int e = tid + q * GR_NT, r = e / GR_BK, c = e % GR_BK;
       const long long k = kk + c;
       T xv = (T)0, yv = (T)0;
       if (k < k1) {
@@ -76,31 +120,41 @@ __global__ void __launch_bounds__(GR_NT) gram_kernel(const T *__restrict__ X, in
         xv = xv < (T)0 ? -xv : xv;
         yv = yv < (T)0 ? -yv : yv;
       }
-      xs[c][r] = xv;
-      ys[c][r] = yv;
+      xn[q] = xv;
+      yn[q] = yv;
+    }
+  };
+  fetch(k0);
+  for (long long kk = k0; kk < k1; kk += GR_BK) {
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      const int e = tid + q * GR_NT, r = e / GR_BK, c = e % GR_BK;
+      xs[c][r] = xn[q];
+      ys[c][r] = yn[q];
     }
     __syncthreads();
-    T part[4][4];
+    if (kk + GR_BK < k1) fetch(kk + GR_BK);
+    T part[RT][RT];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < RT; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) part[a][b] = (T)0;
+      for (int b = 0; b < RT; ++b) part[a][b] = (T)0;
 #pragma unroll 8
     for (int c = 0; c < GR_BK; ++c) {
-      T xr[4], yr[4];
+      T xr[RT], yr[RT];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) xr[a] = xs[c][ty + 16 * a];
+      for (int a = 0; a < RT; ++a) xr[a] = xs[c][ty + 16 * a];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) yr[b] = ys[c][tx + 16 * b];
+      for (int b = 0; b < RT; ++b) yr[b] = ys[c][tx + 16 * b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int a = 0; a < RT; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) part[a][b] += xr[a] * yr[b];
+        for (int b = 0; b < RT; ++b) part[a][b] += xr[a] * yr[b];
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < RT; ++a)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
+      for (int b = 0; b < RT; ++b) {
         const T y = part[a][b] - comp[a][b];
         const T t = acc[a][b] + y;
         comp[a][b] = (t - acc[a][b]) - y;
@@ -109,9 +163,9 @@ __global__ void __launch_bounds__(GR_NT) gram_kernel(const T *__restrict__ X, in
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < RT; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
+    for (int b = 0; b < RT; ++b) {
       const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
       if (i < nx && j < ny) {
         if (partial)
@@ -122,19 +176,27 @@ __global__ void __launch_bounds__(GR_NT) gram_kernel(const T *__restrict__ X, in
     }
 }
 
-// G_ij = sum over the chunks of partial[c]_ij in chunk order (upper_only: j >= i only)
+// G_ij = sum over the chunks of partial[c]_ij in a fixed order (eight interleaved sums; upper_only: j >= i
+// only)
 __global__ void gram_chunks_reduce_kernel(const double *__restrict__ partial, long long chunks, int nx, int ny,
                                           bool upper_only, double *__restrict__ G) {
   const long long ne = (long long)nx * ny;
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (e >= ne || (upper_only && e % ny < e / ny)) return;
-  double s = 0.0;
-  for (long long c = 0; c < chunks; ++c) s += partial[c * ne + e];
-  G[e] = s;
+  double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  long long c = 0;
+  for (; c + 8 <= chunks; c += 8) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s[q] += partial[(c + q) * ne + e];
+  }
+  for (; c < chunks; ++c) s[0] += partial[c * ne + e];
+  G[e] = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
 }
 
 size_t gram_chunks_bytes(int nx, int ny, long long K) {
-  return sizeof(double) * (size_t)((K + GR_CHUNK - 1) / GR_CHUNK) * nx * ny;
+  const long long c = std::max(gram_plan(nx, ny, K, false, GR_LONGEST).chunks,
+                               nx == ny ? gram_plan(nx, ny, K, true, GR_LONGEST).chunks : 0);
+  return sizeof(double) * (size_t)c * nx * ny;
 }
 
 // FP32 operands: 128 x 64 output tile, 256 threads with 8 x 4 outputs each, k-tiles of 16 staged
@@ -451,21 +513,22 @@ cudaError_t launch_gram(const T *X, int nx, const T *Y, int ny, long long K, dou
       return cudaGetLastError();
     }
   }
-  const int nbx = (nx + GR_BM - 1) / GR_BM, nby = (ny + GR_BM - 1) / GR_BM;
-  const int tiles = upper_only ? nbx * (nbx + 1) / 2 : nbx * nby;
-  const long long chunks = (K + GR_CHUNK - 1) / GR_CHUNK;
-  if (chunks > 65535) return cudaErrorInvalidValue;
+  const GramPlan p = gram_plan(nx, ny, K, upper_only, sizeof(T) == 4 ? 4096 : GR_LONGEST);
+  if (p.chunks > 65535) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(G, 0, sizeof(double) * (size_t)nx * ny, st);
   if (e != cudaSuccess) return e;
-  dim3 grid(tiles, (unsigned)chunks);
-  if (abs_values)
-    gram_kernel<T, true><<<grid, GR_NT, 0, st>>>(X, nx, Y, ny, K, scale, upper_only, nbx, G, partial);
+  const dim3 grid(p.tiles, (unsigned)p.chunks);
+  auto run = [&](auto kernel) {
+    kernel<<<grid, GR_NT, 0, st>>>(X, nx, Y, ny, K, p.chunk, scale, upper_only, p.nbx, G, partial);
+  };
+  if (p.bm == 16)
+    abs_values ? run(gram_kernel<T, true, 16>) : run(gram_kernel<T, false, 16>);
   else
-    gram_kernel<T, false><<<grid, GR_NT, 0, st>>>(X, nx, Y, ny, K, scale, upper_only, nbx, G, partial);
+    abs_values ? run(gram_kernel<T, true, 32>) : run(gram_kernel<T, false, 32>);
   e = cudaGetLastError();
   if (e != cudaSuccess || !partial) return e;
   const long long ne = (long long)nx * ny;
-  gram_chunks_reduce_kernel<<<(unsigned)((ne + 127) / 128), 128, 0, st>>>(partial, chunks, nx, ny, upper_only, G);
+  gram_chunks_reduce_kernel<<<(unsigned)((ne + 63) / 64), 64, 0, st>>>(partial, p.chunks, nx, ny, upper_only, G);
   return cudaGetLastError();
 }
 template cudaError_t launch_gram<float>(const float *, int, const float *, int, long long, double, bool, bool,

@@ -228,6 +228,7 @@ ACE_LFACTOR(30, 5, 6)
 ACE_LFACTOR(40, 5, 8)
 ACE_LFACTOR(50, 5, 10)
 ACE_LFACTOR(60, 6, 10)
+ACE_LFACTOR(72, 9, 8)
 ACE_LFACTOR(80, 10, 8)
 ACE_LFACTOR(90, 9, 10)
 ACE_LFACTOR(108, 9, 12)

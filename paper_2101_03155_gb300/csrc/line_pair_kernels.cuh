@@ -95,7 +95,7 @@ struct LpLaunch {
     lp_fwd_kernel<N2, N3><<<dim3(a.n1, npacks), NT, lp_plane_smem(N2, N3), st>>>(a);
     return cudaGetLastError();
   }
-  static cudaError_t inv(const PlaneArgs<float> &a, int npacks, bool, cudaStream_t st) {
+  static cudaError_t inv(const PlaneArgs<float> &a, int npacks, cudaStream_t st) {
     static unsigned long long done = 0;
     const cudaError_t e = smem_attr_once(lp_inv_kernel<N2, N3>, lp_plane_smem(N2, N3), done);
     if (e != cudaSuccess) return e;

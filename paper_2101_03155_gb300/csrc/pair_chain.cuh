@@ -105,7 +105,7 @@ __global__ void __launch_bounds__((PassShape<T, L>::NT)) pair_pass_kernel(PairPa
 
   for (int e = tid; e < L; e += NT) tw[e] = a.tw[e];
 
-  constexpr bool AXIS3 = (MODE == PASS_FWD3_PAIR || MODE == PASS_INV3_ACC);
+  constexpr bool AXIS3 = (MODE == PASS_FWD3_PAIR || MODE == PASS_INV3_ACC || MODE == PASS_INV3);
   long long base, Ns;
   int tvalid;
   if (AXIS3) {
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__((PassShape<T, L>::NT)) pair_pass_kernel(PairPa
     pencil_stage1<T, L, +1, false>(s, tw, tvalid);  // inverse DFT_R1: natural order out
     __syncthreads();
   } else {
-    constexpr int D = (MODE == PASS_INV2 || MODE == PASS_INV3_ACC) ? +1 : -1;
+    constexpr int D = (MODE == PASS_INV2 || MODE == PASS_INV3_ACC || MODE == PASS_INV3) ? +1 : -1;
     pencil_stage1<T, L, D, true>(s, tw, tvalid);
     __syncthreads();
     pencil_stage2<T, L, D>(s, tvalid);
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__((PassShape<T, L>::NT)) pair_pass_kernel(PairPa
         if (!diag2) atomicAdd(a.W + od + e, v.y * a.phi[oc + e]);
       }
     }
-  } else if (MODE == PASS_FWD3_PAIR) {
+  } else if (MODE == PASS_FWD3_PAIR || MODE == PASS_INV3) {
     cpx<T> *dst = z + base;
     for (int e = tid; e < tvalid * L; e += NT) {
       const int t = e / L, k = e - t * L;
@@ -325,7 +325,7 @@ template <typename T, int L>
 cudaError_t launch_pass_L(int mode, const PairPassArgs<T> &a, int npacks, cudaStream_t st) {
   using S = PassShape<T, L>;
   dim3 grid;
-  if (mode == PASS_FWD3_PAIR || mode == PASS_INV3_ACC) {
+  if (mode == PASS_FWD3_PAIR || mode == PASS_INV3_ACC || mode == PASS_INV3) {
     grid.x = (unsigned)(((long long)a.n1 * a.n2 + S::TILE - 1) / S::TILE);
   } else if (mode == PASS_CONV1) {
     grid.x = (unsigned)(((long long)a.n2 * a.n3 + S::TILE - 1) / S::TILE);
@@ -339,6 +339,12 @@ cudaError_t launch_pass_L(int mode, const PairPassArgs<T> &a, int npacks, cudaSt
     case PASS_CONV1: pair_pass_kernel<T, L, PASS_CONV1><<<grid, S::NT, 0, st>>>(a); break;
     case PASS_INV2: pair_pass_kernel<T, L, PASS_INV2><<<grid, S::NT, 0, st>>>(a); break;
     case PASS_INV3_ACC: pair_pass_kernel<T, L, PASS_INV3_ACC><<<grid, S::NT, 0, st>>>(a); break;
+    case PASS_INV3:
+      if constexpr (sizeof(T) == 8) {
+        pair_pass_kernel<T, L, PASS_INV3><<<grid, S::NT, 0, st>>>(a);
+        break;
+      }
+      return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -7,11 +7,10 @@
 // axis-1 pass reads the Coulomb table in the same permuted layout, and the inverse plane pass
 // starts from permuted input and returns natural order, so no reordering pass is needed.
 //
-// The inverse pass handles a group of packs whose pairs share the first orbital i (pairs (i, j1),
-// (i, j2), ...).  With one pack per group (the default) the two W_i contributions of the pack are
-// added with one atomic per point; with larger groups they are summed in shared memory over the
-// group first.  W_j += v_ij phi_i are atomic adds.  Global accesses go one point per lane
-// (coalesced) so that the shared-memory side stays free of bank conflicts.
+// The FP64 form runs these kernels per batch and adds W from the stored potentials afterwards, in pack
+// order (pair_accumulate_kernel); the FP32 bodies serve the persistent chain (persistent_chain.cuh), which
+// adds W atomically.  Global accesses go one point per lane (coalesced) so that the shared-memory side stays
+// free of bank conflicts.
 #pragma once
 
 #include "ace_internal.h"
@@ -392,45 +391,23 @@ __global__ void __launch_bounds__(NT, (plane_min_blocks<T, N2, N3, false>())) pl
 }
 
 // ---------------------------------------------------------------------------------------
-// Inverse plane pass fused with the W accumulation: one CTA per (plane i1, group).
-// Group g covers packs [gstart, gstart + glen); grow >= 0 means every pair of the group has
-// first orbital grow (accumulated in shared memory), grow < 0 a single mixed pack.
+// Inverse plane pass, one CTA per (plane i1, pack): the potentials v_ab + i v_cd in natural order, written
+// over the spectrum plane (read before the first barrier of plane_inverse).
 // ---------------------------------------------------------------------------------------
-template <typename T, int N2, int N3, int NT, bool ACC>
-__global__ void __launch_bounds__(NT, (plane_min_blocks<T, N2, N3, ACC>())) plane_inv_kernel(PlaneArgs<T> a) {
+template <typename T, int N2, int N3, int NT>
+__global__ void __launch_bounds__(NT, (plane_min_blocks<T, N2, N3, false>())) plane_inv_kernel(PlaneArgs<T> a) {
   using S = PlaneShape<N2, N3>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T> *s = reinterpret_cast<cpx<T> *>(smem_raw);
   cpx<T> *tw2 = s + N2 * S::PP;
   cpx<T> *tw3 = tw2 + N2;
-  T *acc = reinterpret_cast<T *>(tw3 + N3);  // NPTS values when ACC
   const int tid = threadIdx.x;
-  const int i1 = blockIdx.x;
-  const int4 grp = a.groups[a.group0 + blockIdx.y];  // (start pack, count, row, unused)
-  const int grow = grp.z;
   for (int e = tid; e < N2; e += NT) tw2[e] = a.tw2[e];
   for (int e = tid; e < N3; e += NT) tw3[e] = a.tw3[e];
-  const bool use_acc = ACC && grow >= 0;
-  if (use_acc)
-    for (int e = tid; e < S::NPTS; e += NT) acc[e] = (T)0;
-  const long long off = (long long)i1 * S::NPTS;
-  for (int q = 0; q < grp.y; ++q) {
-    const int pidx = grp.x + q;
-    const int4 pk = a.packs[pidx];
-    __syncthreads();  // previous pack's epilogue has finished reading s
-    if (!(a.skip_rel > 0.f && inv_plane_negligible(a.pmax, a.gmax, a.n1, i1, pk, a.skip_rel))) {
-      plane_inverse<T, N2, N3, NT>(a.scratch + (long long)(pidx - a.batch0) * a.N + off, s, tw2, tw3);
-      plane_accumulate<T, N2, N3, NT>(a.phi, a.W, a.N, off, pk, s, use_acc ? acc : nullptr);
-    }
-    // the spectrum plane was this pack's last use of it: its lines leave L2 without a write-back
-    // (here, where few registers are live; every read of it ended at plane_inverse's first barrier)
-    if (a.hints & 1) l2_discard<NT>(a.scratch + (long long)(pidx - a.batch0) * a.N + off, sizeof(cpx<T>) * S::NPTS);
-  }
-  if (use_acc) {
-    __syncthreads();
-    T *wr = a.W + (long long)grow * a.N + off;
-    for (int e = tid; e < S::NPTS; e += NT) atomicAdd(wr + e, acc[e]);
-  }
+  cpx<T> *z = a.scratch + (long long)(a.pack0 + (int)blockIdx.y - a.batch0) * a.N + (long long)blockIdx.x * S::NPTS;
+  __syncthreads();
+  plane_inverse<T, N2, N3, NT>(z, s, tw2, tw3);
+  for_points<N2, N3, NT, ACE_INV_UNROLL>([&](int e, int si) { z[e] = s[si]; });
 }
 
 // The dynamic shared-memory limit of a kernel, set once per device (a driver call per launch
@@ -467,10 +444,7 @@ template <typename T, int N2, int N3>
 struct PlaneLaunch {
   static constexpr int NT = plane_threads<T, N2, N3>();
   static size_t fwd_smem() { return sizeof(cpx<T>) * (N2 * PlaneShape<N2, N3>::PP + N2 + N3); }
-  static size_t inv_smem(bool acc) {
-    return fwd_smem() + (acc ? sizeof(T) * (size_t)N2 * N3 : 0);
-  }
-  static bool fits(bool acc) { return inv_smem(acc) <= 227 * 1024 && fwd_smem() <= 227 * 1024; }
+  static bool fits() { return fwd_smem() <= 227 * 1024; }
 
   static cudaError_t fwd(const PlaneArgs<T> &a, int npacks, cudaStream_t st) {
     const size_t sm = fwd_smem();
@@ -480,20 +454,12 @@ struct PlaneLaunch {
     plane_fwd_kernel<T, N2, N3, NT><<<dim3(a.n1, npacks), NT, sm, st>>>(a);
     return cudaGetLastError();
   }
-  static cudaError_t inv(const PlaneArgs<T> &a, int ngroups, bool acc, cudaStream_t st) {
-    const size_t sm = inv_smem(acc);
-    cudaError_t e;
-    if (acc) {
-      static unsigned long long done_acc = 0;
-      e = smem_attr_once(plane_inv_kernel<T, N2, N3, NT, true>, sm, done_acc);
-      if (e != cudaSuccess) return e;
-      plane_inv_kernel<T, N2, N3, NT, true><<<dim3(a.n1, ngroups), NT, sm, st>>>(a);
-    } else {
-      static unsigned long long done = 0;
-      e = smem_attr_once(plane_inv_kernel<T, N2, N3, NT, false>, sm, done);
-      if (e != cudaSuccess) return e;
-      plane_inv_kernel<T, N2, N3, NT, false><<<dim3(a.n1, ngroups), NT, sm, st>>>(a);
-    }
+  static cudaError_t inv(const PlaneArgs<T> &a, int npacks, cudaStream_t st) {
+    const size_t sm = fwd_smem();
+    static unsigned long long done = 0;
+    cudaError_t e = smem_attr_once(plane_inv_kernel<T, N2, N3, NT>, sm, done);
+    if (e != cudaSuccess) return e;
+    plane_inv_kernel<T, N2, N3, NT><<<dim3(a.n1, npacks), NT, sm, st>>>(a);
     return cudaGetLastError();
   }
 };
