@@ -1002,6 +1002,14 @@ template <typename T>
 cudaError_t dense_gram(const T *X, int nx, const T *Y, int ny, long long K, double scale, double *G, int *err,
                        std::vector<void *> &temps, cudaStream_t st, long *launches) {
   if constexpr (sizeof(T) == 4) {
+    if (ace::skinny_gram_ok(X, nx, Y, ny, K)) {
+      void *ws = nullptr;
+      cudaError_t e = cudaMallocAsync(&ws, ace::skinny_gram_bytes(nx, ny, K), st);
+      if (e != cudaSuccess) return e;
+      temps.push_back(ws);
+      *launches += 2;
+      return ace::launch_skinny_gram(X, nx, Y, ny, K, scale, G, ws, st);
+    }
     if (use_tc() && ace::tc_gram_shape_ok(K)) {
       void *ws = nullptr;
       cudaError_t e = cudaMallocAsync(&ws, ace::tc_gram_workspace_bytes(X, nx, Y, ny, K), st);
@@ -1030,6 +1038,7 @@ cudaError_t dense_left_mul(const T *A, int m, int n, const T *Y, long long K, T 
                            long *launches) {
   *launches += 1;
   if constexpr (sizeof(T) == 4) {
+    if (m <= 8) return ace::launch_skinny_left_mul(A, m, n, Y, K, Z, st);
     if (use_tc()) {
       const cudaError_t e = ace::launch_tc_left_mul(A, m, n, Y, K, Z, err, st);
       if (e != cudaErrorNotSupported) return e;  // else the CUDA-core kernel below takes the shape

@@ -163,6 +163,13 @@ cudaError_t launch_gram(const T *X, int nx, const T *Y, int ny, long long K, dou
 size_t gram_chunks_bytes(int nx, int ny, long long K);
 template <typename T>
 cudaError_t launch_left_mul(const T *A, int m, int n, const T *Y, long long K, T *Z, cudaStream_t st);
+// FP32 products with at most 8 rows on one side, on the CUDA cores
+bool skinny_gram_ok(const float *X, int nx, const float *Y, int ny, long long K);
+size_t skinny_gram_bytes(int nx, int ny, long long K);
+cudaError_t launch_skinny_gram(const float *X, int nx, const float *Y, int ny, long long K, double scale, double *G,
+                               void *ws, cudaStream_t st);
+cudaError_t launch_skinny_left_mul(const float *A, int m, int n, const float *Y, long long K, float *Z,
+                                   cudaStream_t st);
 
 // gwork: n*n + n doubles of device workspace, needed when n > 128 (else may be NULL)
 cudaError_t launch_cholesky(const double *M_raw, int n, double spin_factor, double *M, double *L, double *Linv,

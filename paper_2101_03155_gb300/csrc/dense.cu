@@ -537,6 +537,251 @@ template cudaError_t launch_gram<double>(const double *, int, const double *, in
                                          double *, cudaStream_t, double *);
 
 // ----------------------------------------------------------------------------------------
+// FP32 products with at most 8 rows on one side (a few vectors against the stored xi, builds of a
+// few orbitals).  Both are bound by reading the large operand once: 95.5 MB at 64 rows of 72^3, where
+// 4 vectors take 21 us for the coefficients (5.0 TB/s) and a call of ace_apply went from 197 to 86 us.
+// The tensor-core tiles, which take 9 rows and more, pad the short side to 128 and convert every point
+// to BF16 pairs for it; these kernels' FP32 products are also the more exact ones.
+// ----------------------------------------------------------------------------------------
+constexpr int SK_NT = 128;        // threads of both kernels
+constexpr int SK_ROWS = 8;        // large-side rows per warp of the Gram
+constexpr int SK_FOLD = 16;       // 128-point steps summed in FP32 (16 x 4 products per lane) before the FP64 sum
+constexpr int SK_WARPS = 12;      // Gram warps per SM that the split aims at (the 8-row form's residency)
+
+// G_ab = scale * sum_k L_ak S_bk over L of nl rows and S of ns <= MS rows.  A warp takes 8 rows of
+// L and one run of columns; its lanes hold all 8 x MS sums, reading 16 bytes of every row per step.
+// Lane sums are folded into FP64 every SK_FOLD steps; the runs' sums are added by
+// skinny_gram_reduce_kernel in run order.
+template <int MS>
+__global__ void __launch_bounds__(SK_NT, 3) skinny_gram_kernel(const float *__restrict__ L, int nl,
+                                                               const float *__restrict__ S, int ns, long long K,
+                                                               long long run, int groups, int runs,
+                                                               double *__restrict__ partial) {
+  constexpr int NV = SK_ROWS * MS, KEEP = NV >= 32 ? NV / 32 : 1;
+  const int lane = threadIdx.x & 31;
+  const long long task = (long long)blockIdx.x * (SK_NT / 32) + (threadIdx.x >> 5);
+  if (task >= (long long)groups * runs) return;
+  const int g = (int)(task % groups), c = (int)(task / groups);
+  const long long k0 = (long long)c * run, ke = min(K, k0 + run);
+  // rows past the end repeat the last one; their sums are not stored
+  const float *lp[SK_ROWS], *sp[MS];
+#pragma unroll
+  for (int r = 0; r < SK_ROWS; ++r) lp[r] = L + (long long)min(g * SK_ROWS + r, nl - 1) * K;
+#pragma unroll
+  for (int q = 0; q < MS; ++q) sp[q] = S + (long long)min(q, ns - 1) * K;
+  double sum[KEEP];
+#pragma unroll
+  for (int i = 0; i < KEEP; ++i) sum[i] = 0.0;
+  int first = 0;  // index (row * MS + q) of the first value this lane keeps
+  for (long long kb = k0; kb < ke; kb += 128 * SK_FOLD) {
+    float v[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = 0.f;
+    const long long kend = min(ke, kb + 128 * SK_FOLD);
+    for (long long k = kb + 4 * lane; k < kend; k += 128) {
+      float4 s[MS], l[SK_ROWS];
+#pragma unroll
+      for (int r = 0; r < SK_ROWS; ++r) l[r] = __ldg(reinterpret_cast<const float4 *>(lp[r] + k));
+#pragma unroll
+      for (int q = 0; q < MS; ++q) s[q] = __ldg(reinterpret_cast<const float4 *>(sp[q] + k));
+#pragma unroll
+      for (int r = 0; r < SK_ROWS; ++r)
+#pragma unroll
+        for (int q = 0; q < MS; ++q) {
+          float &a = v[r * MS + q];
+          a = fmaf(l[r].x, s[q].x, a);
+          a = fmaf(l[r].y, s[q].y, a);
+          a = fmaf(l[r].z, s[q].z, a);
+          a = fmaf(l[r].w, s[q].w, a);
+        }
+    }
+    __syncwarp();
+    // halving exchange: each step adds the partner's half of the values and keeps the own half
+    first = 0;
+#pragma unroll
+    for (int off = 16, h = NV / 2; off > 0; off >>= 1, h >>= 1) {
+      if (h > 0) {
+        const bool up = (lane & off) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+          const float send = up ? v[i] : v[i + h];
+          v[i] = (up ? v[i + h] : v[i]) + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+        if (up) first += h;
+      } else {
+        v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < KEEP; ++i) sum[i] += (double)v[i];
+  }
+  double *dst = partial + ((long long)c * groups + g) * NV;
+  if (NV < 32 && (lane & (32 / NV - 1))) return;  // lanes that hold the same value
+#pragma unroll
+  for (int i = 0; i < KEEP; ++i) dst[first + i] = sum[i];
+}
+
+// G from the runs' sums: 32 slices of the runs per value (runs of up to 228 at 64 rows: eight loads
+// in flight per thread and one round trip), the slices added in a fixed order.
+constexpr int SKR_SLICES = 32;
+__global__ void __launch_bounds__(32 * SKR_SLICES) skinny_gram_reduce_kernel(const double *__restrict__ partial,
+                                                                             int runs, int groups, int MS, int nl,
+                                                                             int ns, int sl, int ss, double scale,
+                                                                             double *__restrict__ G) {
+  __shared__ double part[SKR_SLICES][33];
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+  const int nv = groups * SK_ROWS * MS, e = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (e < nv) {
+#pragma unroll 8
+    for (int c = slice; c < runs; c += SKR_SLICES) s += partial[(long long)c * nv + e];
+  }
+  part[slice][lane] = s;
+  __syncthreads();
+  if (slice != 0 || e >= nv) return;
+  s = 0.0;
+#pragma unroll
+  for (int i = 0; i < SKR_SLICES; ++i) s += part[i][lane];
+  const int a = e / MS, b = e % MS;
+  if (a < nl && b < ns) G[(long long)a * sl + (long long)b * ss] = scale * s;
+}
+
+struct SkinnyPlan {
+  int ms, groups, runs;
+  long long run;
+};
+static SkinnyPlan skinny_gram_plan(int nl, int ns, long long K) {
+  SkinnyPlan p;
+  p.ms = ns <= 1 ? 1 : ns <= 2 ? 2 : ns <= 4 ? 4 : 8;
+  p.groups = (nl + SK_ROWS - 1) / SK_ROWS;
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long want = std::max(1, sms * SK_WARPS / p.groups);
+  p.run = std::max(128LL, ((K + want - 1) / want + 127) / 128 * 128);
+  p.runs = (int)((K + p.run - 1) / p.run);
+  return p;
+}
+
+bool skinny_gram_ok(const float *X, int nx, const float *Y, int ny, long long K) {
+  return std::min(nx, ny) <= 8 && K % 4 == 0 &&
+         ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0;
+}
+
+size_t skinny_gram_bytes(int nx, int ny, long long K) {
+  const SkinnyPlan p = skinny_gram_plan(std::max(nx, ny), std::min(nx, ny), K);
+  return sizeof(double) * (size_t)p.runs * p.groups * SK_ROWS * p.ms;
+}
+
+// G (nx x ny) = scale X Y^T with min(nx, ny) <= 8 (skinny_gram_ok); ws of skinny_gram_bytes
+cudaError_t launch_skinny_gram(const float *X, int nx, const float *Y, int ny, long long K, double scale, double *G,
+                               void *ws, cudaStream_t st) {
+  const bool ysmall = ny <= nx;
+  const float *L = ysmall ? X : Y, *S = ysmall ? Y : X;
+  const int nl = ysmall ? nx : ny, ns = ysmall ? ny : nx;
+  const SkinnyPlan p = skinny_gram_plan(nl, ns, K);
+  double *partial = static_cast<double *>(ws);
+  const long long tasks = (long long)p.groups * p.runs;
+  const unsigned grid = (unsigned)((tasks + SK_NT / 32 - 1) / (SK_NT / 32));
+  auto run = [&](auto kernel) {
+    kernel<<<grid, SK_NT, 0, st>>>(L, nl, S, ns, K, p.run, p.groups, p.runs, partial);
+  };
+  if (p.ms == 1) run(skinny_gram_kernel<1>);
+  else if (p.ms == 2) run(skinny_gram_kernel<2>);
+  else if (p.ms == 4) run(skinny_gram_kernel<4>);
+  else run(skinny_gram_kernel<8>);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const int nv = p.groups * SK_ROWS * p.ms;
+  skinny_gram_reduce_kernel<<<(nv + 31) / 32, 32 * SKR_SLICES, 0, st>>>(partial, p.runs, p.groups, p.ms, nl, ns,
+                                                            ysmall ? ny : 1, ysmall ? 1 : ny, scale, G);
+  return cudaGetLastError();
+}
+
+// Z (m x K) = A (m x n) Y (n x K) for m <= M: a thread holds the m sums of V neighbouring points
+// and reads Y once, eight rows in flight; A passes through shared memory 256 columns at a time.
+template <int M, int V>
+__global__ void __launch_bounds__(SK_NT) skinny_left_mul_kernel(const float *__restrict__ A, int m, int n,
+                                                                const float *__restrict__ Y, long long K,
+                                                                float *__restrict__ Z) {
+  constexpr int COLS = 256, RB = 8;
+  __shared__ __align__(16) float as[COLS][M];
+  const long long k = ((long long)blockIdx.x * SK_NT + threadIdx.x) * V;
+  float acc[M][V];
+  auto load = [](const float *src, float (&yv)[V]) {
+    if constexpr (V == 4) {
+      const float4 t = __ldg(reinterpret_cast<const float4 *>(src));
+      yv[0] = t.x, yv[1] = t.y, yv[2] = t.z, yv[3] = t.w;
+    } else {
+      yv[0] = __ldg(src);
+    }
+  };
+  auto add = [&](int l, const float (&yv)[V]) {
+#pragma unroll
+    for (int r = 0; r < M; ++r)
+#pragma unroll
+      for (int v = 0; v < V; ++v) acc[r][v] = fmaf(as[l][r], yv[v], acc[r][v]);
+  };
+#pragma unroll
+  for (int r = 0; r < M; ++r)
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[r][v] = 0.f;
+  for (int l0 = 0; l0 < n; l0 += COLS) {
+    const int nl = min(COLS, n - l0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < nl * M; e += SK_NT) {
+      const int r = e / nl, c = e % nl;
+      as[c][r] = r < m ? A[(long long)r * n + l0 + c] : 0.f;
+    }
+    __syncthreads();
+    if (k < K) {
+      const float *y = Y + (long long)l0 * K + k;
+      int l = 0;
+      for (; l + RB <= nl; l += RB) {
+        float yv[RB][V];
+#pragma unroll
+        for (int b = 0; b < RB; ++b) load(y + (long long)(l + b) * K, yv[b]);
+#pragma unroll
+        for (int b = 0; b < RB; ++b) add(l + b, yv[b]);
+      }
+      for (; l < nl; ++l) {
+        float yv[V];
+        load(y + (long long)l * K, yv);
+        add(l, yv);
+      }
+    }
+  }
+  if (k >= K) return;
+#pragma unroll
+  for (int r = 0; r < M; ++r) {
+    if (r >= m) break;
+    if constexpr (V == 4)
+      *reinterpret_cast<float4 *>(Z + (long long)r * K + k) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+    else
+      Z[(long long)r * K + k] = acc[r][0];
+  }
+}
+
+// Left multiply with m <= 8 rows of A.  Four points per thread where that still gives every SM
+// 512 threads and the rows lie on 16-byte boundaries; else one point per thread.
+cudaError_t launch_skinny_left_mul(const float *A, int m, int n, const float *Y, long long K, float *Z,
+                                   cudaStream_t st) {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const bool wide = K % 4 == 0 && K / 4 >= 512LL * sms &&
+                    ((reinterpret_cast<uintptr_t>(Y) | reinterpret_cast<uintptr_t>(Z)) & 15) == 0;
+  const long long threads = wide ? K / 4 : K;
+  const unsigned grid = (unsigned)((threads + SK_NT - 1) / SK_NT);
+  auto run = [&](auto kernel) { kernel<<<grid, SK_NT, 0, st>>>(A, m, n, Y, K, Z); };
+  if (m <= 1) wide ? run(skinny_left_mul_kernel<1, 4>) : run(skinny_left_mul_kernel<1, 1>);
+  else if (m <= 2) wide ? run(skinny_left_mul_kernel<2, 4>) : run(skinny_left_mul_kernel<2, 1>);
+  else if (m <= 4) wide ? run(skinny_left_mul_kernel<4, 4>) : run(skinny_left_mul_kernel<4, 1>);
+  else wide ? run(skinny_left_mul_kernel<8, 4>) : run(skinny_left_mul_kernel<8, 1>);
+  return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------------------
 // Left multiply Z (m x K) = A (m x n) * Y (n x K); 64 x 64 tile, k-step 16, 4 x 4 per thread.
 // ----------------------------------------------------------------------------------------
 constexpr int LM_BM = 64, LM_BN = 64, LM_BK = 16, LM_NT = 256;
