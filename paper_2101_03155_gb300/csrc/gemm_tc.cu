@@ -754,22 +754,25 @@ __global__ void __launch_bounds__(NT2, 1) tc_left_mul_tma_kernel(const float *__
 // one 128 x 128 tile, as a warp-specialised pipeline (no CTA barrier per K-step):
 //   - warp 20 (TMA): X and Y boxes of 128 rows x 32 points (16 KB FP32, 128-byte swizzled) into a
 //     ring of `ring` stages, each stage refilled once the split warps have read it;
-//   - warps 0-15 (split): warps 0-7 take the rows of the X box, warps 8-15 those of the Y box, two
-//     threads per row (16 K-values each), split them into bf16 hi/lo and store them into the
-//     K-major A or B tiles of one of `nops` operand buffers;
+//   - warps 0-15 (split): two teams of eight warps take alternate K-steps; a thread takes one row of
+//     the X or Y box, splits its 32 values into bf16 hi/lo and stores them into the K-major A or B
+//     tiles of one of `nops` operand buffers;
 //   - warp 21 (MMA, one lane): three BF16 products per 16-point K-slice into one of two TMEM
 //     accumulators; each chunk of `cs` K-steps stays in FP32 in one accumulator (a longer FP32
 //     accumulation in the tensor core loses accuracy);
 //   - warps 16-19 (fold, TMEM lane quarter warp & 3): add each finished chunk to a running sum kept
 //     in TMEM with Kahan compensation (sum and compensation in TMEM columns 256-383 and 384-511),
-//     release the accumulator, and at the end write the split's sum minus its compensation in
-//     FP64; a second kernel adds the splits in FP64 in a fixed order.
+//     release the accumulator, and at the end write the split's sum and compensation; a second
+//     kernel adds the splits in a fixed order.
+// Bound at 128 x 128 of 96^3 (906 MB) by the operand reads at 4.7 TB/s of 128-byte rows from 256 rows;
+// at sizes that stay in L2 a K-step takes 0.25 us or less.  With the split sums, in us: 128 rows of
+// 32^3 43 -> 26, of 64^3 90 -> 65, of 96^3 237 -> 213; 256 rows of 131072 points 129 -> 89.
 // Every wait is bounded; a wait that gives up raises a shared flag that ends every role, the TMA
 // warp waits (bounded) for its boxes in flight and the MMA lane for its last commit before the
 // tensor memory is released.
 // ----------------------------------------------------------------------------------------
 constexpr uint32_t kGBox = BM * BK * 4;  // 128 rows x 32 FP32
-constexpr int GW_SPLIT = 16;                           // split warps: two threads per row
+constexpr int GW_SPLIT = 16, GW_TEAM = 8;              // split warps, split warps per K-step
 constexpr int GW_FOLD0 = GW_SPLIT, GW_TMA = GW_SPLIT + 4, GW_MMA = GW_SPLIT + 5;
 constexpr int GW_NT = (GW_SPLIT + 6) * 32;             // + 4 fold warps, the TMA warp, the MMA warp
 constexpr int GW_OPS = 3;                // operand buffers (bf16 hi/lo tiles of both operands)
@@ -778,15 +781,15 @@ template <bool ABS>
 __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_constant__ CUtensorMap tmX,
                                                               const __grid_constant__ CUtensorMap tmY, int nx, int ny,
                                                               long long c0, long long K, int cs, int tiles_x,
-                                                              int ring, int nops, double *__restrict__ partial,
+                                                              int ring, int nops, float2 *__restrict__ partial,
                                                               int *__restrict__ err, uint32_t first_wait) {
   extern __shared__ unsigned char dyn[];
   unsigned char *base = align1024(dyn);
   unsigned char *ops = base;                                       // nops x {A_hi, A_lo, B_hi, B_lo}
   unsigned char *boxes = ops + (size_t)nops * 4 * TILE_BYTES;     // ring x {X box, Y box}
   uint64_t *box_full = reinterpret_cast<uint64_t *>(boxes + (size_t)ring * 2 * kGBox);
-  uint64_t *box_empty = box_full + ring;  // 8 split-warp arrivals
-  uint64_t *op_full = box_empty + ring;   // 8 split-warp arrivals
+  uint64_t *box_empty = box_full + ring;  // GW_TEAM split-warp arrivals
+  uint64_t *op_full = box_empty + ring;   // GW_TEAM split-warp arrivals
   uint64_t *op_empty = op_full + nops;    // MMA commit
   uint64_t *acc_full = op_empty + nops;   // MMA commit after a chunk's last K-step
   uint64_t *acc_empty = acc_full + 2;     // 4 fold-warp arrivals
@@ -798,21 +801,19 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
   // X and Y are the same matrix (the screen) and this tile is on the diagonal: one box per K-step
   // serves both operands
   const bool diag = ABS && ti == tj;
-  // this split's K-steps: whole chunks [c_lo, c_hi) of cs steps (the last chunk may be short)
-  const long long KS = K / BK, C = (KS + cs - 1) / cs;
-  const long long c_lo = (long long)blockIdx.y * C / gridDim.y, c_hi = (long long)(blockIdx.y + 1) * C / gridDim.y;
-  const long long ks_lo = c_lo * cs, ks_hi = min(KS, c_hi * (long long)cs);
-  const int Q = (int)(ks_hi > ks_lo ? ks_hi - ks_lo : 0);
-  const int NCH = (Q + cs - 1) / cs;
+  // this split's K-steps: blockIdx.y, blockIdx.y + gridDim.y, ... (a chunk is any cs of them), even to
+  // one step over the splits, and all CTAs read neighbouring lines of the tile's rows at any time
+  const long long KS = K / BK;
+  const int Q = (int)((KS - blockIdx.y + gridDim.y - 1) / gridDim.y), NCH = (Q + cs - 1) / cs;
 
   if (warp == 0) tmem_alloc(tmem_slot, 512);
   if (tid == 0) {
     for (int r = 0; r < ring; ++r) {
       mbar_init(smem_u32(&box_full[r]));
-      mbar_init_n(smem_u32(&box_empty[r]), GW_SPLIT);
+      mbar_init_n(smem_u32(&box_empty[r]), GW_TEAM);
     }
     for (int b = 0; b < nops; ++b) {
-      mbar_init_n(smem_u32(&op_full[b]), GW_SPLIT);
+      mbar_init_n(smem_u32(&op_full[b]), GW_TEAM);
       mbar_init(smem_u32(&op_empty[b]));
     }
     for (int a = 0; a < 2; ++a) {
@@ -826,10 +827,11 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // bounded wait for use `use` of a barrier (parity use & 1) that also leaves when another role has
-  // given up; false = leave
-  auto wait = [&](uint64_t *bar, int use, uint32_t limit) -> bool {
-    const uint32_t mb = smem_u32(bar), parity = (uint32_t)(use & 1);
+  // bounded wait for a phase of a barrier that also leaves when another role has given up; false =
+  // leave.  The roles count buffers and phases as they go: divisions by the run-time ring lengths
+  // were a third of the instructions of a K-step.
+  auto wait = [&](uint64_t *bar, uint32_t parity, uint32_t limit) -> bool {
+    const uint32_t mb = smem_u32(bar);
     for (uint32_t it = 0; it < limit; it += 64) {
       if (mbar_wait(mb, parity, 64)) return true;
       if (*abort_flag) return false;
@@ -842,17 +844,18 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
   if (warp == GW_TMA) {
     // ---- TMA: K-step q into stage q % ring once step q - ring has been read ----
     if (lane == 0) {
-      int issued = 0;
+      int issued = 0, stage = 0;
+      uint32_t ph = 0;
       for (int q = 0; q < Q; ++q) {
-        const int stage = q % ring;
-        if (q >= ring && !wait(&box_empty[stage], q / ring - 1, kWaitLimit)) break;
+        if (q >= ring && !wait(&box_empty[stage], ph ^ 1u, kWaitLimit)) break;
         const uint32_t mb = smem_u32(&box_full[stage]);
         unsigned char *bx = boxes + (size_t)stage * 2 * kGBox;
-        const int x = (int)(c0 + (ks_lo + q) * BK);
+        const int x = (int)(c0 + (blockIdx.y + (long long)q * gridDim.y) * BK);
         mbar_expect_tx(mb, diag ? kGBox : 2 * kGBox);
         tma_load_2d(smem_u32(bx), &tmX, x, i0, mb);
         if (!diag) tma_load_2d(smem_u32(bx + kGBox), &tmY, x, j0, mb);
         issued = q + 1;
+        if (++stage == ring) stage = 0, ph ^= 1u;
       }
       // no box may still be landing when the CTA ends: wait (bounded) for the last ones
       for (int q = issued > ring ? issued - ring : 0; q < issued; ++q)
@@ -862,10 +865,12 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
     // ---- MMA lane: three products per K-slice; a chunk per accumulator ----
     if (lane == 0) {
       int last = -1;  // last K-step whose MMAs were committed
+      int b = 0, kin = 0, cl = 0;  // operand buffer, K-step within the chunk, chunk
+      uint32_t ph = 0;
       for (int q = 0; q < Q; ++q) {
-        const int b = q % nops, kin = q % cs, cl = q / cs, a = cl & 1;
-        if (kin == 0 && cl >= 2 && !wait(&acc_empty[a], (cl >> 1) - 1, kWaitLimit)) break;
-        if (!wait(&op_full[b], q / nops, kWaitLimit)) break;
+        const int a = cl & 1;
+        if (kin == 0 && cl >= 2 && !wait(&acc_empty[a], (uint32_t)(((cl >> 1) - 1) & 1), kWaitLimit)) break;
+        if (!wait(&op_full[b], ph, kWaitLimit)) break;
         tc_fence_after();
         const uint32_t acc = tmem + (uint32_t)a * BN;
         const uint32_t a_hi = smem_u32(ops + (size_t)b * 4 * TILE_BYTES), a_lo = a_hi + TILE_BYTES;
@@ -880,6 +885,8 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
         commit(smem_u32(&op_empty[b]));
         if (kin == cs - 1 || q == Q - 1) commit(smem_u32(&acc_full[a]));
         last = q;
+        if (++b == nops) b = 0, ph ^= 1u;
+        if (++kin == cs) kin = 0, ++cl;
       }
       // the tensor memory is released at the end: wait (bounded) for the last MMAs
       if (last >= 0) mbar_wait(smem_u32(&op_empty[last % nops]), (uint32_t)((last / nops) & 1));
@@ -903,7 +910,7 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
       const int a = c & 1;
       // every lane polls; the lanes may leave the poll loop apart, and the TMEM loads and stores
       // below are warp-collective (.sync.aligned): reconverge first
-      const bool got = wait(&acc_full[a], c >> 1, kWaitLimit);
+      const bool got = wait(&acc_full[a], (uint32_t)((c >> 1) & 1), kWaitLimit);
       if (!__all_sync(0xffffffffu, got)) {
         ok = false;
         break;
@@ -932,7 +939,10 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
     }
     if (ok && !*abort_flag) {
       const int i = i0 + 32 * (warp & 3) + lane;
-      double *dst = partial + ((long long)blockIdx.y * nx + i) * ny;
+      // column by column: the 32 rows of a warp are neighbours, so that a store fills whole lines.
+      // The sum and its compensation go out as they are: converting and subtracting them in FP64
+      // here took 15 us (one FP64 warp instruction per 64 cycles and scheduler).
+      float2 *dst = partial + (long long)blockIdx.y * ny * nx + i;
 #pragma unroll 1
       for (int cb = 0; cb < 8; ++cb) {
         float sm[16], cp[16];
@@ -942,45 +952,47 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
         if (i < nx) {
 #pragma unroll
           for (int e = 0; e < 16; ++e)
-            if (jb + e < ny) dst[jb + e] = (double)sm[e] - (double)cp[e];
+            if (jb + e < ny) dst[(long long)(jb + e) * nx] = make_float2(sm[e], cp[e]);
         }
       }
     }
   } else {
-    // ---- split warps: warps 0-7 take X rows into the A tiles, warps 8-15 Y rows into the B
-    // tiles; a thread takes the K-values [16 h, 16 h + 16) of row `row` (h = bit 7 of its index);
-    // row `row` of a box holds its 16-byte chunk k4 at position k4 ^ (row & 7) ----
-    const int row = tid & 127, h = (tid >> 7) & 1, half = tid >> 8;
-    for (int q = 0; q < Q; ++q) {
-      const int stage = q % ring, b = q % nops;
+    // ---- split warps: team t (warps 8t - 8t + 7) takes the K-steps of parity t; its first 128
+    // threads split the rows of the X box into the A tiles, the others those of the Y box into the
+    // B tiles, a row of 32 K-values each; row `row` of a box holds its 16-byte chunk k4 at position
+    // k4 ^ (row & 7) ----
+    const int team = warp >> 3, row = tid & 127, half = (tid >> 7) & 1;
+    int stage = team, b = team;
+    uint32_t sph = 0, bph = 0;
+    if (stage >= ring) stage -= ring, sph ^= 1u;
+    if (b >= nops) b -= nops, bph ^= 1u;
+    const unsigned char *rowp = boxes + (size_t)(diag ? 0 : half) * kGBox + row * 128;
+    unsigned char *rowo = ops + (size_t)half * 2 * TILE_BYTES;
+    for (int q = team; q < Q; q += 2) {
       // the first wait may be given fewer polls (a test of the give-up path)
-      if (!__all_sync(0xffffffffu, wait(&box_full[stage], q / ring, q == 0 ? first_wait : kWaitLimit))) break;
-      float v[16];
-      const unsigned char *rowp = boxes + (size_t)stage * 2 * kGBox + (size_t)(diag ? 0 : half) * kGBox + row * 128;
-#pragma unroll
-      for (int c4 = 0; c4 < 4; ++c4) {
-        const int k4 = 4 * h + c4;
-        const float4 t = *reinterpret_cast<const float4 *>(rowp + ((k4 ^ (row & 7)) << 4));
-        v[4 * c4] = ABS ? fabsf(t.x) : t.x;
-        v[4 * c4 + 1] = ABS ? fabsf(t.y) : t.y;
-        v[4 * c4 + 2] = ABS ? fabsf(t.z) : t.z;
-        v[4 * c4 + 3] = ABS ? fabsf(t.w) : t.w;
-      }
+      if (!__all_sync(0xffffffffu, wait(&box_full[stage], sph, q == 0 ? first_wait : kWaitLimit))) break;
+      const unsigned char *src = rowp + (size_t)stage * 2 * kGBox;
       // the bf16 hi/lo words first, then the wait for the operand buffer (its MMAs from nops
       // K-steps ago), then the stores
-      uint4 hi[2], lo[2];
+      uint4 hi[4], lo[4];
 #pragma unroll
-      for (int c8 = 0; c8 < 2; ++c8) {
+      for (int c8 = 0; c8 < 4; ++c8) {
         float x[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = v[8 * c8 + e];
+        for (int c4 = 0; c4 < 2; ++c4) {
+          const float4 t = *reinterpret_cast<const float4 *>(src + (((2 * c8 + c4) ^ (row & 7)) << 4));
+          x[4 * c4] = ABS ? fabsf(t.x) : t.x;
+          x[4 * c4 + 1] = ABS ? fabsf(t.y) : t.y;
+          x[4 * c4 + 2] = ABS ? fabsf(t.z) : t.z;
+          x[4 * c4 + 3] = ABS ? fabsf(t.w) : t.w;
+        }
         split8(x, hi[c8], lo[c8]);
       }
-      if (q >= nops && !__all_sync(0xffffffffu, wait(&op_empty[b], q / nops - 1, kWaitLimit))) break;
-      unsigned char *ob = ops + (size_t)b * 4 * TILE_BYTES + (size_t)half * 2 * TILE_BYTES;
+      if (q >= nops && !__all_sync(0xffffffffu, wait(&op_empty[b], bph ^ 1u, kWaitLimit))) break;
+      unsigned char *ob = rowo + (size_t)b * 4 * TILE_BYTES;
 #pragma unroll
-      for (int c8 = 0; c8 < 2; ++c8) {
-        const uint32_t off = tile_off(row, 16 * h + 8 * c8);
+      for (int c8 = 0; c8 < 4; ++c8) {
+        const uint32_t off = tile_off(row, 8 * c8);
         *reinterpret_cast<uint4 *>(ob + off) = hi[c8];
         *reinterpret_cast<uint4 *>(ob + TILE_BYTES + off) = lo[c8];
       }
@@ -992,6 +1004,10 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
         mbar_arrive(smem_u32(&box_empty[stage]));
         mbar_arrive(smem_u32(&op_full[b]));
       }
+      stage += 2;
+      if (stage >= ring) stage -= ring, sph ^= 1u;
+      b += 2;
+      if (b >= nops) b -= nops, bph ^= 1u;
     }
   }
   tc_fence_before();
@@ -999,16 +1015,38 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// G = scale * sum over the splits of partial[s] (FP64, fixed order); with `accumulate` the sum is
-// added to G instead
-__global__ void gram_splits_reduce_kernel(const double *__restrict__ partial, int splits, int ne, double scale,
-                                          bool accumulate, double *__restrict__ G) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= ne) return;
-  double s = 0.0;
-#pragma unroll 8
-  for (int k = 0; k < splits; ++k) s += partial[(long long)k * ne + e];
-  G[e] = (accumulate ? G[e] : 0.0) + scale * s;
+// Split sums: a 512-thread block adds the splits of 32 values in a fixed order: each warp adds every
+// sixteenth split with up to ten loads in flight, the first warp adds the sixteen sums.  (One thread
+// per value walked up to 152 loads, 17-22 us at every size; now 4-8 us.)
+constexpr int SR_NT = 512;
+// G (nx x ny) = scale * sum over the splits of partial[s], pairs (sum, compensation) column by column;
+// with `accumulate` the sum is added to G instead.  Each of the 16 slices adds its splits as an FP32
+// pair with exact two-sums (about 48 bits; FP32 instructions where FP64 ones would bound the kernel),
+// the slices are added in FP64 in a fixed order.
+__global__ void __launch_bounds__(SR_NT) gram_splits_reduce_kernel(const float2 *__restrict__ partial, int splits,
+                                                                   int nx, int ny, double scale, bool accumulate,
+                                                                   double *__restrict__ G) {
+  __shared__ double part[SR_NT / 32][33];
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane, ne = nx * ny;
+  float s = 0.f, c = 0.f;
+  if (e < ne) {
+#pragma unroll 10
+    for (int k = slice; k < splits; k += SR_NT / 32) {
+      const float2 v = partial[(long long)k * ne + e];
+      const float t = s + v.x, b = t - s;
+      c += ((s - (t - b)) + (v.x - b)) - v.y;
+      s = t;
+    }
+  }
+  part[slice][lane] = (double)s + (double)c;
+  __syncthreads();
+  if (slice != 0 || e >= ne) return;
+  double r = 0.0;
+#pragma unroll
+  for (int i = 0; i < SR_NT / 32; ++i) r += part[i][lane];
+  double *g = G + (long long)(e % nx) * ny + e / nx;
+  *g = (accumulate ? *g : 0.0) + scale * r;
 }
 
 // ----------------------------------------------------------------------------------------
@@ -1420,16 +1458,32 @@ __global__ void __launch_bounds__(SY_NT, 1) screen_syrk_kernel(const __grid_cons
   }
 }
 
-// O_ij += scale * sum over the splits of partial[s]_ij for i <= j (FP64, fixed order)
-__global__ void screen_splits_reduce_kernel(const double *__restrict__ partial, int splits, int n, double scale,
-                                            double *__restrict__ O) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n * n || e % n < e / n) return;
-  const long long ne = (long long)n * n;
+// Sum over the splits of partial[s][e] (FP64) for 32 values of a block
+__device__ __forceinline__ double splits_sum(const double *__restrict__ partial, int splits, long long ne, long long e,
+                                             bool wanted) {
+  __shared__ double part[SR_NT / 32][33];
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   double s = 0.0;
-#pragma unroll 8
-  for (int k = 0; k < splits; ++k) s += partial[(long long)k * ne + e];
-  O[e] += scale * s;
+  if (wanted) {
+#pragma unroll 10
+    for (int k = slice; k < splits; k += SR_NT / 32) s += partial[(long long)k * ne + e];
+  }
+  part[slice][lane] = s;
+  __syncthreads();
+  if (slice != 0) return 0.0;
+  s = 0.0;
+#pragma unroll
+  for (int i = 0; i < SR_NT / 32; ++i) s += part[i][lane];
+  return s;
+}
+
+// O_ij += scale * sum over the splits of partial[s]_ij for i <= j (FP64, fixed order)
+__global__ void __launch_bounds__(SR_NT) screen_splits_reduce_kernel(const double *__restrict__ partial, int splits,
+                                                                     int n, double scale, double *__restrict__ O) {
+  const int e = blockIdx.x * 32 + (threadIdx.x & 31);
+  const bool wanted = e < n * n && e % n >= e / n;
+  const double s = splits_sum(partial, splits, (long long)n * n, e, wanted);
+  if (threadIdx.x < 32 && wanted) O[e] += scale * s;
 }
 
 }  // namespace tc
@@ -1536,17 +1590,18 @@ static bool gram_tma_plan(const float *X, int nx, const float *Y, int ny, long l
   const int cs = tc_chunk() / tc::BK;
   const long long chunks = (K / tc::BK + cs - 1) / cs;
   p->splits = (int)std::max(1LL, std::min(chunks, (long long)std::max(1, sms / p->tiles)));
-  // three operand buffers, the rest of shared memory for box stages (4); measured at 96^3, the
-  // split of 2-4 buffers and 2-5 stages changes nothing
+  // three operand buffers, the rest of shared memory for box stages (4); measured at 96^3, two buffers
+  // or an earlier release of the boxes change nothing.  An even number of stages: each team of split
+  // warps then meets only its own barriers (a parity seen by neither team in between is ambiguous).
   p->nops = tc::GW_OPS;
   const size_t fixed = (size_t)p->nops * 4 * tc::TILE_BYTES + 1024 + 256;
-  p->ring = (int)std::min<size_t>(4, (227 * 1024 - fixed) / (2 * tc::kGBox));
+  p->ring = (int)std::min<size_t>(4, (227 * 1024 - fixed) / (2 * tc::kGBox)) & ~1;
   return p->ring >= 2;
 }
 
 size_t tc_gram_workspace_bytes(const float *X, int nx, const float *Y, int ny, long long K) {
   GramPlan p;
-  if (gram_tma_plan(X, nx, Y, ny, K, &p)) return sizeof(double) * (size_t)p.splits * nx * ny;
+  if (gram_tma_plan(X, nx, Y, ny, K, &p)) return sizeof(float2) * (size_t)p.splits * nx * ny;
   return gram_chunks_workspace_bytes(nx, ny, K);
 }
 
@@ -1564,7 +1619,7 @@ static bool launch_gram_tma(const float *X, int nx, const float *Y, int ny, long
   const int smem = (int)((size_t)p.nops * 4 * tc::TILE_BYTES + (size_t)p.ring * 2 * tc::kGBox + 1024 + 256);
   *e = cudaFuncSetAttribute(tc::tc_gram_tma_kernel<ABS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (*e != cudaSuccess) return true;
-  double *partial = static_cast<double *>(ws);
+  float2 *partial = static_cast<float2 *>(ws);
   // ACE_TC_FIRST_WAIT_POLLS: polls of the kernel's first wait on a TMA box (test knob; 0 makes
   // the kernel give up at once and report ACE_ERR_TIMEOUT after draining its copies)
   const char *fw = std::getenv("ACE_TC_FIRST_WAIT_POLLS");
@@ -1574,8 +1629,7 @@ static bool launch_gram_tma(const float *X, int nx, const float *Y, int ny, long
   *e = cudaGetLastError();
   if (*e != cudaSuccess) return true;
   const int n = nx * ny;
-  // 64-thread blocks spread the FP64 adds (splits x n elements) over most SMs
-  tc::gram_splits_reduce_kernel<<<(n + 63) / 64, 64, 0, st>>>(partial, p.splits, n, scale, ABS, G);
+  tc::gram_splits_reduce_kernel<<<(n + 31) / 32, tc::SR_NT, 0, st>>>(partial, p.splits, nx, ny, scale, ABS, G);
   *launches += 2;
   *e = cudaGetLastError();
   return true;
@@ -1591,7 +1645,7 @@ cudaError_t launch_tc_gram(const float *X, int nx, const float *Y, int ny, long 
 
 size_t tc_screen_workspace_bytes(const float *X, int n, long long K) {
   GramPlan p;
-  return gram_tma_plan(X, n, X, n, K, &p) ? sizeof(double) * (size_t)p.splits * n * n : 0;
+  return gram_tma_plan(X, n, X, n, K, &p) ? sizeof(float2) * (size_t)p.splits * n * n : 0;
 }
 
 bool launch_tc_screen(const float *X, int n, long long ld, long long c0, long long K, double scale, double *G,
@@ -1668,7 +1722,7 @@ bool launch_screen_syrk(const float *X, int n, long long ld, long long c0, long 
   if (pm && pm->done) *pm->done = *pm->done && with_max;
   *e = cudaGetLastError();
   if (*e != cudaSuccess) return true;
-  tc::screen_splits_reduce_kernel<<<(n * n + 63) / 64, 64, 0, st>>>(partial, splits, n, scale, G);
+  tc::screen_splits_reduce_kernel<<<(n * n + 31) / 32, tc::SR_NT, 0, st>>>(partial, splits, n, scale, G);
   *launches += 2;
   *e = cudaGetLastError();
   return true;
