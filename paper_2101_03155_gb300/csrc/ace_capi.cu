@@ -282,6 +282,8 @@ struct ace_op {
   float *pmax = nullptr;      // plane maxima of the working orbitals [n][N1] for the plane skip
   float *gmax = nullptr;      // and the orbitals' maxima [n]
   bool queued = false;        // screened build whose chain ran in a device pack queue
+  char *small = nullptr;      // rest of the block that small buffers are cut from (op_alloc)
+  size_t small_left = 0;
   bool graph = false;         // recorded into a CUDA graph: no host waits, no timing events,
                               // uploads from pinned buffers that live as long as the handle
   std::vector<std::pair<void *, size_t>> staged;  // those pinned upload buffers
@@ -289,17 +291,38 @@ struct ace_op {
 
 namespace {
 
+// Size of a buffer within a handle's small block.
+constexpr size_t small_size(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
 // Buffers the handle owns (results and pair lists).  A handle recorded into a graph takes them
 // from cudaMalloc, outside the graph, so that they keep their addresses over every launch.
+// Buffers that fit into what is left of the handle's small block are cut from it.
 template <typename P>
 cudaError_t op_alloc(ace_op *op, P **p, size_t bytes) {
   void *v = nullptr;
+  if (small_size(bytes) <= op->small_left) {
+    *p = reinterpret_cast<P *>(op->small);
+    op->small += small_size(bytes);
+    op->small_left -= small_size(bytes);
+    return cudaSuccess;
+  }
   cudaError_t e = op->graph ? cudaMalloc(&v, bytes > 0 ? bytes : 16)
                             : cudaMallocAsync(&v, bytes > 0 ? bytes : 16, op->stream);
   if (e != cudaSuccess) return e;
   op->owned.push_back(v);
   *p = static_cast<P *>(v);
   return cudaSuccess;
+}
+
+// One allocation for the handle's n x n matrices, pair list, counters and plane maxima: each
+// cudaMallocAsync and cudaFreeAsync costs the host 1-2 us, and at 16 orbitals of 32^3 the host's share
+// of a build (270 us, 156 of them on the device) was the larger part of what could be saved.
+cudaError_t op_reserve(ace_op *op, size_t bytes) {
+  char *v = nullptr;
+  op->small_left = 0;
+  const cudaError_t e = op_alloc(op, &v, bytes);
+  if (e == cudaSuccess) op->small = v, op->small_left = bytes;
+  return e;
 }
 
 void op_free_all(ace_op *op) {
@@ -1128,6 +1151,12 @@ ace_status build_begin(ace_op *op, const void *phi_in, ace_dtype dtype) {
 
   // ---- screen (section II): O_ij = dV sum |phi_i phi_j|, pair list ----
   const size_t maxpairs = (size_t)n * (n + 1) / 2;
+  // O, O_sym, M_raw, M, L, L^-1; L^-1 in FP32; pairs, packs; count, status, energy; plane maxima
+  ACE_CUDA(op_reserve(op, 6 * small_size(sizeof(double) * n * n) + small_size(sizeof(float) * n * n) +
+                              small_size(sizeof(int2) * (maxpairs + 2)) + small_size(sizeof(int4) * (maxpairs / 2 + 2)) +
+                              3 * small_size(16) + small_size(sizeof(float) * (size_t)n * d.n[0]) +
+                              small_size(sizeof(float) * (size_t)n)),
+           "alloc small buffers");
   ACE_CUDA(op_alloc(op, &op->O, sizeof(double) * n * n), "alloc O");
   ACE_CUDA(op_alloc(op, &op->O_sym, sizeof(double) * n * n), "alloc O_sym");
   ACE_CUDA(op_alloc(op, &op->pairs, sizeof(int2) * (maxpairs + 2)), "alloc pairs");
@@ -1366,8 +1395,7 @@ ace_status factor_and_project(ace_op *op, const T *W) {
   if (sizeof(T) == 8) {
     Linv_T = reinterpret_cast<const T *>(op->Linv);
   } else {
-    ACE_CUDA(cudaMallocAsync(&tmp, sizeof(T) * n * n, st), "alloc Linv32");
-    temps.push_back(tmp);
+    ACE_CUDA(op_alloc(op, &tmp, sizeof(T) * n * n), "alloc Linv32");
     ACE_CUDA((ace::launch_convert<double, T>(op->Linv, static_cast<T *>(tmp), (long long)n * n, 1.0, st)), "Linv32");
     ++op->launches;
     Linv_T = static_cast<const T *>(tmp);
@@ -1580,11 +1608,13 @@ ace_status apply_coeffs_impl(const ace_op *op, const void *psi_in, ace_dtype dty
 // out = -xi C (m rows of op->N points, any side) from C (n x m FP64, device)
 template <typename T>
 ace_status apply_finish_impl(const ace_op *op, const double *C, ace_dtype dtype, int m, void *out, int *err_d,
-                             cudaStream_t st, std::vector<void *> &temps) {
-  void *tmp = nullptr;
-  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(T) * op->n * m, st), "alloc A");
-  temps.push_back(tmp);
-  T *A = static_cast<T *>(tmp);
+                             cudaStream_t st, std::vector<void *> &temps, T *A = nullptr) {
+  if (!A) {
+    void *tmp = nullptr;
+    ACE_CUDA(cudaMallocAsync(&tmp, sizeof(T) * op->n * m, st), "alloc A");
+    temps.push_back(tmp);
+    A = static_cast<T *>(tmp);
+  }
   ACE_CUDA(ace::launch_transpose_scale<T>(C, op->n, m, -1.0, A, st), "transpose");
   T *res = nullptr;
   ace_status s = result_target<T>(out, dtype, (long long)m * op->N, st, temps, &res);
@@ -1618,17 +1648,17 @@ ace_status apply_impl(const ace_op *op, const void *psi_in, ace_dtype dtype, int
   std::vector<void *> temps;
   TempGuard guard{&temps, st};
   void *tmp = nullptr;
-  // C = dV xi psi^T  (n x m, FP64 across chunks)
-  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(double) * n * m, st), "alloc C");
+  // one buffer for C = dV xi psi^T (n x m, FP64 across chunks), its transpose in T and the flag
+  const size_t cb = small_size(sizeof(double) * n * m), ab = small_size(sizeof(T) * n * m);
+  ACE_CUDA(cudaMallocAsync(&tmp, cb + ab + sizeof(int), st), "alloc C");
   temps.push_back(tmp);
   double *C = static_cast<double *>(tmp);
-  ACE_CUDA(cudaMallocAsync(&tmp, sizeof(int), st), "alloc flag");
-  temps.push_back(tmp);
-  int *err_d = static_cast<int *>(tmp);
+  T *A = reinterpret_cast<T *>(static_cast<char *>(tmp) + cb);
+  int *err_d = reinterpret_cast<int *>(static_cast<char *>(tmp) + cb + ab);
   ACE_CUDA(cudaMemsetAsync(err_d, 0, sizeof(int), st), "zero flag");
   ace_status s = apply_coeffs_impl<T>(op, psi_in, dtype, m, C, err_d, st, temps);
   if (s != ACE_OK) return s;
-  s = apply_finish_impl<T>(op, C, dtype, m, out, err_d, st, temps);
+  s = apply_finish_impl<T>(op, C, dtype, m, out, err_d, st, temps, A);
   if (s != ACE_OK) return s;
   return finish_flag(err_d, st, "apply");
 }
