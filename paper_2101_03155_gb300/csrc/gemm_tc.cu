@@ -558,60 +558,93 @@ __global__ void __launch_bounds__(NT) tc_left_mul_kernel(const float *__restrict
 }
 
 // ----------------------------------------------------------------------------------------
-// Left multiply fed by TMA: Z[i][c] = sum_l A[i][l] Y[l][c] for rows [i0, i0 + 128) of A.
-//   - A rows: split into bf16 hi/lo once per CTA, resident in shared memory (n/32 K-steps).
-//   - Y: boxes of 32 rows x 128 columns (16 KB FP32) arrive by TMA in a ring of `ring` stages,
-//     issued `ring` items ahead by thread 0; an item is one (column tile, K-step).
-//   - Each thread splits column `tid` of a box into the K-major B tile (two B buffers, so that
-//     the split of item q overlaps the MMAs of item q - 1).
-//   - Two TMEM accumulators: tile j accumulates in accumulator j & 1 while the epilogue of
-//     tile j - 1 reads the other one.
-// Every wait is bounded; after a timeout the kernel waits (bounded) for its copies and MMAs in
-// flight, releases TMEM and reports through *err.
+// Left multiply fed by TMA: Z[i][c] = sum_l A[i][l] Y[l][c] for rows [i0, i0 + 128) of A, as a
+// warp-specialised pipeline over items (column tile, 32-row K-step), no CTA barrier per item:
+//   - A rows: split into bf16 hi/lo once per CTA, resident in shared memory (n/32 K-steps);
+//   - warp 12 (TMA): boxes of 32 rows x 128 columns of Y (16 KB FP32) into a ring of `ring` stages;
+//   - warps 0-7 (split): two teams of four warps take alternate items; a thread splits one column of
+//     the box (32 K-values) into bf16 hi/lo in one of `nops` K-major B buffers;
+//   - warp 13 (MMA, one lane): three BF16 products per 16-row K-slice; two TMEM accumulators, tile j
+//     in accumulator j & 1;
+//   - warps 8-11 (output, TMEM lane quarter warp & 3): 32 rows x 32 columns at a time through two
+//     staging boxes per warp and TMA stores, while the next tile accumulates.
+// Every wait is bounded; a wait that gives up raises a shared flag that ends every role; copies and
+// MMAs in flight are waited for (bounded), TMEM is released and *err is set.
+// Bound by reading Y and writing Z: 128 rows of 96^3 (906 MB) in 152 us, 5.9 TB/s; one loop of eight
+// warps with CTA barriers took 1.1 us per item from L2 as from memory, 209 us.  64 rows of 72^3
+// 62 -> 36 us; 256 rows of 128^3, where each box feeds two row blocks, 1610 -> 1375 us.
 // ----------------------------------------------------------------------------------------
-constexpr uint32_t kLmBox = BK * BN * 4;   // one Y box: 32 rows x 128 FP32 columns
-constexpr uint32_t kEpiBox = BM * 32 * 4;  // one Z box: 128 rows x 32 FP32 columns
+constexpr uint32_t kLmBox = BK * BN * 4;  // one Y box: 32 rows x 128 FP32 columns
+constexpr uint32_t kZBox = 32 * 32 * 4;   // one Z box: 32 rows x 32 FP32 columns
+constexpr int LW_TEAMS = 2, LW_TEAM = 4, LW_SPLIT = LW_TEAMS * LW_TEAM;
+constexpr int LW_OUT0 = LW_SPLIT, LW_TMA = LW_SPLIT + 4, LW_MMA = LW_SPLIT + 5;
+constexpr int LW_NT = (LW_SPLIT + 6) * 32;
 
-__global__ void __launch_bounds__(NT2, 1) tc_left_mul_tma_kernel(const float *__restrict__ A, int m, int n,
-                                                                const __grid_constant__ CUtensorMap tmY,
-                                                                const __grid_constant__ CUtensorMap tmZ, long long K,
-                                                                int ring, int *__restrict__ err) {
+__global__ void __launch_bounds__(LW_NT, 1) tc_left_mul_tma_kernel(const float *__restrict__ A, int m, int n,
+                                                                  const __grid_constant__ CUtensorMap tmY,
+                                                                  const __grid_constant__ CUtensorMap tmZ, long long K,
+                                                                  int ring, int nops, int *__restrict__ err) {
   extern __shared__ unsigned char dyn[];
   unsigned char *base = align1024(dyn);
   const int nsteps = (n + BK - 1) / BK;
-  unsigned char *a_tiles = base;                                    // nsteps x {hi, lo}
-  unsigned char *b_ops = a_tiles + (size_t)nsteps * 2 * TILE_BYTES;  // 2 buffers x {hi, lo}
-  unsigned char *epi = b_ops + 2 * 2 * TILE_BYTES;                  // 2 x 128 rows x 32 FP32 (swizzled)
-  unsigned char *boxes = epi + 2 * kEpiBox;                         // ring x kLmBox
-  uint64_t *full = reinterpret_cast<uint64_t *>(boxes + (size_t)ring * kLmBox);
-  uint64_t *mmad = full + ring;  // MMAs of the items that read B buffer b
-  uint64_t *accf = mmad + 2;     // every MMA of the tile in accumulator a
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(accf + 2);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int quarter = warp & 3, half = warp >> 2;  // TMEM lane quarter; K-half / column half
-  const int col = tid & 127;                       // row of the A tile / column of the Y box
+  unsigned char *a_tiles = base;                                     // nsteps x {hi, lo}
+  unsigned char *b_ops = a_tiles + (size_t)nsteps * 2 * TILE_BYTES;  // nops x {hi, lo}
+  unsigned char *zbox = b_ops + (size_t)nops * 2 * TILE_BYTES;       // output warp x 2 boxes (swizzled)
+  unsigned char *boxes = zbox + 8 * kZBox;                           // ring x kLmBox
+  uint64_t *box_full = reinterpret_cast<uint64_t *>(boxes + (size_t)ring * kLmBox);
+  uint64_t *box_empty = box_full + ring;  // LW_TEAM split-warp arrivals
+  uint64_t *op_full = box_empty + ring;   // LW_TEAM split-warp arrivals
+  uint64_t *op_empty = op_full + nops;    // MMA commit
+  uint64_t *acc_full = op_empty + nops;   // MMA commit after a tile's last K-step
+  uint64_t *acc_empty = acc_full + 2;     // 4 output-warp arrivals
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
+  volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int i0 = blockIdx.y * BM;
   // a last tile of fewer than BN columns reads zeros past column K (the map's bounds) and stores
   // only its columns below K
   const long long ntiles = (K + BN - 1) / BN;
-  const long long mytiles = ntiles > (long long)blockIdx.x ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-  const long long Q = mytiles * nsteps;
+  const int mytiles =
+      ntiles > (long long)blockIdx.x ? (int)((ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+  const int Q = mytiles * nsteps;
 
   if (warp == 0) tmem_alloc(tmem_slot, 256);
   if (tid == 0) {
-    for (int r = 0; r < ring; ++r) mbar_init(smem_u32(&full[r]));
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(smem_u32(&mmad[b]));
-      mbar_init(smem_u32(&accf[b]));
+    for (int r = 0; r < ring; ++r) {
+      mbar_init(smem_u32(&box_full[r]));
+      mbar_init_n(smem_u32(&box_empty[r]), LW_TEAM);
     }
+    for (int b = 0; b < nops; ++b) {
+      mbar_init_n(smem_u32(&op_full[b]), LW_TEAM);
+      mbar_init(smem_u32(&op_empty[b]));
+    }
+    for (int c = 0; c < 2; ++c) {
+      mbar_init(smem_u32(&acc_full[c]));
+      mbar_init_n(smem_u32(&acc_empty[c]), 4);
+    }
+    *abort_flag = 0;
     mbar_init_fence();
   }
+  tc_fence_before();
   __syncthreads();
-  // items are numbered q = tile_slot * nsteps + kstep; the producer walks them with counters
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  // bounded wait for a phase of a barrier that also leaves when another role has given up
+  auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
+    const uint32_t mb = smem_u32(bar);
+    for (uint32_t it = 0; it < kWaitLimit; it += 64) {
+      if (mbar_wait(mb, parity, 64)) return true;
+      if (*abort_flag) return false;
+    }
+    *abort_flag = 1;
+    atomicExch(err, 1);
+    return false;
+  };
+  // items q = tile slot * nsteps + K-step
   int p_stage = 0, p_step = 0;
   long long p_tile = blockIdx.x;
-  auto issue_next = [&]() {  // thread 0: the next item into stage p_stage
-    const uint32_t mb = smem_u32(&full[p_stage]);
+  auto issue_next = [&]() {  // TMA lane: the next item into stage p_stage
+    const uint32_t mb = smem_u32(&box_full[p_stage]);
     mbar_expect_tx(mb, kLmBox);
     tma_load_2d(smem_u32(boxes + (size_t)p_stage * kLmBox), &tmY, (int)(p_tile * BN), p_step * BK, mb);
     if (++p_stage == ring) p_stage = 0;
@@ -620,130 +653,142 @@ __global__ void __launch_bounds__(NT2, 1) tc_left_mul_tma_kernel(const float *__
       p_tile += gridDim.x;
     }
   };
-  const int Qi = (int)Q;
-  int issued = Qi < ring ? Qi : ring;
-  if (tid == 0)
-    for (int k = 0; k < issued; ++k) issue_next();
-  // resident A: row i0 + col, K-values [16 half, 16 half + 16) of every K-step (overlaps the first copies)
-  for (int it = 0; it < nsteps; ++it) {
-    float v[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int k = it * BK + 16 * half + j;
-      v[j] = (i0 + col < m && k < n) ? __ldg(A + (long long)(i0 + col) * n + k) : 0.f;
-    }
-    unsigned char *t = a_tiles + (size_t)it * 2 * TILE_BYTES;
-    store_half_row(v, col, half, t, t + TILE_BYTES);
-  }
-  fence_async_smem();
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  Pipe pipe;
-  pipe.init();
-  bool ok = true;
-  int q = 0;
-  auto epilogue = [&](int j) -> bool {
-    const int a = j & 1;
-    const bool w = mbar_wait(smem_u32(&accf[a]), (uint32_t)((j >> 1) & 1));
-    if (__syncthreads_or(!w)) return false;
-    tc_fence_after();
-    const long long c0 = (blockIdx.x + (long long)j * gridDim.x) * BN;
-    const int row = 32 * quarter + (tid & 31);  // TMEM lane = row of the tile
-    // two rounds: warps 0-3 stage column block r in buffer 0, warps 4-7 block r + 2 in buffer 1
-#pragma unroll 1
-    for (int r = 0; r < 2; ++r) {
-      const int cb = r + 2 * half;
-      float v[32];
-      tmem_ld32(tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)a * BN + 32 * cb, v);
-      unsigned char *eb = epi + (size_t)half * kEpiBox;
-      if (tid == 0) bulk_wait_read<0>();  // both buffers have been read by the previous stores
-      __syncthreads();
-      // row `row`: 128 bytes, 16-byte chunk q at position q ^ (row & 7) (the map's 128-byte swizzle)
-#pragma unroll
-      for (int q = 0; q < 8; ++q)
-        *reinterpret_cast<float4 *>(eb + row * 128 + ((q ^ (row & 7)) << 4)) =
-            make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-      fence_async_smem();
-      __syncthreads();
-      if (tid == 0) {
-        if (c0 + 32 * r < K) tma_store_2d(&tmZ, (int)(c0 + 32 * r), i0, smem_u32(epi));
-        if (c0 + 32 * (r + 2) < K) tma_store_2d(&tmZ, (int)(c0 + 32 * (r + 2)), i0, smem_u32(epi + kEpiBox));
-        bulk_commit();
-      }
-    }
-    tc_fence_before();
-    __syncthreads();  // accumulator a is read before tile j + 2 writes it
-    return true;
-  };
-  int stage = 0, st = 0, j = 0;
-  uint32_t fpar = 0;  // parity of the current pass over the ring
-  for (; q < Qi; ++q) {
-    const int b = q & 1;
-    const bool got = mbar_wait(smem_u32(&full[stage]), fpar);
-    const bool freed = pipe.drain(mmad, b);
-    if (__syncthreads_or(!(got && freed))) {
-      ok = false;
-      break;
-    }
-    {
-      // column `col` of the box, rows [16 half, 16 half + 16)
+  const int first = Q < ring ? Q : ring;
+  if (warp == LW_TMA && lane == 0)
+    for (int q = 0; q < first; ++q) issue_next();
+  // resident A (overlaps the first copies): row i0 + row, K-values [16 half, 16 half + 16) of every step
+  if (tid < 256) {
+    const int row = tid & 127, half = tid >> 7;
+    for (int it = 0; it < nsteps; ++it) {
       float v[16];
-      const float *box = reinterpret_cast<const float *>(boxes + (size_t)stage * kLmBox);
 #pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = box[(16 * half + k) * BN + col];
-      unsigned char *bt = b_ops + (size_t)b * 2 * TILE_BYTES;
-      store_half_row(v, col, half, bt, bt + TILE_BYTES);
+      for (int j = 0; j < 16; ++j) {
+        const int k = it * BK + 16 * half + j;
+        v[j] = (i0 + row < m && k < n) ? __ldg(A + (long long)(i0 + row) * n + k) : 0.f;
+      }
+      unsigned char *t = a_tiles + (size_t)it * 2 * TILE_BYTES;
+      store_half_row(v, row, half, t, t + TILE_BYTES);
     }
     fence_async_smem();
-    __syncthreads();  // the box is consumed and the B tile written
-    if (tid == 0) {
-      if (issued < Qi) {
+  }
+  __syncthreads();
+
+  if (warp == LW_TMA) {
+    if (lane == 0) {
+      int issued = first;
+      uint32_t ph = 0;  // phase of box_empty that frees the stage for item `issued`
+      for (int q = first; q < Q; ++q) {
+        if (!wait(&box_empty[p_stage], ph)) break;
         issue_next();
-        ++issued;
+        if (p_stage == 0) ph ^= 1u;
+        issued = q + 1;
       }
-      tc_fence_after();
-      const uint32_t acc = tmem + (uint32_t)(j & 1) * BN;
-      const uint32_t a_hi = smem_u32(a_tiles + (size_t)st * 2 * TILE_BYTES), a_lo = a_hi + TILE_BYTES;
-      const uint32_t b_hi = smem_u32(b_ops + (size_t)b * 2 * TILE_BYTES), b_lo = b_hi + TILE_BYTES;
+      // no box may still be landing when the CTA ends: wait (bounded) for the last ones
+      for (int q = issued > ring ? issued - ring : 0; q < issued; ++q)
+        mbar_wait(smem_u32(&box_full[q % ring]), (uint32_t)((q / ring) & 1));
+    }
+  } else if (warp == LW_MMA) {
+    if (lane == 0) {
+      int last = -1;  // last item whose MMAs were committed
+      int b = 0, st = 0, j = 0;
+      uint32_t ph = 0;
+      for (int q = 0; q < Q; ++q) {
+        const int a = j & 1;
+        if (st == 0 && j >= 2 && !wait(&acc_empty[a], (uint32_t)(((j >> 1) - 1) & 1))) break;
+        if (!wait(&op_full[b], ph)) break;
+        tc_fence_after();
+        const uint32_t acc = tmem + (uint32_t)a * BN;
+        const uint32_t a_hi = smem_u32(a_tiles + (size_t)st * 2 * TILE_BYTES), a_lo = a_hi + TILE_BYTES;
+        const uint32_t b_hi = smem_u32(b_ops + (size_t)b * 2 * TILE_BYTES), b_lo = b_hi + TILE_BYTES;
 #pragma unroll
-      for (int ks = 0; ks < BK / 16; ++ks) {
-        const uint32_t o = ks * 2 * LBO;
-        mma(acc, sdesc(a_hi + o), sdesc(b_hi + o), (st > 0 || ks > 0) ? 1u : 0u);
-        mma(acc, sdesc(a_hi + o), sdesc(b_lo + o), 1u);
-        mma(acc, sdesc(a_lo + o), sdesc(b_hi + o), 1u);
+        for (int ks = 0; ks < BK / 16; ++ks) {
+          const uint32_t o = ks * 2 * LBO;
+          mma(acc, sdesc(a_hi + o), sdesc(b_hi + o), (st > 0 || ks > 0) ? 1u : 0u);
+          mma(acc, sdesc(a_hi + o), sdesc(b_lo + o), 1u);
+          mma(acc, sdesc(a_lo + o), sdesc(b_hi + o), 1u);
+        }
+        commit(smem_u32(&op_empty[b]));
+        if (st == nsteps - 1) commit(smem_u32(&acc_full[a]));
+        last = q;
+        if (++b == nops) b = 0, ph ^= 1u;
+        if (++st == nsteps) st = 0, ++j;
       }
-      commit(smem_u32(&mmad[b]));
-      if (st == nsteps - 1) commit(smem_u32(&accf[j & 1]));
-    } else if (issued < Qi) {
-      ++issued;  // every thread tracks what thread 0 has issued
+      // the tensor memory is released at the end: wait (bounded) for the last MMAs
+      if (last >= 0) mbar_wait(smem_u32(&op_empty[last % nops]), (uint32_t)((last / nops) & 1));
     }
-    pipe.pending[b] = 1;
-    const bool first = st == 0;
-    if (++stage == ring) {
-      stage = 0;
-      fpar ^= 1u;
+  } else if (warp >= LW_OUT0) {
+    // ---- output: TMEM lanes 32 (warp & 3) .. + 31 are rows i0 + 32 (warp & 3) + lane of Z ----
+    const int quarter = warp & 3, r0 = i0 + 32 * quarter;
+    unsigned char *zb = zbox + (size_t)(warp - LW_OUT0) * 2 * kZBox;
+    for (int j = 0; j < mytiles; ++j) {
+      const int a = j & 1;
+      // the TMEM loads are warp-collective: leave or go on together
+      if (!__all_sync(0xffffffffu, wait(&acc_full[a], (uint32_t)((j >> 1) & 1)))) break;
+      tc_fence_after();
+      const long long c0 = (blockIdx.x + (long long)j * gridDim.x) * BN;
+#pragma unroll 1
+      for (int cb = 0; cb < 4; ++cb) {
+        float v[32];
+        tmem_ld32(tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)a * BN + 32 * cb, v);
+        unsigned char *eb = zb + (size_t)(cb & 1) * kZBox;
+        if (lane == 0) bulk_wait_read<1>();  // the store of two blocks ago has read this box
+        __syncwarp();
+        // row `lane`: 128 bytes, 16-byte chunk q at position q ^ (lane & 7) (the map's 128-byte swizzle)
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          *reinterpret_cast<float4 *>(eb + lane * 128 + ((q ^ (lane & 7)) << 4)) =
+              make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          if (c0 + 32 * cb < K && r0 < m) tma_store_2d(&tmZ, (int)(c0 + 32 * cb), r0, smem_u32(eb));
+          bulk_commit();
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&acc_empty[a]));  // tile j + 2 may overwrite the accumulator
     }
-    if (first && j > 0 && !epilogue(j - 1)) {
-      ok = false;
-      ++q;  // item q was consumed
-      break;
-    }
-    if (++st == nsteps) {
-      st = 0;
-      ++j;
+    if (lane == 0) bulk_wait_all();  // the stores have left shared memory before the CTA exits
+  } else {
+    // ---- split: team t takes the items of parity t; a thread splits column `col` of the box.  The
+    // number of stages is even, so that each team meets only its own box barriers (a parity seen by
+    // neither team in between is ambiguous) ----
+    const int team = warp >> 2, col = tid & 127;
+    int stage = team, b = team;
+    uint32_t sph = 0, bph = 0;
+    for (int q = team; q < Q; q += LW_TEAMS) {
+      if (!__all_sync(0xffffffffu, wait(&box_full[stage], sph))) break;
+      const float *src = reinterpret_cast<const float *>(boxes + (size_t)stage * kLmBox) + col;
+      uint4 hi[4], lo[4];
+#pragma unroll
+      for (int c8 = 0; c8 < 4; ++c8) {
+        float x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = src[(8 * c8 + e) * BN];
+        split8(x, hi[c8], lo[c8]);
+      }
+      if (q >= nops && !__all_sync(0xffffffffu, wait(&op_empty[b], bph ^ 1u))) break;
+      unsigned char *ob = b_ops + (size_t)b * 2 * TILE_BYTES;
+#pragma unroll
+      for (int c8 = 0; c8 < 4; ++c8) {
+        const uint32_t off = tile_off(col, 8 * c8);
+        *reinterpret_cast<uint4 *>(ob + off) = hi[c8];
+        *reinterpret_cast<uint4 *>(ob + TILE_BYTES + off) = lo[c8];
+      }
+      fence_async_smem();  // the tiles are read by the tensor cores (async proxy)
+      __syncwarp();
+      // released only now that every lane has used the values it loaded from the box
+      if (lane == 0) {
+        mbar_arrive(smem_u32(&box_empty[stage]));
+        mbar_arrive(smem_u32(&op_full[b]));
+      }
+      stage += LW_TEAMS;
+      if (stage >= ring) stage -= ring, sph ^= 1u;
+      b += LW_TEAMS;
+      if (b >= nops) b -= nops, bph ^= 1u;
     }
   }
-  if (ok && Qi > 0) ok = epilogue((int)mytiles - 1);
-  if (!ok) {
-    // bounded waits for the copies still in flight (items q .. issued - 1) and the last MMAs
-    for (int r = q; r < issued; ++r) mbar_wait(smem_u32(&full[r % ring]), (uint32_t)((r / ring) & 1));
-    pipe.drain(mmad, 0);
-    pipe.drain(mmad, 1);
-    if (tid == 0) atomicExch(err, 1);
-  }
-  if (tid == 0) bulk_wait_all();  // the stores have left shared memory before the CTA exits
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 256);
@@ -1733,12 +1778,17 @@ cudaError_t launch_tc_left_mul(const float *A, int m, int n, const float *Y, lon
   if (K % 4 != 0) return cudaErrorNotSupported;
   if (use_tma()) {
     const int nsteps = (n + tc::BK - 1) / tc::BK;
-    const size_t fixed = ((size_t)nsteps * 2 + 4) * tc::TILE_BYTES + 2 * tc::kEpiBox + 1024 + 256;
+    // three B buffers while four boxes fit beside them (n <= 160), else two; an even number of boxes
     const size_t cap = 227 * 1024;
-    const int ring = fixed + 2 * tc::kLmBox <= cap ? (int)std::min<size_t>(8, (cap - fixed) / tc::kLmBox) : 0;
+    auto fixed_for = [&](int nops) {
+      return ((size_t)nsteps + nops) * 2 * tc::TILE_BYTES + 8 * tc::kZBox + 1024 + 256;
+    };
+    const int nops = fixed_for(3) + 4 * tc::kLmBox <= cap ? 3 : 2;
+    const size_t fixed = fixed_for(nops);
+    const int ring = fixed + 2 * tc::kLmBox <= cap ? (int)std::min<size_t>(8, (cap - fixed) / tc::kLmBox) & ~1 : 0;
     CUtensorMap map, zmap;
     if (ring >= 2 && make_map_f32(&map, Y, n, K, tc::BK, tc::BN, false) &&
-        make_map_f32(&zmap, Z, m, K, tc::BM, 32, true)) {
+        make_map_f32(&zmap, Z, m, K, 32, 32, true)) {
       const int smem = (int)(fixed + (size_t)ring * tc::kLmBox);
       cudaError_t e =
           cudaFuncSetAttribute(tc::tc_left_mul_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1749,7 +1799,7 @@ cudaError_t launch_tc_left_mul(const float *A, int m, int n, const float *Y, lon
       const long long tiles = (K + tc::BN - 1) / tc::BN;
       const int rows = (m + tc::BM - 1) / tc::BM;
       const unsigned gx = (unsigned)std::max(1LL, std::min(tiles, (long long)std::max(1, sms / rows)));
-      tc::tc_left_mul_tma_kernel<<<dim3(gx, rows), tc::NT2, smem, st>>>(A, m, n, map, zmap, K, ring, err);
+      tc::tc_left_mul_tma_kernel<<<dim3(gx, rows), tc::LW_NT, smem, st>>>(A, m, n, map, zmap, K, ring, nops, err);
       return cudaGetLastError();
     }
   }
