@@ -942,8 +942,17 @@ ace_status run_chain_f64(ace_op *op, const double *phi, const DeviceTables *tab,
   const ace_desc &d = op->desc;
   const long long N = op->N;
   cudaStream_t st = op->stream;
-  const int nstreams = std::min(kSide, std::max(1, cp.streams));
-  const int B = std::min(65535, std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams)));
+  int nstreams = std::min(kSide, std::max(1, cp.streams));
+  int B = std::min(65535, std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams)));
+  // the pencil route keeps within ACE_SCRATCH_MB where it is set (one pack at least); W does not depend
+  // on the batches
+  const int budget_mb = pops ? 0 : env_int("ACE_SCRATCH_MB", 0);
+  if (budget_mb > 0) {
+    const double per = sizeof(cpx<double>) * (double)N;
+    const int slots = (int)std::min(65535.0, std::max(1.0, std::floor(budget_mb * 1048576.0 / per)));
+    nstreams = std::min(nstreams, slots);
+    B = std::min(B, slots / nstreams);
+  }
   std::vector<int4> packs;
   form_packs(op->pairs_h, cp.RB, packs);
   void *tmp = nullptr;

@@ -52,3 +52,20 @@ def test_w_from_stored_potentials(grid, pairs):
     torch.cuda.synchronize()
     assert torch.equal(W[0], W[1])
     assert rel_max(W[0].cpu().numpy(), W[2].cpu().numpy()) <= FP64_ARRAY_RTOL
+
+
+@pytest.mark.parametrize("mb", ["1", "3", "64"])
+def test_pencil_scratch_budget_leaves_w_alone(monkeypatch, mb):
+    import torch
+
+    grid = (5, 135, 81)  # a plane shape of the pencil route, 0.83 MB per pack
+    lat = np.diag([6.0 + 0.05 * g for g in grid])
+    phi, _, _ = gaussian_orbitals(grid, lat, 5, 2, np.random.default_rng(3))
+    x = torch.from_numpy(phi).cuda()
+    d = ace.make_desc(grid, lat, 5, prec=ace.ACE_FP64)
+    W = [torch.full_like(x, 7.0) for _ in range(2)]
+    abi.ace_exchange_w(d, x, PAIRS[-1], W[0])
+    monkeypatch.setenv("ACE_SCRATCH_MB", mb)
+    abi.ace_exchange_w(d, x, PAIRS[-1], W[1])
+    torch.cuda.synchronize()
+    assert torch.equal(W[0], W[1])
