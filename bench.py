@@ -33,18 +33,17 @@ METRIC = "ACE builds/s (128 orb, 96^3), mixed vs FP64 GPU form; E_x err <=1e-6 H
 UNIT = "builds/s"
 GOLDEN = os.path.join(ROOT, "tests", "golden", "oracle_values.json")
 # DRAM bytes (read + write) of the pair chain per build of the water32 workload, from one ncu capture
-# of the current chain kernels with caches not flushed (profiles/pair_chain_plane_water32_96c.md);
-# set to None whenever those kernels change.
-CHAIN_DRAM_BYTES_PER_BUILD = 8.17e9
-# DRAM bytes (read + write) per launch of the dense kernels of the same workload: M and xi from one
-# ncu capture with caches not flushed (profiles/dense_tc_water32_96c.md), the CUDA-core screen from
-# its capture with the plane maxima (profiles/screen_syrk_water32_96c.md: 950.9 GB/s over 482.0 us,
-# 458.3 MB), xi from the capture of the left multiply with its short-last-tile support (4.22 TB/s
-# over 207.8 us, 876.5 MB); None once a kernel changes
-DENSE_DRAM_BYTES = {"screen": 458.3e6, "M": 929.8e6, "xi": 876.5e6}
-# DRAM bytes per SCDM localisation of the 128-orbital 96^3 set: 128 selection passes at 436.1 MB
-# (ncu, profiles/scdm_water32_96c.md) + the left multiply Phi = U^T Psi (876.5 MB) + the transpose
-SCDM_DRAM_BYTES = 128 * 436.1e6 + 876.5e6 + 906e6
+# of the current chain kernels with caches not flushed (profiles/pair_chain_plane_water32_96c.md:
+# 11.03 GB for 2666 pairs of a like input, scaled to this workload's 2346); set to None whenever those
+# kernels change.
+CHAIN_DRAM_BYTES_PER_BUILD = 11.03e9 * 2346 / 2666
+# DRAM bytes (read + write) per launch of the dense kernels of the same workload, from ncu captures with
+# caches not flushed: M and xi (profiles/dense_tc_water32_96c.md), the CUDA-core screen with the plane
+# maxima (profiles/screen_syrk_water32_96c.md: 950.9 GB/s over 482.0 us, 458.3 MB); None once a kernel
+# changes
+DENSE_DRAM_BYTES = {"screen": 458.3e6, "M": 936.0e6, "xi": 888.3e6}
+# DRAM bytes per SCDM localisation of the 128-orbital 96^3 set (ncu, profiles/scdm_water32_96c.md)
+SCDM_DRAM_BYTES = 2649e6
 
 
 def _peaks():
@@ -669,9 +668,9 @@ def run_scdm(args):
         del src, out
     mixed = res[ace.ACE_MIXED]
     peaks, peak_kind = _peaks()
-    # per selection step: read Psi (n N FP32) and read + write the residual norms (N FP64);
-    # then Phi = U^T Psi reads Psi and writes Phi
-    alg = n * (4.0 * n * N + 16.0 * N) + 8.0 * n * N
+    # the norms read Psi (n N FP32), Phi = U^T Psi reads Psi and writes Phi; the selection steps read only
+    # the blocks of points that can hold the pivot (not counted)
+    alg = 12.0 * n * N
     achieved = alg / (mixed["ms"] * 1e-3) / 1e9
     line = {
         "metric": "SCDM localisations/s (128 orb, 96^3)", "value": mixed["per_s"], "unit": "localisations/s",
@@ -682,10 +681,10 @@ def run_scdm(args):
         "fp64_form": {"value": res[ace.ACE_FP64]["per_s"], "unit": "localisations/s",
                       "ms_per_step": res[ace.ACE_FP64]["ms"],
                       "same_pivots_as_mixed": bool(np.array_equal(res[ace.ACE_FP64]["piv"], mixed["piv"]))},
-        "roofline": {"kernel": "whole ace_scdm call (n selection passes over Psi dominate)", "bound": "hbm",
+        "roofline": {"kernel": "whole ace_scdm call (n dependent selection steps dominate)", "bound": "latency",
                      "achieved": achieved, "peak": peaks.get("hbm_gbs"), "unit": "GB/s",
                      "frac": achieved / peaks.get("hbm_gbs"), "traffic": SCDM_DRAM_BYTES, "peak_kind": peak_kind,
-                     "algorithmic_bytes": f"n (4 n N + 16 N) + 8 n N = {alg:.4g} B per localisation"},
+                     "algorithmic_bytes": f"12 n N = {alg:.4g} B per localisation"},
         "e2e": res["e2e"],
         "gpu_launches": mixed["launches"],
         "clocks": mixed["clk"],

@@ -245,8 +245,9 @@ ace_status ace_apply(const ace_op *op, const void *psi, ace_dtype dtype, int m, 
  *   phi:  output [norb][npts] of `dtype`, on the same side as psi (may not alias it).
  *   piv_host: optional host int32 [norb] receiving c_0..c_{n-1}; u_host: optional host double
  *         [norb][norb] receiving U; launches: optional, the number of this library's kernels run.
- *   prec: ACE_FP64 every step in FP64.  ACE_MIXED: psi in FP32, residual norms in FP64 with the
- *         projections u_k . psi(r) summed as FP32 products in 8-term FP32 partials; M, U and
+ *   prec: ACE_FP64 every step in FP64.  ACE_MIXED: psi in FP32, residual norms as 64-bit fixed-point
+ *         numbers (60 bits below the largest norm) with the projections u_k . psi(r) summed in FP32
+ *         trees; M, U and
  *         (M^T M)^{-1/2} (coupled Newton-Schulz) in FP64; Phi = U^T Psi by BF16x3 tensor-core
  *         products (FP32-level).  Near-equal residuals may then select another, equally valid,
  *         point than FP64 arithmetic would.
@@ -295,8 +296,8 @@ ace_status ace_kernel_launches(const ace_op *op, long *launches);
  * Screens `phi` as ace_build does, then times the pair chain on a sample of up to 480 of its packs
  * for each candidate setting of the stream-batched chain: packs per batch {1,2,3,4,6}, side streams
  * {2,4,8}, L2 set-aside for the scratch {0, 60 MB}, rows per block of the pack order {1,2,4,8};
- * then, on the best of those, the pencil tile of the axis-1 pass (FP32: 32 columns with the default
- * or the other thread count, or 16 columns); and the persistent chain (one launch walking the pack
+ * then, on the best of those, the pencil tile of the axis-1 pass (FP32: 8 pairs of lines per warp in
+ * blocks of two or four warps, or 4 pairs per warp); and the persistent chain (one launch walking the pack
  * list through a device task queue) with queue lags {2,3,4} where its grid is compiled.  The
  * fastest setting is kept for this grid and precision and used by later builds in the process;
  * with the environment variable ACE_TUNE_FILE set, the table is also read from and written to that

@@ -572,7 +572,8 @@ __global__ void __launch_bounds__(NT) tc_left_mul_kernel(const float *__restrict
 // MMAs in flight are waited for (bounded), TMEM is released and *err is set.
 // Bound by reading Y and writing Z: 128 rows of 96^3 (906 MB) in 152 us, 5.9 TB/s; one loop of eight
 // warps with CTA barriers took 1.1 us per item from L2 as from memory, 209 us.  64 rows of 72^3
-// 62 -> 36 us; 256 rows of 128^3, where each box feeds two row blocks, 1610 -> 1375 us.
+// 62 -> 36 us; 256 rows of 128^3, where each box feeds two row blocks, 1610 -> 1375 us.  An L2
+// set-aside of 60 MB in the context (the pair chain's) slows streaming writes: 200 us at 96^3 then.
 // ----------------------------------------------------------------------------------------
 constexpr uint32_t kLmBox = BK * BN * 4;  // one Y box: 32 rows x 128 FP32 columns
 constexpr uint32_t kZBox = 32 * 32 * 4;   // one Z box: 32 rows x 32 FP32 columns
