@@ -1525,6 +1525,102 @@ __global__ void __cluster_dims__(CHC_C, 1, 1) __launch_bounds__(CHC_NT)
   if (rank == 0 && tid == 0) *status = 0;
 }
 
+// ----------------------------------------------------------------------------------------
+// The same for n <= 32 in one CTA.  A chain of n pivots bounds it: each FP64 instruction of the chain takes
+// a scheduler about 64 cycles, and the cluster form adds its barriers and panel copies (26 us at n = 16,
+// this one 19).
+//   - Lane i of every warp is row i; warp w holds the columns k = w, w + 8, ... of -M and of Y in
+//     registers.  Elimination in LDL^T form: column j, published in shared memory by its warp, gives
+//     t_i = A_ij / d_j = U_ij, then A_ik -= t_i A_kj (k > j) and Y_ic -= t_i Y_jc (c <= j), so that
+//     Y = U^-1 grows along with U and only one reciprocal per column is on the chain.
+//   - The warp that owns column j + 1 updates it first and publishes it before the rest of its work.
+//   - At the end L = U sqrt(D) and L^-1 = D^-1/2 Y, all square roots side by side.
+// Every element's arithmetic is fixed, so the result repeats bit for bit.  Same status codes as above.
+// ----------------------------------------------------------------------------------------
+constexpr int CHS_MAX_N = 32, CHS_W = 8, CHS_NT = CHS_W * 32, CHS_S = CHS_MAX_N / CHS_W;
+
+__global__ void __launch_bounds__(CHS_NT) cholesky_small_kernel(const double *__restrict__ M_raw, int n,
+                                                                double spin_factor, double *__restrict__ M,
+                                                                double *__restrict__ L, double *__restrict__ Linv,
+                                                                double *__restrict__ energy,
+                                                                int *__restrict__ status) {
+  __shared__ double col[2][CHS_MAX_N], diag[CHS_MAX_N], U[CHS_MAX_N][CHS_MAX_N + 1];
+  const int tid = threadIdx.x, i = tid & 31, w = tid >> 5;
+  double a[CHS_S], y[CHS_S];
+  bool ok = true;
+#pragma unroll
+  for (int s = 0; s < CHS_S; ++s) {
+    const int k = s * CHS_W + w;
+    a[s] = 0.0;
+    y[s] = 0.0;
+    if (i < n && k < n) {
+      const double v = i == k ? M_raw[i * n + i] : 0.5 * (M_raw[i * n + k] + M_raw[k * n + i]);
+      M[i * n + k] = v;
+      ok = ok && finite_bits(v);
+      a[s] = -v;
+    }
+  }
+  if (w == 0) {
+    double part = i < n ? M_raw[i * n + i] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
+    if (i == 0) *energy = 0.5 * spin_factor * part;
+    col[0][i] = a[0];
+  }
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0) *status = 2000000;
+    return;
+  }
+#pragma unroll
+  for (int jb = 0; jb < CHS_S; ++jb) {
+    for (int jw = 0; jw < CHS_W; ++jw) {
+      const int j = jb * CHS_W + jw;
+      if (j >= n) break;
+      if (j > 0) __syncthreads();
+      const double *c = col[j & 1];
+      const double d = c[j];
+      if (__double_as_longlong(d) <= 0 || !finite_bits(d)) {  // the same value in every thread
+        if (tid == 0) *status = 1000000 + j;
+        return;
+      }
+      const double t = i > j ? c[i] * __drcp_rn(d) : 0.0;
+      bool first = w == ((j + 1) & (CHS_W - 1));  // owner of column j + 1, not published yet
+#pragma unroll
+      for (int s = jb; s < CHS_S; ++s) {
+        const int k = s * CHS_W + w;
+        if (k > j && k < n) {
+          a[s] = fma(-t, c[k], a[s]);
+          if (first) {
+            col[(j + 1) & 1][i] = a[s];
+            first = false;
+          }
+        }
+      }
+      if (w == jw) U[j][i] = t;
+      if (tid == 0) diag[j] = d;
+#pragma unroll
+      for (int s = 0; s <= jb; ++s) {
+        const int cc = s * CHS_W + w;
+        const double yj = __shfl_sync(0xffffffffu, y[s], j);
+        if (cc <= j) y[s] = fma(-t, cc == j ? 1.0 : yj, y[s]);
+      }
+    }
+  }
+  __syncthreads();
+  const double di = i < n ? diag[i] : 1.0;
+  const double root = sqrt(di), inv = 1.0 / root;
+  if (w == 0) col[0][i] = root;
+  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < CHS_S; ++s) {
+    const int k = s * CHS_W + w;
+    if (i < n && k < n) {
+      L[i * n + k] = k < i ? U[k][i] * col[0][k] : k == i ? root : 0.0;
+      Linv[i * n + k] = k < i ? y[s] * inv : k == i ? inv : 0.0;
+    }
+  }
+  if (tid == 0) *status = 0;
+}
+
 static bool cluster_cholesky_off() {
   static const bool off = [] {
     const char *v = std::getenv("ACE_CHOLESKY_ONE_CTA");
@@ -1559,6 +1655,12 @@ static bool cluster_ready(K kernel, size_t smax, int *state, cudaStream_t st) {
 
 cudaError_t launch_cholesky(const double *M_raw, int n, double spin_factor, double *M, double *L, double *Linv,
                             double *energy, int *status, double *gwork, cudaStream_t st) {
+  // up to 32 rows (one lane each) in one CTA; stage times, small against cluster: 14 and 23 us at n = 12, 19
+  // and 26 at 16, 27 and 37 at 24
+  if (!cluster_cholesky_off() && n <= CHS_MAX_N) {
+    cholesky_small_kernel<<<1, CHS_NT, 0, st>>>(M_raw, n, spin_factor, M, L, Linv, energy, status);
+    return cudaGetLastError();
+  }
   if (!cluster_cholesky_off() && n <= CHC_MAX_N) {
     static int state[64] = {};
     const size_t smax = sizeof(double) * ((size_t)CHC_MAX_N * (CHC_MAX_N | 1) + (size_t)CHC_MAX_N);
