@@ -1067,7 +1067,7 @@ cudaError_t dense_gram(const T *X, int nx, const T *Y, int ny, long long K, doub
 // Z = A Y, A (m x n) in T
 template <typename T>
 cudaError_t dense_left_mul(const T *A, int m, int n, const T *Y, long long K, T *Z, int *err, cudaStream_t st,
-                           long *launches) {
+                           long *launches, bool lower = false) {
   *launches += 1;
   if constexpr (sizeof(T) == 4) {
     if (m <= 8) return ace::launch_skinny_left_mul(A, m, n, Y, K, Z, st);
@@ -1076,7 +1076,7 @@ cudaError_t dense_left_mul(const T *A, int m, int n, const T *Y, long long K, T 
       if (e != cudaErrorNotSupported) return e;  // else the CUDA-core kernel below takes the shape
     }
   }
-  return ace::launch_left_mul<T>(A, m, n, Y, K, Z, st);
+  return ace::launch_left_mul<T>(A, m, n, Y, K, Z, st, lower);
 }
 
 // Relative distance from rho_cut within which screen values are recomputed (twice the BF16x3
@@ -1409,7 +1409,7 @@ ace_status factor_and_project(ace_op *op, const T *W) {
     ++op->launches;
     Linv_T = static_cast<const T *>(tmp);
   }
-  ACE_CUDA(dense_left_mul<T>(Linv_T, n, n, W, N, static_cast<T *>(op->xi), op->tc_err, st, &op->launches), "xi");
+  ACE_CUDA(dense_left_mul<T>(Linv_T, n, n, W, N, static_cast<T *>(op->xi), op->tc_err, st, &op->launches, true), "xi");
   ACE_CUDA(mark(op, 5, st), "event record");
   char *rb = static_cast<char *>(op->readback);
   ACE_CUDA(cudaMemcpyAsync(rb + 4, op->status_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, st), "status readback");

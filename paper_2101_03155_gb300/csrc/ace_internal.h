@@ -162,7 +162,8 @@ cudaError_t launch_gram(const T *X, int nx, const T *Y, int ny, long long K, dou
                         bool upper_only, double *G, cudaStream_t st, double *partial = nullptr);
 size_t gram_chunks_bytes(int nx, int ny, long long K);
 template <typename T>
-cudaError_t launch_left_mul(const T *A, int m, int n, const T *Y, long long K, T *Z, cudaStream_t st);
+cudaError_t launch_left_mul(const T *A, int m, int n, const T *Y, long long K, T *Z, cudaStream_t st,
+                            bool lower = false);  // lower: A is lower triangular (m = n)
 // FP32 products with at most 8 rows on one side, on the CUDA cores
 bool skinny_gram_ok(const float *X, int nx, const float *Y, int ny, long long K);
 size_t skinny_gram_bytes(int nx, int ny, long long K);

@@ -782,49 +782,59 @@ cudaError_t launch_skinny_left_mul(const float *A, int m, int n, const float *Y,
 }
 
 // ----------------------------------------------------------------------------------------
-// Left multiply Z (m x K) = A (m x n) * Y (n x K); 64 x 64 tile, k-step 16, 4 x 4 per thread.
+// Left multiply Z (m x K) = A (m x n) * Y (n x K); 16 R x 64 tile, k-step 16, R x 4 per thread.
+// Bound by the FP64 pipe (two FMA per clock and SM) in double, so rows of padding cost their full
+// time: the launcher takes as few row blocks as tiles of 64 rows would need and the smallest R that
+// covers m with them (12 rows: a tile of 16, not 64; 70 rows: two of 48, not of 64).  With a lower
+// triangular A (m = n) a row block stops at its last diagonal element, and blocks are 16 rows: at 64 rows
+// that leaves 5/8 of the products.  Every output adds its terms in the same order whatever R is.
+// xi in FP64: 12 rows of 40x45x48 149 -> 37 us, 64 rows of 72^3 2.49 -> 1.55 ms.
 // ----------------------------------------------------------------------------------------
-constexpr int LM_BM = 64, LM_BN = 64, LM_BK = 16, LM_NT = 256;
+constexpr int LM_BN = 64, LM_BK = 16, LM_NT = 256, LM_RMAX = 4;
 
-template <typename T>
+template <typename T, int R>
 __global__ void __launch_bounds__(LM_NT) left_mul_kernel(const T *__restrict__ A, int m, int n,
-                                                         const T *__restrict__ Y, long long K, T *__restrict__ Z) {
+                                                         const T *__restrict__ Y, long long K, T *__restrict__ Z,
+                                                         bool lower) {
+  constexpr int LM_BM = 16 * R;
   __shared__ T as[LM_BK][LM_BM + 1];
   __shared__ T ys[LM_BK][LM_BN];
   const int i0 = blockIdx.y * LM_BM;
   const long long c0 = (long long)blockIdx.x * LM_BN;
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  T acc[4][4];
+  T acc[R][4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < R; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = (T)0;
-  for (int l0 = 0; l0 < n; l0 += LM_BK) {
+  const int le = lower ? min(n, i0 + LM_BM) : n;  // columns of A past here are zero
+  for (int l0 = 0; l0 < le; l0 += LM_BK) {
     for (int e = tid; e < LM_BM * LM_BK; e += LM_NT) {
       const int r = e / LM_BK, c = e % LM_BK;
-      as[c][r] = (i0 + r < m && l0 + c < n) ? A[(long long)(i0 + r) * n + l0 + c] : (T)0;
+      as[c][r] = (i0 + r < m && l0 + c < le) ? A[(long long)(i0 + r) * n + l0 + c] : (T)0;
     }
     for (int e = tid; e < LM_BK * LM_BN; e += LM_NT) {
       const int r = e / LM_BN, c = e % LM_BN;
-      ys[r][c] = (l0 + r < n && c0 + c < K) ? Y[(long long)(l0 + r) * K + c0 + c] : (T)0;
+      ys[r][c] = (l0 + r < le && c0 + c < K) ? Y[(long long)(l0 + r) * K + c0 + c] : (T)0;
     }
     __syncthreads();
 #pragma unroll
     for (int c = 0; c < LM_BK; ++c) {
-      T ar[4], yr[4];
+      if (l0 + c >= le) break;
+      T ar[R], yr[4];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) ar[a] = as[c][ty + 16 * a];
+      for (int a = 0; a < R; ++a) ar[a] = as[c][ty + 16 * a];
 #pragma unroll
       for (int b = 0; b < 4; ++b) yr[b] = ys[c][tx + 16 * b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int a = 0; a < R; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[a][b] += ar[a] * yr[b];
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < R; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const int i = i0 + ty + 16 * a;
@@ -834,14 +844,21 @@ __global__ void __launch_bounds__(LM_NT) left_mul_kernel(const T *__restrict__ A
 }
 
 template <typename T>
-cudaError_t launch_left_mul(const T *A, int m, int n, const T *Y, long long K, T *Z, cudaStream_t st) {
-  dim3 grid((unsigned)((K + LM_BN - 1) / LM_BN), (unsigned)((m + LM_BM - 1) / LM_BM));
-  left_mul_kernel<T><<<grid, LM_NT, 0, st>>>(A, m, n, Y, K, Z);
+cudaError_t launch_left_mul(const T *A, int m, int n, const T *Y, long long K, T *Z, cudaStream_t st, bool lower) {
+  const int rmax = lower ? 1 : LM_RMAX;
+  const int blocks = (m + 16 * rmax - 1) / (16 * rmax), R = ((m + blocks - 1) / blocks + 15) / 16;
+  const dim3 grid((unsigned)((K + LM_BN - 1) / LM_BN), (unsigned)blocks);
+  auto run = [&](auto kernel) { kernel<<<grid, LM_NT, 0, st>>>(A, m, n, Y, K, Z, lower); };
+  if (R <= 1) run(left_mul_kernel<T, 1>);
+  else if (R == 2) run(left_mul_kernel<T, 2>);
+  else if (R == 3) run(left_mul_kernel<T, 3>);
+  else run(left_mul_kernel<T, 4>);
   return cudaGetLastError();
 }
-template cudaError_t launch_left_mul<float>(const float *, int, int, const float *, long long, float *, cudaStream_t);
+template cudaError_t launch_left_mul<float>(const float *, int, int, const float *, long long, float *, cudaStream_t,
+                                            bool);
 template cudaError_t launch_left_mul<double>(const double *, int, int, const double *, long long, double *,
-                                             cudaStream_t);
+                                             cudaStream_t, bool);
 
 // ----------------------------------------------------------------------------------------
 // Cholesky of -M, L^-1 and E_x in one CTA (FP64).  A = -M lives in shared memory when n <= 128
