@@ -955,6 +955,9 @@ ace_status run_chain_f64(ace_op *op, const double *phi, const DeviceTables *tab,
   }
   std::vector<int4> packs;
   form_packs(op->pairs_h, cp.RB, packs);
+  // only the side streams that get a batch: each of them is joined by its batches' events, and a stream
+  // capture wants every forked stream joined
+  nstreams = std::min(nstreams, ((int)packs.size() + B - 1) / B);
   void *tmp = nullptr;
   ACE_CUDA(cudaMallocAsync(&tmp, sizeof(int4) * packs.size(), st), "alloc packs");
   temps.push_back(tmp);
