@@ -1807,7 +1807,7 @@ cudaError_t launch_tc_left_mul(const float *A, int m, int n, const float *Y, lon
   if (K % tc::BN != 0) return cudaErrorNotSupported;  // the register-staged kernel stores whole tiles
   const int nsteps = (n + tc::BK - 1) / tc::BK;
   const int smem = (int)(((size_t)nsteps * 2 + 4) * tc::TILE_BYTES + 2048);
-  if (smem > 227 * 1024) return cudaErrorInvalidValue;
+  if (smem > 227 * 1024) return cudaErrorNotSupported;  // the rows of A do not fit (n > 384)
   cudaError_t e = cudaFuncSetAttribute(tc::tc_left_mul_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 152;
