@@ -245,9 +245,9 @@ ace_status ace_apply(const ace_op *op, const void *psi, ace_dtype dtype, int m, 
  *   phi:  output [norb][npts] of `dtype`, on the same side as psi (may not alias it).
  *   piv_host: optional host int32 [norb] receiving c_0..c_{n-1}; u_host: optional host double
  *         [norb][norb] receiving U; launches: optional, the number of this library's kernels run.
- *   prec: ACE_FP64 every step in FP64.  ACE_MIXED: psi in FP32, residual norms as 64-bit fixed-point
- *         numbers (60 bits below the largest norm) with the projections u_k . psi(r) summed in FP32
- *         trees; M, U and
+ *   prec: ACE_FP64 every step in FP64.  ACE_MIXED: psi in FP32; |psi(r)|^2 and the projections
+ *         u_k . psi(r) are summed in FP32 trees, and the residual norms lose the projections' squares
+ *         with 55 bits per step; M, U and
  *         (M^T M)^{-1/2} (coupled Newton-Schulz) in FP64; Phi = U^T Psi by BF16x3 tensor-core
  *         products (FP32-level).  Near-equal residuals may then select another, equally valid,
  *         point than FP64 arithmetic would.

@@ -16,6 +16,7 @@
 #include <cstdint>
 
 #include "ace_internal.h"
+#include "residual_key.h"
 
 namespace ace {
 namespace {
@@ -34,39 +35,9 @@ constexpr double kDependent32 = 1e-10;  // the same with FP32 Gram-Schmidt
 // Order key of an FP64 residual norm: the bits of a double compare like the values for non-negative ones,
 // with chosen points (-1) below them and NaN (never chosen) at kNone.  Comparisons of FP64 values would run
 // on the FP64 pipe, which issues one warp instruction per 64 cycles.
-constexpr long long kNone = (long long)0x8000000000000000ull;
 __device__ __forceinline__ long long res_key(double v) {
   const long long b = __double_as_longlong(v);
   return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? kNone : b;
-}
-
-// The FP32 selection keeps its residual norms as 64-bit fixed-point numbers in units of 2^(E - 60), E the
-// exponent of the largest |psi(r)|^2: exact sums of exact squares down to 2^-60 of the largest norm (an FP64
-// sum rounds to 2^-53 of each residual), with integer adds of a few cycles where a chain of dependent FP64
-// updates took 200 cycles a step.  -1 marks chosen points, kNone a norm that is not a number.  Until a
-// block is first updated its norms are the FP32 values of the start, as their bits with kRaw set (E is not
-// known before every norm is); they are ordered like the numbers.
-constexpr long long kRaw = 1ll << 62;
-__device__ __forceinline__ long long raw_norm(float v) {
-  return v >= 0.f ? kRaw | (long long)__float_as_uint(v) : kNone;  // a sum of squares: never negative
-}
-__device__ __forceinline__ int float_exp(unsigned b) { return max((int)(b >> 23 & 255), 1) - 150; }  // of the last bit
-__device__ __forceinline__ unsigned float_mant(unsigned b) { return (b & 0x7fffff) | (b >> 23 & 255 ? 0x800000u : 0u); }
-__device__ __forceinline__ long long shift_to(unsigned long long m, int t) {
-  return t >= 0 ? (long long)(m << min(t, 63)) : (t > -64 ? (long long)(m >> -t) : 0);
-}
-// the value of a stored norm (raw or fixed) in fixed point; unit exponent e0 = E - 60
-__device__ __forceinline__ long long to_fixed(long long v, int e0) {
-  if (v < kRaw) return v;
-  const unsigned b = (unsigned)v;
-  return shift_to(float_mant(b), float_exp(b) - e0);
-}
-// v - p^2, not below 0 (0 when p is not finite), for v >= 0
-__device__ __forceinline__ long long downdate(long long v, float p, int e0) {
-  const unsigned b = __float_as_uint(p) & 0x7fffffff;
-  const unsigned long long m = float_mant(b);
-  const long long t = v - shift_to(m * m, 2 * float_exp(b) - e0);
-  return v < 0 ? v : (t < 0 || b >= 0x7f800000u ? 0 : t);
 }
 
 // (key, index) maximum, the smaller index winning ties
@@ -113,7 +84,6 @@ struct SelArgs {
   long long *bmax;       // [blocks]
   int *bcnt;             // [blocks]
   long long *thr;        // [n + 1], from 0
-  int *unit;             // exponent of the fixed-point unit, set by the first pivot step
 };
 
 template <typename T>
@@ -143,7 +113,7 @@ struct __align__(16) ScdmSmem {
   double rv[kUpdNT / 32], rv0[kUpdNT / 32];
   long long rk[kUpdNT / 32], ri[kUpdNT / 32], tk[kUpdNT / 32], ti[kUpdNT / 32];
   long long chosen, top;
-  int last, unit;
+  int last;
 };
 
 __device__ __forceinline__ float dot4(float4 a, float4 b) {
@@ -257,13 +227,12 @@ __device__ __forceinline__ void stage_rows(const float *Ub, int nf, int j, int u
 // use (loads from L2 one vector at a time took most of a long catch-up).
 __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ psi, int n, long long N, long long *d,
                                                     const SelArgs &s, long long blk, long long r0, int lim, int j, int k,
-                                                    int upto, bool stop, int e0, long long dr, float (&x)[32],
+                                                    int upto, bool stop, long long dr, float (&x)[32],
                                                     float4 *stage,
                                                     long long &best, long long &bi) {
   const int j_in = j;
   const long long thr = stop ? __ldcg(s.thr + k) : kNone;
   const float *Ub = static_cast<const float *>(s.Ub);
-  dr = to_fixed(dr, e0);
   long long mx = blk_max(dr);
   if (n <= 128) {
     const int c = threadIdx.x & 3, nf = (n + 3) / 4;
@@ -296,7 +265,7 @@ __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ ps
       }
 #pragma unroll
       for (int q = 0; q < kRows; ++q)
-        if (q < m) dr = downdate(dr, pm[q], e0);
+        if (q < m) dr = key_downdate(dr, __float_as_uint(pm[q]));
       j += m;
       mx = blk_max(dr);
       buf ^= 1;
@@ -311,7 +280,7 @@ __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ ps
       const int m = min(4, upto - j);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        if (q < m) dr = downdate(dr, pm[q], e0);
+        if (q < m) dr = key_downdate(dr, __float_as_uint(pm[q]));
       j += m;
       mx = blk_max(dr);
     }
@@ -320,16 +289,16 @@ __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ ps
   return mx;
 }
 __device__ long long refresh_block(const float *__restrict__ psi, int n, long long N, long long *d, const SelArgs &s,
-                                   long long blk, int k, int upto, bool stop, int e0, float4 *stage,
+                                   long long blk, int k, int upto, bool stop, float4 *stage,
                                    long long &best, long long &bi) {
   long long r0, dr;
   int lim, j;
   float x[32];
   load_state(psi, n, N, d, s, blk, r0, lim, j, dr, x);
-  return refresh_loaded(psi, n, N, d, s, blk, r0, lim, j, k, upto, stop, e0, dr, x, stage, best, bi);
+  return refresh_loaded(psi, n, N, d, s, blk, r0, lim, j, k, upto, stop, dr, x, stage, best, bi);
 }
 
-// Stored residuals: FP64 values, or the fixed-point numbers of the FP32 selection
+// Stored residuals: FP64 values, or the keys of the FP32 selection (residual_key.h)
 template <typename T>
 struct Resid {
   using type = double;
@@ -371,11 +340,6 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
       sm.chosen = bi < N ? bi : 0;
       s.piv[k] = (int)sm.chosen;
       d[sm.chosen] = -1;
-      if constexpr (sizeof(T) == 4) {
-        // the largest norm of all gives the fixed-point unit (an infinite one: any)
-        if (k == 0) *s.unit = float_exp((unsigned)best) + 23 - 60;
-        sm.unit = k == 0 ? float_exp((unsigned)best) + 23 - 60 : *s.unit;
-      }
     }
   }
   __syncthreads();
@@ -499,7 +463,7 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
       __syncthreads();  // u_k for the CTA, in L2
       if (seed < N) {
         if (sr0 + (lane >> 2) == cr) seed_d = -1;
-        refresh_loaded(psi, n, N, d, s, seed, sr0, slim, sj, k + 1, k + 1, true, sm.unit, seed_d, sv, stage + warp * kStage, best, bi);
+        refresh_loaded(psi, n, N, d, s, seed, sr0, slim, sj, k + 1, k + 1, true, seed_d, sv, stage + warp * kStage, best, bi);
       }
     }
   }
@@ -626,7 +590,7 @@ __global__ void __launch_bounds__(kUpdNT) scdm_norm_kernel(const float *__restri
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
       for (int l = 0; l < o; ++l) acc[l] += acc[l + o];
-    const long long dr = r < N ? raw_norm(acc[0]) : -1;
+    const long long dr = r < N ? key_of_bits(__float_as_uint(acc[0])) : -1;
     long long mx = dr;  // over the 8 lanes of a block
     for (int o = kBlk / 2; o > 0; o >>= 1) {
       const long long v = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -650,7 +614,6 @@ __global__ void __launch_bounds__(kUpdNT) scdm_norm_kernel(const float *__restri
 // threshold and which a later step will need: without it the longest catch-up of a step was 57 vectors on
 // average (128 orbitals on 96^3), a chain of dependent FP64 updates (8.0 ms per call).  A CTA leaves out the
 // block with its largest bound, which the pivot step may be working on.
-constexpr int kSoonFrac = 5;   // bounds from 1 - 1 / kSoonFrac of the threshold on
 constexpr int kAhead = 8;      // vectors per step and block
 constexpr int kAheadMost = 2;  // blocks per warp and step
 __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__restrict__ psi, int n, long long N,
@@ -663,18 +626,17 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
   const long long nb = (N + kBlk - 1) / kBlk;
   const long long nwarps = (long long)gridDim.x * (kUpdNT / 32);
   const long long w = (long long)blockIdx.x * (kUpdNT / 32) + (threadIdx.x >> 5);
-  const int e0 = *s.unit;
   long long thr = __ldcg(s.thr + s.k);
-  const long long soon = thr - thr / kSoonFrac;
+  const long long soon = key_somewhat_below(thr);
   long long best = kNone, bi = N, top = kNone, ti = N;
   for (long long b0 = w; b0 < nb; b0 += 32 * nwarps) {
     const long long b = b0 + lane * nwarps;
-    long long bound = b < nb ? to_fixed(s.bmax[b], e0) : kNone;
+    long long bound = b < nb ? s.bmax[b] : kNone;
     unsigned left = __ballot_sync(full, bound >= 0 && bound >= thr);
     while (left) {
       const int src = __ffs(left) - 1;
       left &= left - 1;
-      const long long mx = refresh_block(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, s.k, true, e0, stage, best, bi);
+      const long long mx = refresh_block(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, s.k, true, stage, best, bi);
       if (lane == src) bound = mx;
       if (left) {
         thr = __ldcg(s.thr + s.k);
@@ -687,12 +649,12 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
   int most = kAheadMost;
   for (long long b0 = w; b0 < nb && most > 0; b0 += 32 * nwarps) {
     const long long b = b0 + lane * nwarps;
-    const long long bound = b < nb ? to_fixed(s.bmax[b], e0) : kNone;
+    const long long bound = b < nb ? s.bmax[b] : kNone;
     const int cnt = bound >= 0 && bound >= soon && b != sm.top ? s.bcnt[b] : s.k;
     for (unsigned ahead = __ballot_sync(full, cnt < s.k); ahead && most > 0; ahead &= ahead - 1, --most) {
       const int src = __ffs(ahead) - 1;
       refresh_block(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, min(s.k, __shfl_sync(full, cnt, src) + kAhead), false,
-                    e0, stage, best, bi);
+                    stage, best, bi);
     }
   }
 }
@@ -826,7 +788,7 @@ __global__ void scdm_factor_kernel(const double *__restrict__ M, const double *_
 }
 
 struct Layout {
-  size_t d, bval, bidx, tval, tidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count, bmax, bcnt, thr, unit, total;
+  size_t d, bval, bidx, tval, tidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count, bmax, bcnt, thr, total;
 };
 
 Layout layout(int n, long long N, size_t elem) {
@@ -863,7 +825,6 @@ Layout layout(int n, long long N, size_t elem) {
   L.bmax = take(sizeof(long long) * nb);
   L.bcnt = take(sizeof(int) * nb);
   L.thr = take(sizeof(long long) * (n + 1));
-  L.unit = take(sizeof(int));
   L.total = off;
   return L;
 }
@@ -900,7 +861,7 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
   // column selection: n passes; the last block of each pass takes the pivot step
   SelArgs sa{bval, bidx, count, Ub, res->piv, res->dependent, 0, reinterpret_cast<long long *>(w + L.tval),
              reinterpret_cast<long long *>(w + L.tidx), reinterpret_cast<long long *>(w + L.bmax),
-             reinterpret_cast<int *>(w + L.bcnt), reinterpret_cast<long long *>(w + L.thr), reinterpret_cast<int *>(w + L.unit)};
+             reinterpret_cast<int *>(w + L.bcnt), reinterpret_cast<long long *>(w + L.thr)};
   constexpr bool kLazy = sizeof(T) == 4;  // FP32: block bounds, see scdm_step_kernel
   // one resident wave of blocks
   int dev = 0, sms = 0, per_sm = 0;
