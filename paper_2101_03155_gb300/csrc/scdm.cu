@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <cstdlib>
 
 #include "ace_internal.h"
 #include "residual_key.h"
@@ -84,6 +85,12 @@ struct SelArgs {
   long long *bmax;       // [blocks]
   int *bcnt;             // [blocks]
   long long *thr;        // [n + 1], from 0
+  // clock cycles: the longest CTA of the current pass, and by how much the last passes have cost more than
+  // passes over every point would have; then 0, or the step from which on every point is updated
+  int *work;
+  long long *excess;
+  int *left;
+  int full_cost, leave_cost, leave_step;
 };
 
 template <typename T>
@@ -314,7 +321,7 @@ struct Resid<float> {
 // choice of the pivots (U and Phi are computed from the pivots and Psi alone).  A column whose
 // residual is at the rounding level of T (|residual|^2 below kDependent(T) |psi(c_k)|^2) gives
 // u_k = 0 and sets *dependent.
-template <typename T>
+template <typename T, bool LAZY>
 __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr, int n, long long N, int nblk,
                            typename Resid<T>::type *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm,
                            float4 *stage) {
@@ -344,7 +351,7 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
   }
   __syncthreads();
   const long long cr = sm.chosen;
-  // FP32: the next step's threshold comes from the blocks with the largest bounds, one per warp from its
+  // LAZY: the next step's threshold comes from the blocks with the largest bounds, one per warp from its
   // share of the CTAs, brought up to date with u_k at the end of this step.  Away from c_k bounds near the
   // top hardly change, so one of these is the next pivot's block, or close to it in value.  Their points are
   // loaded here, ahead of the basis vector.
@@ -352,7 +359,7 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
   int slim = 0, sj = 0;
   long long seed_d = -1;
   float sv[32];
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (LAZY) {
     if (k + 1 < n) {
       long long tb = kNone, tbi = N;
       for (int b = warp + kWarps * lane; b < nblk; b += kWarps * 32) amax(tb, tbi, __ldcg(s.tval + b), __ldcg(s.tidx + b));
@@ -457,7 +464,7 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
   const T inv = c[0];
   T *Uw = static_cast<T *>(s.Ub);
   for (int i = tid; i < ldu; i += kUpdNT) Uw[(long long)k * ldu + i] = i < n ? u[i] * inv : (T)0;
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (LAZY) {
     if (k + 1 < n) {
       __threadfence();
       __syncthreads();  // u_k for the CTA, in L2
@@ -471,14 +478,14 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
 
 // End of a pass for one block: publish the block maximum; the last block to publish takes the
 // pivot step and resets the counter for the next pass (true for that block).  Orbital i at point r is psi[i si + r sr].
-template <typename T>
-__device__ bool finish_pass(long long best, long long bi, long long top, long long ti, const T *__restrict__ psi, long long si, long long sr, int n,
-                            long long N, typename Resid<T>::type *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm,
-                           float4 *stage) {
+template <typename T, bool LAZY>
+__device__ bool finish_pass(long long best, long long bi, long long top, long long ti, long long start,
+                            const T *__restrict__ psi, long long si, long long sr, int n, long long N,
+                            typename Resid<T>::type *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm, float4 *stage) {
   const int tid = threadIdx.x;
   constexpr int kWarps = kUpdNT / 32;
   warp_amax(best, bi);
-  if constexpr (sizeof(T) == 4) warp_amax(top, ti);
+  if constexpr (LAZY) warp_amax(top, ti);
   if ((tid & 31) == 0) {
     sm.rk[tid >> 5] = best;
     sm.ri[tid >> 5] = bi;
@@ -490,7 +497,7 @@ __device__ bool finish_pass(long long best, long long bi, long long top, long lo
     best = tid < kWarps ? sm.rk[tid] : kNone;
     bi = tid < kWarps ? sm.ri[tid] : N;
     warp_amax(best, bi);
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (LAZY) {
       top = tid < kWarps ? sm.tk[tid] : kNone;
       ti = tid < kWarps ? sm.ti[tid] : N;
       warp_amax(top, ti);
@@ -498,6 +505,7 @@ __device__ bool finish_pass(long long best, long long bi, long long top, long lo
         s.tval[blockIdx.x] = top;
         s.tidx[blockIdx.x] = ti;
         sm.top = ti;
+        if (s.k > 0) atomicMax(s.work, (int)min(clock64() - start, 1LL << 30));
       }
     }
     if (tid == 0) {
@@ -510,8 +518,17 @@ __device__ bool finish_pass(long long best, long long bi, long long top, long lo
   __syncthreads();
   if (!sm.last) return false;
   __threadfence();
-  pivot_step<T>(psi, si, sr, n, N, gridDim.x, d, s, sm, stage);
-  if (tid == 0) *s.count = 0u;
+  pivot_step<T, LAZY>(psi, si, sr, n, N, gridDim.x, d, s, sm, stage);
+  if (tid == 0) {
+    *s.count = 0u;
+    if constexpr (LAZY) {
+      if (s.k > 0) {
+        *s.excess = max(0ll, *s.excess + __ldcg(s.work) - s.full_cost);
+        *s.work = 0;
+        if (*s.excess > s.leave_cost || s.k == s.leave_step) *s.left = s.k + 1;
+      }
+    }
+  }
   return true;
 }
 
@@ -547,20 +564,25 @@ __global__ void __launch_bounds__(kUpdNT) scdm_pass_kernel(const T *__restrict__
     }
     amax(best, bi, res_key(dr), r);
   }
-  finish_pass<T>(best, bi, kNone, N, psi, N, 1, n, N, d, s, sm, nullptr);
+  finish_pass<T, false>(best, bi, kNone, N, 0, psi, N, 1, n, N, d, s, sm, nullptr);
 }
 
 // The FP32 selection.  The residual norms only fall from step to step, so the residual a point had when
 // it was last brought up to date bounds its present one: a step has to look only at the blocks whose
 // bound reaches the largest up-to-date residual.  For 128 orbitals on 96^3 that is 27,000 block visits in
 // all 128 steps, a quarter of the blocks once, where passes over every point (the plain greedy selection)
-// read Psi 128 times: 11.4 ms per call, bound by HBM at 0.8 of its bandwidth; now 5.0 ms, of which the
-// chain of the 127 steps (launch, look at the bounds, visits, pivot step: about 30 us each) is 3.9 ms.
-//   Every residual goes through the same operations in the same order as when all points are updated in
-// every step, so the pivots are the same.
+// read Psi 128 times: 12.3 ms per call, bound by HBM at 0.8 of its bandwidth; now 4.9 ms, most of it the
+// chain of the 127 steps (launch, look at the bounds, visits, pivot step: about 30 us each).
+//   Orbitals that no rotation localises (plane waves of a metal) flatten the residuals, and the visits of a step
+// then cost more than a pass over every point: the steps measure themselves, and when the last ones have lost
+// about what changing over costs, the rest are passes over every point.  64 such orbitals on 72^3: 5.8 ms on
+// bounds alone, 3.4 with passes alone, 3.8 with the change; 200 on 64^3: 30, 13.4 and 14.2 ms.
+//   Every residual goes through the same operations in the same order in all of these, so the pivots are the
+// same whichever way a step goes.
 
 // d[r] = |psi(r)|^2 (FP32), one point per thread; the sum has the order of refresh_block's (32 partial sums over
 // orbitals 4 l .. 4 l + 3 (+ 128 f), then the pairwise tree).
+template <bool LAZY>
 __global__ void __launch_bounds__(kUpdNT) scdm_norm_kernel(const float *__restrict__ psi, int n, long long N,
                                                            long long *__restrict__ d, SelArgs s) {
   __shared__ __align__(16) ScdmSmem<float> sm;
@@ -600,12 +622,143 @@ __global__ void __launch_bounds__(kUpdNT) scdm_norm_kernel(const float *__restri
       d[r] = dr;
       amax(best, bi, dr, r);
     }
-    if (r < N && r % kBlk == 0) {
+    if (LAZY && r < N && r % kBlk == 0) {
       s.bmax[r / kBlk] = mx;
       s.bcnt[r / kBlk] = 0;
     }
   }
-  finish_pass<float>(best, bi, best, bi < N ? bi / kBlk : N, psi, N, 1, n, N, d, s, sm, stage_all);
+  finish_pass<float, LAZY>(best, bi, best, bi < N ? bi / kBlk : N, 0, psi, N, 1, n, N, d, s, sm, stage_all);
+}
+
+// Few points (see launch_scdm): step k >= 1 over every point, one per thread.  u_{k-1} . psi(r) is summed in the order
+// of refresh_block's.
+__global__ void __launch_bounds__(kUpdNT) scdm_full_kernel(const float *__restrict__ psi, int n, long long N,
+                                                           long long *__restrict__ d, SelArgs s) {
+  __shared__ __align__(16) ScdmSmem<float> sm;
+  const int tid = threadIdx.x, nf = (n + 3) / 4;
+  for (int i = tid; i < (nf + 31) / 32 * 128; i += kUpdNT)
+    sm.us[i] = i < 4 * nf ? static_cast<const float *>(s.Ub)[(long long)(s.k - 1) * (4 * nf) + i] : 0.f;
+  __syncthreads();
+  const float4 *u4 = reinterpret_cast<const float4 *>(sm.us);
+  long long best = kNone, bi = N;
+  for (long long r = blockIdx.x * (long long)kUpdNT + tid; r < N; r += (long long)gridDim.x * kUpdNT) {
+    float acc[32];
+#pragma unroll
+    for (int l = 0; l < 32; ++l) acc[l] = 0.f;
+    for (int f0 = 0; f0 < nf; f0 += 32) {
+#pragma unroll
+      for (int l8 = 0; l8 < 32; l8 += 8) {
+        if (f0 + l8 >= nf) break;
+#pragma unroll
+        for (int l = l8; l < l8 + 8; ++l) {
+          float x[4];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const int i = 4 * (f0 + l) + t;
+            x[t] = i < n ? __ldg(psi + (long long)i * N + r) : 0.f;
+          }
+          acc[l] += dot4(u4[f0 + l], make_float4(x[0], x[1], x[2], x[3]));
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int l = 0; l < o; ++l) acc[l] += acc[l + o];
+    const long long dr = key_downdate(d[r], __float_as_uint(acc[0]));
+    d[r] = dr;
+    amax(best, bi, dr, r);
+  }
+  finish_pass<float, false>(best, bi, kNone, N, 0, psi, N, 1, n, N, d, s, sm, nullptr);
+}
+
+// Point-major copy pt[r][i] = psi[i][r] for i < n, zero for n <= i < ld: 32 points x 32 orbitals per block.
+__global__ void scdm_points_copy_kernel(const float *__restrict__ psi, int n, long long N, int ld, float *__restrict__ pt) {
+  __shared__ float tile[32][33];
+  const long long r0 = blockIdx.x * 32ll;
+  const int i0 = blockIdx.y * 32;
+  for (int y = threadIdx.y; y < 32; y += 8) {
+    const int i = i0 + y;
+    tile[y][threadIdx.x] = i < n && r0 + threadIdx.x < N ? psi[(long long)i * N + r0 + threadIdx.x] : 0.f;
+  }
+  __syncthreads();
+  for (int y = threadIdx.y; y < 32; y += 8)
+    if (r0 + y < N && i0 + threadIdx.x < ld) pt[(r0 + y) * ld + i0 + threadIdx.x] = tile[threadIdx.x][y];
+}
+
+// Every block up to date with u_0 .. u_{k-2}.
+__global__ void __launch_bounds__(kUpdNT, 2) scdm_catch_up_kernel(const float *__restrict__ psi, int n, long long N,
+                                                                  long long *__restrict__ d, SelArgs s) {
+  extern __shared__ float4 stage_all[];  // kStage per warp
+  const long long nb = (N + kBlk - 1) / kBlk, nwarps = (long long)gridDim.x * (kUpdNT / 32);
+  long long best = kNone, bi = N;
+  for (long long b = (long long)blockIdx.x * (kUpdNT / 32) + (threadIdx.x >> 5); b < nb; b += nwarps)
+    if (s.bcnt[b] < s.k - 1)
+      refresh_block(psi, n, N, d, s, b, s.k, s.k - 1, false, stage_all + (threadIdx.x >> 5) * kStage, best, bi);
+}
+
+// Step k >= 1 over every point, from the point-major copy pt.  Every warp takes an equal share of the blocks, 32
+// points at a time in four blocks: lane l loads the float4 of orbitals 4 l .. 4 l + 3 (+ 128 f) of a block's points
+// (whole rows; 128-byte pieces of 128 rows of Psi run at 2.1 TB/s), the lanes' sums are added by refresh_block's
+// pairwise tree, and lane l keeps point l of the 32.  In the first such step (FIRST) the blocks that the last
+// pivot step looked at have u_{k-1} already.
+template <bool FIRST>
+__global__ void __launch_bounds__(kUpdNT, 3) scdm_points_kernel(const float *__restrict__ psi, const float *__restrict__ pt,
+                                                                int n, long long N, long long *__restrict__ d, SelArgs s) {
+  __shared__ __align__(16) ScdmSmem<float> sm;
+  const int tid = threadIdx.x, lane = tid & 31, nf = (n + 3) / 4, k = s.k;
+  const unsigned full = 0xffffffffu;
+  const float4 *ub = static_cast<const float4 *>(s.Ub), *pt4 = reinterpret_cast<const float4 *>(pt);
+  for (int i = tid; i < nf; i += kUpdNT) reinterpret_cast<float4 *>(sm.us)[i] = ub[(long long)(k - 1) * nf + i];
+  __syncthreads();
+  const float4 *us = reinterpret_cast<const float4 *>(sm.us);
+  const long long nb = (N + kBlk - 1) / kBlk, nwarps = (long long)gridDim.x * (kUpdNT / 32);
+  const long long w = (long long)blockIdx.x * (kUpdNT / 32) + (tid >> 5);
+  const long long ra = nb * w / nwarps * kBlk, rb = min(N, nb * (w + 1) / nwarps * kBlk);
+  long long best = kNone, bi = N;
+  for (long long r0 = ra; r0 < rb; r0 += 32) {
+    const long long r = r0 + lane;
+    long long dr = r < rb ? d[r] : -1;
+    const bool done = FIRST && r < rb && s.bcnt[r / kBlk] == k;
+    float mine = 0.f;
+#pragma unroll 1
+    for (int grp = 0; grp < 4; ++grp) {
+      const long long rg = r0 + kBlk * grp;
+      float acc[kBlk] = {};
+#pragma unroll 1
+      for (int f0 = 0; f0 < nf; f0 += 32) {
+        const int f = f0 + lane, lim = f < nf ? (int)min((long long)kBlk, rb - rg) : 0;
+        const float4 uu = f < nf ? us[f] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 *base = pt4 + rg * nf + f;
+        float4 v[kBlk];
+#pragma unroll
+        for (int p = 0; p < kBlk; ++p) v[p] = p < lim ? __ldcs(base + p * nf) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int p = 0; p < kBlk; ++p) acc[p] += dot4(uu, v[p]);
+      }
+#pragma unroll
+      for (int p = 0; p < kBlk; ++p) {
+        acc[p] += __shfl_xor_sync(full, acc[p], 16);
+        acc[p] += __shfl_xor_sync(full, acc[p], 8);
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int p = 0; p < o; ++p) {
+          const float send = up ? acc[p] : acc[p + o], keep = up ? acc[p + o] : acc[p];
+          acc[p] = keep + __shfl_xor_sync(full, send, o);
+        }
+      }
+      if ((lane >> 3) == grp) mine = acc[0];
+    }
+    if (!done) dr = key_downdate(dr, __float_as_uint(mine));
+    if (r < rb) {
+      d[r] = dr;
+      amax(best, bi, dr, r);
+    }
+  }
+  finish_pass<float, false>(best, bi, kNone, N, 0, psi, N, 1, n, N, d, s, sm, nullptr);
 }
 
 // Step k >= 1: the warps look through the blocks' bounds, 32 at a time (neighbouring blocks belong to
@@ -623,12 +776,13 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
   float4 *stage = stage_all + (threadIdx.x >> 5) * kStage;
   const int lane = threadIdx.x & 31;
   const unsigned full = 0xffffffffu;
-  const long long nb = (N + kBlk - 1) / kBlk;
+  const long long start = clock64(), nb = (N + kBlk - 1) / kBlk;
   const long long nwarps = (long long)gridDim.x * (kUpdNT / 32);
   const long long w = (long long)blockIdx.x * (kUpdNT / 32) + (threadIdx.x >> 5);
   long long thr = __ldcg(s.thr + s.k);
   const long long soon = key_somewhat_below(thr);
   long long best = kNone, bi = N, top = kNone, ti = N;
+  if (*s.left) return;
   for (long long b0 = w; b0 < nb; b0 += 32 * nwarps) {
     const long long b = b0 + lane * nwarps;
     long long bound = b < nb ? s.bmax[b] : kNone;
@@ -645,7 +799,7 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
     }
     amax(top, ti, bound, b);
   }
-  if (finish_pass<float>(best, bi, top, ti, psi, N, 1, n, N, d, s, sm, stage_all)) return;
+  if (finish_pass<float, true>(best, bi, top, ti, start, psi, N, 1, n, N, d, s, sm, stage_all)) return;
   int most = kAheadMost;
   for (long long b0 = w; b0 < nb && most > 0; b0 += 32 * nwarps) {
     const long long b = b0 + lane * nwarps;
@@ -788,7 +942,7 @@ __global__ void scdm_factor_kernel(const double *__restrict__ M, const double *_
 }
 
 struct Layout {
-  size_t d, bval, bidx, tval, tidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count, bmax, bcnt, thr, total;
+  size_t d, bval, bidx, tval, tidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count, bmax, bcnt, thr, work, excess, left, total;
 };
 
 Layout layout(int n, long long N, size_t elem) {
@@ -825,6 +979,9 @@ Layout layout(int n, long long N, size_t elem) {
   L.bmax = take(sizeof(long long) * nb);
   L.bcnt = take(sizeof(int) * nb);
   L.thr = take(sizeof(long long) * (n + 1));
+  L.work = take(sizeof(int));
+  L.excess = take(sizeof(long long));
+  L.left = take(sizeof(int));
   L.total = off;
   return L;
 }
@@ -832,6 +989,11 @@ Layout layout(int n, long long N, size_t elem) {
 }  // namespace
 
 int scdm_max_iterations() { return kNsMax; }
+
+static int env_value(const char *name, int dflt) {
+  const char *v = std::getenv(name);
+  return v && *v ? std::atoi(v) : dflt;
+}
 
 size_t scdm_workspace_bytes(int n, long long N, size_t elem) { return layout(n, N, elem).total; }
 
@@ -861,46 +1023,86 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
   // column selection: n passes; the last block of each pass takes the pivot step
   SelArgs sa{bval, bidx, count, Ub, res->piv, res->dependent, 0, reinterpret_cast<long long *>(w + L.tval),
              reinterpret_cast<long long *>(w + L.tidx), reinterpret_cast<long long *>(w + L.bmax),
-             reinterpret_cast<int *>(w + L.bcnt), reinterpret_cast<long long *>(w + L.thr)};
-  constexpr bool kLazy = sizeof(T) == 4;  // FP32: block bounds, see scdm_step_kernel
-  // one resident wave of blocks
-  int dev = 0, sms = 0, per_sm = 0;
+             reinterpret_cast<int *>(w + L.bcnt), reinterpret_cast<long long *>(w + L.thr),
+             reinterpret_cast<int *>(w + L.work), reinterpret_cast<long long *>(w + L.excess),
+             reinterpret_cast<int *>(w + L.left), 0, 0, 0};
+  int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) {
-    if constexpr (kLazy) {
-      // shared memory above 48 KB, asked for once per call (a driver call of a microsecond)
-      e = cudaFuncSetAttribute(scdm_norm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(scdm_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
-      if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scdm_norm_kernel, kUpdNT, kStageBytes);
-    } else
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, scdm_pass_kernel<T, false>, kUpdNT, 0);
-  }
+  if (e == cudaSuccess) e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st);
   if (e != cudaSuccess) return e;
-  auto blocks = [&](int per, long long most) {
-    return (unsigned)std::max<long long>(1, std::min({(long long)std::max(per, 1) * sms, (long long)kUpdBlocks, most}));
+  // at most one resident wave of blocks, with at least `least` points each
+  auto blocks = [&](auto kernel, size_t smem, long long least, unsigned *grid) {
+    int per_sm = 0;
+    // shared memory above 48 KB, asked for once per call (a driver call of a microsecond)
+    cudaError_t q = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+    if (q == cudaSuccess) q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kUpdNT, smem);
+    *grid = (unsigned)std::max<long long>(1, std::min({(long long)std::max(per_sm, 1) * sms, (long long)kUpdBlocks,
+                                                       (N + least - 1) / least}));
+    return q;
   };
-  const unsigned grid = blocks(per_sm, (N + 255) / 256);
-  e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(sa.thr, 0, sizeof(long long) * (n + 1), st);
-  if (e != cudaSuccess) return e;
-  for (int k = 0; k < n; ++k) {
-    sa.k = k;
-    if constexpr (kLazy) {
-      const unsigned steps = blocks(2, (N + kBlk * kUpdNT - 1) / (kBlk * kUpdNT));  // a block per lane
-      if (k == 0)
-        scdm_norm_kernel<<<grid, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
-      else
-        scdm_step_kernel<<<steps, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
-    } else {
-      if (k == 0)
-        scdm_pass_kernel<T, true><<<grid, kUpdNT, 0, st>>>(psi, n, N, d, sa);
-      else
-        scdm_pass_kernel<T, false><<<grid, kUpdNT, 0, st>>>(psi, n, N, d, sa);
+  unsigned first = 1, next = 1;
+  auto steps = [&](auto kernel, size_t smem, int k0, int k1) {
+    for (sa.k = k0; sa.k < k1; ++sa.k) kernel<<<next, kUpdNT, smem, st>>>(psi, n, N, d, sa);
+    return cudaGetLastError();
+  };
+  if constexpr (sizeof(T) == 8) {
+    e = blocks(scdm_pass_kernel<T, true>, 0, kUpdNT, &first);
+    if (e == cudaSuccess) e = blocks(scdm_pass_kernel<T, false>, 0, kUpdNT, &next);
+    if (e != cudaSuccess) return e;
+    scdm_pass_kernel<T, true><<<first, kUpdNT, 0, st>>>(psi, n, N, d, sa);
+    e = steps(scdm_pass_kernel<T, false>, 0, 1, n);
+  } else if (4.0 * n * N < 1e6 * env_value("ACE_SCDM_BOUNDS_MB", 70)) {
+    // Psi stays in L2 and a pass over every point is cheaper than the bounds (ms per call, with them / without:
+    // 64 orbitals on 48^3 1.94 / 1.64, on 64^3 2.14 / 2.11; 32 on 64^3 1.35 / 1.10; on 72^3 64 take 2.2 / 3.2)
+    e = blocks(scdm_norm_kernel<false>, 0, kUpdNT, &first);
+    if (e == cudaSuccess) e = blocks(scdm_full_kernel, 0, kUpdNT, &next);
+    if (e != cudaSuccess) return e;
+    scdm_norm_kernel<false><<<first, kUpdNT, 0, st>>>(psi, n, N, d, sa);
+    e = steps(scdm_full_kernel, 0, 1, n);
+  } else {
+    // a pass over every point reads Psi at about 6.5 TB/s (at 1.9 GHz); leaving takes the point-major copy, the
+    // vectors that the blocks miss, about three passes' time
+    sa.full_cost = (int)std::min(5e8, 4.0 * n * N / 3400.0);
+    sa.leave_cost = 3 * sa.full_cost + 114000;
+    sa.leave_step = env_value("ACE_SCDM_LEAVE_STEP", 0);
+    // thresholds, clocks and the step of leaving (neighbours in the workspace)
+    e = cudaMemsetAsync(sa.thr, 0, L.total - L.thr, st);
+    if (e == cudaSuccess) e = blocks(scdm_norm_kernel<true>, kStageBytes, kUpdNT, &first);
+    if (e == cudaSuccess) e = blocks(scdm_catch_up_kernel, kStageBytes, kUpdNT, &next);
+    if (e == cudaSuccess) e = blocks(scdm_step_kernel, kStageBytes, kBlk * kUpdNT, &next);  // a block per lane
+    if (e != cudaSuccess) return e;
+    scdm_norm_kernel<true><<<first, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
+    // the host looks every 64 steps whether the steps over bounds were left (each look idles the device for
+    // about 15 us, a step that returns at once takes 2.5)
+    int left = 0;
+    for (int k = 1; k < n && left == 0; k += 64) {
+      e = steps(scdm_step_kernel, kStageBytes, k, std::min(n, k + 64));
+      if (e == cudaSuccess) e = cudaMemcpyAsync(&left, sa.left, sizeof(int), cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e != cudaSuccess) return e;
+    }
+    if (left > 0 && left < n) {
+      const int ld = basis_ld<float>(n);
+      float *pt = nullptr;
+      e = cudaMallocAsync(&pt, sizeof(float) * (size_t)N * ld, st);
+      if (e != cudaSuccess) return e;
+      scdm_points_copy_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)((ld + 31) / 32)), dim3(32, 8), 0, st>>>(psi, n, N, ld, pt);
+      sa.k = left;
+      scdm_catch_up_kernel<<<next, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
+      *launches += 2;
+      e = blocks(scdm_points_kernel<false>, 0, kUpdNT, &next);
+      for (sa.k = left; sa.k < n && e == cudaSuccess; ++sa.k) {
+        if (sa.k == left)
+          scdm_points_kernel<true><<<next, kUpdNT, 0, st>>>(psi, pt, n, N, d, sa);
+        else
+          scdm_points_kernel<false><<<next, kUpdNT, 0, st>>>(psi, pt, n, N, d, sa);
+        e = cudaGetLastError();
+      }
+      cudaFreeAsync(pt, st);
     }
   }
+  if (e != cudaSuccess) return e;
   *launches += n;
   // Loewdin factor.  The n x n FP64 products run as one output per thread in 64-thread blocks, so
   // that they spread over most SMs (FP64 throughput per SM is low).
