@@ -1066,26 +1066,39 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
 // per value walked up to 152 loads, 17-22 us at every size; now 4-8 us.)
 constexpr int SR_NT = 512;
 // G (nx x ny) = scale * sum over the splits of partial[s], pairs (sum, compensation) column by column;
-// with `accumulate` the sum is added to G instead.  Each of the 16 slices adds its splits as an FP32
-// pair with exact two-sums (about 48 bits; FP32 instructions where FP64 ones would bound the kernel),
-// the slices are added in FP64 in a fixed order.
+// with `accumulate` the sum is added to G instead.  Each of the 16 slices adds its splits as three FP32 numbers
+// with exact two-sums, of which only the third is rounded (2^-70 of the sum; an FP64 sum rounds to 2^-53 at
+// every addition, and its instructions and conversions would bound the kernel); the slices are added in FP64
+// in a fixed order.
 __global__ void __launch_bounds__(SR_NT) gram_splits_reduce_kernel(const float2 *__restrict__ partial, int splits,
                                                                    int nx, int ny, double scale, bool accumulate,
                                                                    double *__restrict__ G) {
   __shared__ double part[SR_NT / 32][33];
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane, ne = nx * ny;
-  float s = 0.f, c = 0.f;
+  // a += x; returns what the rounded sum leaves out, exactly
+  auto two_sum = [](float &a, float x) {
+    const float t = a + x, b = t - a, r = (a - (t - b)) + (x - b);
+    a = t;
+    return r;
+  };
+  float s = 0.f, c = 0.f, d = 0.f;
   if (e < ne) {
 #pragma unroll 10
     for (int k = slice; k < splits; k += SR_NT / 32) {
       const float2 v = partial[(long long)k * ne + e];
-      const float t = s + v.x, b = t - s;
-      c += ((s - (t - b)) + (v.x - b)) - v.y;
-      s = t;
+      d += two_sum(c, two_sum(s, v.x)) + two_sum(c, -v.y);
     }
   }
-  part[slice][lane] = (double)s + (double)c;
+  double own = (double)s + ((double)c + (double)d);
+  if (!(fabsf(s) < __int_as_float(0x7f800000)) && e < ne) {  // the FP32 sum left the range, or a partial is not finite
+    own = 0.0;
+    for (int k = slice; k < splits; k += SR_NT / 32) {
+      const float2 v = partial[(long long)k * ne + e];
+      own += (double)v.x - (double)v.y;
+    }
+  }
+  part[slice][lane] = own;
   __syncthreads();
   if (slice != 0 || e >= ne) return;
   double r = 0.0;
