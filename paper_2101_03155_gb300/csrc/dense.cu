@@ -1599,7 +1599,10 @@ __global__ void __launch_bounds__(CHS_NT) cholesky_small_kernel(const double *__
         if (tid == 0) *status = 1000000 + j;
         return;
       }
-      const double t = i > j ? c[i] * __drcp_rn(d) : 0.0;
+      // a division would cost the chain 1 us per column more (the reciprocal and the product round twice, as
+      // scaling by rsqrt does in the cluster form); it is taken where the reciprocal is not a normal number
+      const int dh = __double2hiint(d);
+      const double t = i > j ? (dh >= 0x00200000 && dh < 0x7fd00000 ? c[i] * __drcp_rn(d) : c[i] / d) : 0.0;
       bool first = w == ((j + 1) & (CHS_W - 1));  // owner of column j + 1, not published yet
 #pragma unroll
       for (int s = jb; s < CHS_S; ++s) {
