@@ -198,8 +198,8 @@ cudaError_t get_tables(int dev, const ace_desc &d, cudaStream_t st, const Device
   std::vector<T> Kp(Kt.size());
   {
     int a2, b2, a3, b3;
-    ace::axis_factors(d.n[1], &a2, &b2);
-    ace::axis_factors(d.n[2], &a3, &b3);
+    ace::axis_factors<T>(d.n[1], &a2, &b2);
+    ace::axis_factors<T>(d.n[2], &a3, &b3);
     const int n2 = d.n[1], n3 = d.n[2];
     for (int m1 = 0; m1 < d.n[0]; ++m1)
       for (int p2 = 0; p2 < n2; ++p2) {

@@ -152,6 +152,7 @@ bool pass_length_supported(int L);
 bool conv_length_supported(int L);
 // Two-stage factorisation L = r1 * r2 of a compiled axis length (output index k sits at
 // position (k % r1) * r2 + k / r1 after a forward transform).
+template <typename T>
 bool axis_factors(int L, int *r1, int *r2);
 
 // Dense steps.

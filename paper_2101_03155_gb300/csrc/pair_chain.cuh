@@ -35,8 +35,8 @@ namespace ace {
 // shared memory (FP64 beyond about 190 points).
 template <typename T, int L>
 struct PassShape {
-  static constexpr int R1 = Factor<L>::R1;
-  static constexpr int R2 = Factor<L>::R2;
+  static constexpr int R1 = FactorOf<L, T>::R1;
+  static constexpr int R2 = FactorOf<L, T>::R2;
   static constexpr int TILE = (16LL * (L + 1) + L) * (long long)sizeof(cpx<T>) <= 48LL * 1024 ? 16 : 8;
   static constexpr int LP = L + 1;  // odd pitch: lanes over lines hit distinct banks
   static constexpr int NT = TILE * (R1 > R2 ? R1 : R2);
@@ -87,9 +87,9 @@ __device__ __forceinline__ void pencil_stage2(cpx<T> *s, int tvalid) {
   }
 }
 
-template <int L>
+template <typename T, int L>
 __device__ __forceinline__ int perm_pos(int k) {
-  return (k % Factor<L>::R1) * Factor<L>::R2 + k / Factor<L>::R1;
+  return (k % FactorOf<L, T>::R1) * FactorOf<L, T>::R2 + k / FactorOf<L, T>::R1;
 }
 
 template <typename T, int L, int MODE>
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__((PassShape<T, L>::NT)) pair_pass_kernel(PairPa
     const bool diag1 = pk.x == pk.y, diag2 = pk.z == pk.w;
     for (int e = tid; e < tvalid * L; e += NT) {
       const int t = e / L, k = e - t * L;
-      const cpx<T> v = s[t * LP + perm_pos<L>(k)];
+      const cpx<T> v = s[t * LP + perm_pos<T, L>(k)];
       atomicAdd(a.W + oa + e, v.x * a.phi[ob + e]);
       if (!diag1) atomicAdd(a.W + ob + e, v.x * a.phi[oa + e]);
       if (two) {
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__((PassShape<T, L>::NT)) pair_pass_kernel(PairPa
     cpx<T> *dst = z + base;
     for (int e = tid; e < tvalid * L; e += NT) {
       const int t = e / L, k = e - t * L;
-      dst[e] = s[t * LP + perm_pos<L>(k)];
+      dst[e] = s[t * LP + perm_pos<T, L>(k)];
     }
   } else if (MODE == PASS_CONV1) {
     cpx<T> *dst = z + base;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__((PassShape<T, L>::NT)) pair_pass_kernel(PairPa
     cpx<T> *dst = z + base;
     for (int e = tid; e < TILE * L; e += NT) {
       const int k = e / TILE, t = e - k * TILE;
-      if (t < tvalid) dst[(long long)k * Ns + t] = s[t * LP + perm_pos<L>(k)];
+      if (t < tvalid) dst[(long long)k * Ns + t] = s[t * LP + perm_pos<T, L>(k)];
     }
   }
 }
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__((PassShape<T, L>::NT)) pair_pass_kernel(PairPa
 // ---------------------------------------------------------------------------------------
 template <int L>
 struct ConvShape {
-  static constexpr int R1 = Factor<L>::R1, R2 = Factor<L>::R2;
+  static constexpr int R1 = FactorOf<L, double>::R1, R2 = FactorOf<L, double>::R2;
   static constexpr int TILE = 32;  // columns per CTA (lanes over columns)
   static constexpr int LP = L + 1;
   // threads: 128 up to 108 points (more CTAs per SM), 256 for the longer pencils

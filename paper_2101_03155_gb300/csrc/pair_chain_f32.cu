@@ -20,12 +20,13 @@ cudaError_t launch_pair_pass<float>(int mode, const PairPassArgs<float> &a, int 
   return cudaErrorInvalidValue;
 }
 
+template <typename T>
 bool axis_factors(int L, int *r1, int *r2) {
   switch (L) {
-#define ACE_CASE(L_)        \
-  case L_:                  \
-    *r1 = Factor<L_>::R1;   \
-    *r2 = Factor<L_>::R2;   \
+#define ACE_CASE(L_)              \
+  case L_:                        \
+    *r1 = FactorOf<L_, T>::R1;    \
+    *r2 = FactorOf<L_, T>::R2;    \
     return true;
     ACE_PASS_LENGTHS(ACE_CASE)
 #undef ACE_CASE
@@ -33,6 +34,8 @@ bool axis_factors(int L, int *r1, int *r2) {
       return false;
   }
 }
+template bool axis_factors<float>(int, int *, int *);
+template bool axis_factors<double>(int, int *, int *);
 
 bool pass_length_supported(int L) {
   switch (L) {

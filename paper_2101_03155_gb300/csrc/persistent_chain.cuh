@@ -66,7 +66,7 @@ __device__ __forceinline__ void red_release_add(int *p, int v) {
 template <typename T, int L, int G, int NT>
 __device__ __forceinline__ void pencil_convolve(cpx<T> *z, const T *__restrict__ Kperm, int cols, int c0, cpx<T> *s,
                                                 const cpx<T> *tw) {
-  constexpr int LP = L + 1, R1 = Factor<L>::R1, R2 = Factor<L>::R2;
+  constexpr int LP = L + 1, R1 = FactorOf<L, T>::R1, R2 = FactorOf<L, T>::R2;
   const int gv = min(G, cols - c0);
   cpx<T> *zc = z + c0;
   // forward stage 1: tasks (t, n2): DFT_R1 over n1 of column t at i1 = n1 R2 + n2

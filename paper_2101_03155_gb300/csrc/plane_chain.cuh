@@ -46,8 +46,6 @@ constexpr int plane_min_blocks() {
 
 template <int N2, int N3>
 struct PlaneShape {
-  static constexpr int R1c = Factor<N2>::R1, R2c = Factor<N2>::R2;  // axis 2 (columns of the plane)
-  static constexpr int R1r = Factor<N3>::R1, R2r = Factor<N3>::R2;  // axis 3 (rows of the plane)
   static constexpr int PP = N3 + 1;                                  // odd pitch (complex elements)
   static constexpr int NPTS = N2 * N3;
   static_assert(N3 % 4 == 0, "rows are processed in groups of four points");
@@ -75,7 +73,7 @@ struct PlaneStages {
   //   tasks (l, n2): DFT_R1 over n1 of x[n1 R2 + n2]; optional twiddle w_L^{D n2 k1}; result k1 at k1 R2 + n2
   template <int L, int NL, int LS, int PS, int D, bool TW>
   static __device__ __forceinline__ void stage1(cpx<T> *s, const cpx<T> *tw) {
-    constexpr int R1 = Factor<L>::R1, R2 = Factor<L>::R2;
+    constexpr int R1 = FactorOf<L, T>::R1, R2 = FactorOf<L, T>::R2;
     for_tasks<NL, R2, NT>([&](int l, int n2) {
       cpx<T> *line = s + l * LS + n2 * PS;
       cpx<T> x[R1];
@@ -96,7 +94,7 @@ struct PlaneStages {
   // stage 2: tasks (l, k1): DFT_R2 of the contiguous block k1 R2 + n2; output k2 at k1 R2 + k2
   template <int L, int NL, int LS, int PS, int D>
   static __device__ __forceinline__ void stage2(cpx<T> *s) {
-    constexpr int R1 = Factor<L>::R1, R2 = Factor<L>::R2;
+    constexpr int R1 = FactorOf<L, T>::R1, R2 = FactorOf<L, T>::R2;
     for_tasks<NL, R1, NT>([&](int l, int k1) {
       cpx<T> *blk = s + l * LS + k1 * R2 * PS;
       cpx<T> x[R2];
@@ -112,7 +110,7 @@ struct PlaneStages {
   // the table's exact 1 + 0i, so every n2 > 0 term is multiplied without a branch on k1.
   template <int L, int NL, int LS, int PS>
   static __device__ __forceinline__ void inv_stageA(cpx<T> *s, const cpx<T> *tw) {
-    constexpr int R1 = Factor<L>::R1, R2 = Factor<L>::R2;
+    constexpr int R1 = FactorOf<L, T>::R1, R2 = FactorOf<L, T>::R2;
     for_tasks<NL, R1, NT>([&](int l, int k1) {
       cpx<T> *blk = s + l * LS + k1 * R2 * PS;
       cpx<T> x[R2];
@@ -236,13 +234,13 @@ __device__ __forceinline__ void plane_forward(const T *__restrict__ phi, long lo
   // axis 2 (columns): stage 1 in shared memory, stage 2 straight to the scratch plane
   F::template stage1<N2, N3, 1, S::PP, -1, true>(s, tw2);
   __syncthreads();
-  for_tasks<N3, S::R1c, NT>([&](int p3, int k1) {
-    cpx<T> x[S::R2c];
+  for_tasks<N3, FactorOf<N2, T>::R1, NT>([&](int p3, int k1) {
+    cpx<T> x[FactorOf<N2, T>::R2];
 #pragma unroll
-    for (int n2 = 0; n2 < S::R2c; ++n2) x[n2] = s[(k1 * S::R2c + n2) * S::PP + p3];
-    Dft<S::R2c, -1, T>::run(x);
+    for (int n2 = 0; n2 < FactorOf<N2, T>::R2; ++n2) x[n2] = s[(k1 * FactorOf<N2, T>::R2 + n2) * S::PP + p3];
+    Dft<FactorOf<N2, T>::R2, -1, T>::run(x);
 #pragma unroll
-    for (int k2 = 0; k2 < S::R2c; ++k2) dst[(k1 * S::R2c + k2) * N3 + p3] = x[k2];
+    for (int k2 = 0; k2 < FactorOf<N2, T>::R2; ++k2) dst[(k1 * FactorOf<N2, T>::R2 + k2) * N3 + p3] = x[k2];
   });
 }
 
@@ -266,21 +264,21 @@ template <typename T, int N2, int N3, int NT>
 __device__ __forceinline__ void plane_inverse(const cpx<T> *src, cpx<T> *s, const cpx<T> *tw2, const cpx<T> *tw3) {
   using S = PlaneShape<N2, N3>;
   using F = PlaneStages<T, NT>;
-  // axis 2 inverse, stage A straight from the scratch plane (permuted rows p2 = k1 R2c + k2);
+  // axis 2 inverse, stage A straight from the scratch plane (permuted rows p2 = k1 R2 + k2);
   // the k1 = 0 twiddles are the table's exact 1 + 0i
-  for_tasks<N3, S::R1c, NT>([&](int p3, int k1) {
-    cpx<T> x[S::R2c];
+  for_tasks<N3, FactorOf<N2, T>::R1, NT>([&](int p3, int k1) {
+    cpx<T> x[FactorOf<N2, T>::R2];
 #pragma unroll
-    for (int k2 = 0; k2 < S::R2c; ++k2) x[k2] = ldcg_cpx(src + (k1 * S::R2c + k2) * N3 + p3);
-    Dft<S::R2c, +1, T>::run(x);
+    for (int k2 = 0; k2 < FactorOf<N2, T>::R2; ++k2) x[k2] = ldcg_cpx(src + (k1 * FactorOf<N2, T>::R2 + k2) * N3 + p3);
+    Dft<FactorOf<N2, T>::R2, +1, T>::run(x);
 #pragma unroll
-    for (int n2 = 0; n2 < S::R2c; ++n2) {
+    for (int n2 = 0; n2 < FactorOf<N2, T>::R2; ++n2) {
       cpx<T> v = x[n2];
       if (n2 > 0) {
         const cpx<T> w = tw2[n2 * k1];
         v = cmul(v, cpx<T>{w.x, -w.y});
       }
-      s[(k1 * S::R2c + n2) * S::PP + p3] = v;
+      s[(k1 * FactorOf<N2, T>::R2 + n2) * S::PP + p3] = v;
     }
   });
   __syncthreads();
