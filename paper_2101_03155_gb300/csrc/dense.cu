@@ -24,12 +24,14 @@ namespace ace {
 
 // ----------------------------------------------------------------------------------------
 // General Gram (the FP64 form, and FP32 point counts off the 16-byte grid): BM x BM output tile per CTA
-// (BM 16 or 32), 16 x 16 threads with (BM / 16)^2 outputs each, one chunk of K per CTA.
-//   Bound by the FP64 pipe (2 multiply-adds per cycle and SM), so what counts is that no output of a tile
+// (BM 16 or 32, in FP32 also 64), 16 x 16 threads with (BM / 16)^2 outputs each, one chunk of K per CTA.
+//   FP64 is bound by its pipe (2 multiply-adds per cycle and SM), so what counts is that no output of a tile
 // is padding and that every SM has the same number of chunks: 64 x 64 tiles of 4096-point chunks left 12
 // orbitals at 28 times the work on 21 SMs (4.8 ms for 86,400 points), and 64 orbitals on 72^3 on 91 of
 // 152 SMs (5.3 ms).  Small tiles cost loads (each row is read once per tile of the other operand), which
-// stay below 2% of the FP64 time.
+// stay below 2% of the FP64 time.  FP32 is bound by its shared-memory loads, 2 BM / 16 for (BM / 16)^2
+// multiply-adds, and takes tiles of 64 where they add at most half as much again in padding: 128 orbitals on
+// 125^3 in tiles of 32 / 64: M 4.15 / 2.53 ms, screen 2.79 / 2.19 ms.
 // ----------------------------------------------------------------------------------------
 constexpr int GR_BK = 32, GR_NT = 256;
 constexpr long long GR_LONGEST = 1ll << 17;  // FP64 (FP32 sums go to FP64 every 4096 points)
@@ -38,11 +40,14 @@ struct GramPlan {
   int bm, nbx, tiles;
   long long chunk, chunks;
 };
-// Chunks of K, at most `longest` points, such that tiles x chunks CTAs spread evenly over the SMs (four to
+// Chunks of K, at most GR_LONGEST points (FP32: 4096), such that tiles x chunks CTAs spread evenly over the SMs (four to
 // sixteen per SM).
-static GramPlan gram_plan(int nx, int ny, long long K, bool upper_only, long long longest) {
+static GramPlan gram_plan(int nx, int ny, long long K, bool upper_only, bool fp64) {
+  const long long longest = fp64 ? GR_LONGEST : 4096;
+  auto padded = [](int n, int b) { return (double)((n + b - 1) / b * b); };
   GramPlan p;
   p.bm = nx <= 16 && ny <= 16 ? 16 : 32;
+  if (!fp64 && padded(nx, 64) * padded(ny, 64) <= 1.5 * padded(nx, 32) * padded(ny, 32)) p.bm = 64;
   p.nbx = (nx + p.bm - 1) / p.bm;
   const int nby = (ny + p.bm - 1) / p.bm;
   p.tiles = upper_only ? p.nbx * (p.nbx + 1) / 2 : p.nbx * nby;
@@ -194,8 +199,8 @@ __global__ void gram_chunks_reduce_kernel(const double *__restrict__ partial, lo
 }
 
 size_t gram_chunks_bytes(int nx, int ny, long long K) {
-  const long long c = std::max(gram_plan(nx, ny, K, false, GR_LONGEST).chunks,
-                               nx == ny ? gram_plan(nx, ny, K, true, GR_LONGEST).chunks : 0);
+  const long long c = std::max(gram_plan(nx, ny, K, false, true).chunks,
+                               nx == ny ? gram_plan(nx, ny, K, true, true).chunks : 0);
   return sizeof(double) * (size_t)c * nx * ny;
 }
 
@@ -513,7 +518,7 @@ cudaError_t launch_gram(const T *X, int nx, const T *Y, int ny, long long K, dou
       return cudaGetLastError();
     }
   }
-  const GramPlan p = gram_plan(nx, ny, K, upper_only, sizeof(T) == 4 ? 4096 : GR_LONGEST);
+  const GramPlan p = gram_plan(nx, ny, K, upper_only, sizeof(T) == 8);
   if (p.chunks > 65535) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(G, 0, sizeof(double) * (size_t)nx * ny, st);
   if (e != cudaSuccess) return e;
@@ -523,7 +528,9 @@ cudaError_t launch_gram(const T *X, int nx, const T *Y, int ny, long long K, dou
   };
   if (p.bm == 16)
     abs_values ? run(gram_kernel<T, true, 16>) : run(gram_kernel<T, false, 16>);
-  else
+  else if (p.bm == 64) {
+    if constexpr (sizeof(T) == 4) abs_values ? run(gram_kernel<T, true, 64>) : run(gram_kernel<T, false, 64>);
+  } else
     abs_values ? run(gram_kernel<T, true, 32>) : run(gram_kernel<T, false, 32>);
   e = cudaGetLastError();
   if (e != cudaSuccess || !partial) return e;
@@ -787,7 +794,10 @@ cudaError_t launch_skinny_left_mul(const float *A, int m, int n, const float *Y,
 // time: the launcher takes as few row blocks as tiles of 64 rows would need and the smallest R that
 // covers m with them (12 rows: a tile of 16, not 64; 70 rows: two of 48, not of 64).  With a lower
 // triangular A (m = n) a row block stops at its last diagonal element, and blocks are 16 rows: at 64 rows
-// that leaves 5/8 of the products.  Every output adds its terms in the same order whatever R is.
+// that leaves 5/8 of the products.  FP32 is bound by its shared-memory loads (R + 4 for 4 R multiply-adds) and
+// keeps the tall blocks for a triangular A too: 128 rows of 125^3 take 3.33 ms in blocks of 16 rows, 2.03 in
+// blocks of 64.
+// Every output adds its terms in the same order whatever R is.
 // xi in FP64: 12 rows of 40x45x48 149 -> 37 us, 64 rows of 72^3 2.49 -> 1.55 ms.
 // ----------------------------------------------------------------------------------------
 constexpr int LM_BN = 64, LM_BK = 16, LM_NT = 256, LM_RMAX = 4;
@@ -820,7 +830,7 @@ __global__ void __launch_bounds__(LM_NT) left_mul_kernel(const T *__restrict__ A
     __syncthreads();
 #pragma unroll
     for (int c = 0; c < LM_BK; ++c) {
-      if (l0 + c >= le) break;
+      if (sizeof(T) == 8 && l0 + c >= le) break;  // in FP32 the test costs more than the zeros
       T ar[R], yr[4];
 #pragma unroll
       for (int a = 0; a < R; ++a) ar[a] = as[c][ty + 16 * a];
@@ -845,7 +855,7 @@ __global__ void __launch_bounds__(LM_NT) left_mul_kernel(const T *__restrict__ A
 
 template <typename T>
 cudaError_t launch_left_mul(const T *A, int m, int n, const T *Y, long long K, T *Z, cudaStream_t st, bool lower) {
-  const int rmax = lower ? 1 : LM_RMAX;
+  const int rmax = lower && sizeof(T) == 8 ? 1 : LM_RMAX;
   const int blocks = (m + 16 * rmax - 1) / (16 * rmax), R = ((m + blocks - 1) / blocks + 15) / 16;
   const dim3 grid((unsigned)((K + LM_BN - 1) / LM_BN), (unsigned)blocks);
   auto run = [&](auto kernel) { kernel<<<grid, LM_NT, 0, st>>>(A, m, n, Y, K, Z, lower); };
