@@ -831,6 +831,16 @@ ace_status run_chain_persistent(ace_op *op, cudaStream_t st, const DeviceTables 
   return ACE_OK;
 }
 
+// Side streams and packs per batch of a chain within ACE_SCRATCH_MB of scratch (unset: dflt_mb, 0 for no
+// bound), one pack at least.
+void fit_scratch(size_t pack_bytes, int dflt_mb, int *nstreams, int *B) {
+  const int mb = env_int("ACE_SCRATCH_MB", dflt_mb);
+  if (mb <= 0) return;
+  const int slots = (int)std::min(65535.0, std::max(1.0, std::floor(mb * 1048576.0 / (double)pack_bytes)));
+  *nstreams = std::min(*nstreams, slots);
+  *B = std::min(*B, slots / *nstreams);
+}
+
 // Side streams of a chain on op's lane, forked from op->stream.
 ace_status fork_side(ace_op *op, int nstreams, cudaStream_t *side, cudaEvent_t *ev) {
   for (int k = 0; k < kSide; ++k) side[k] = op->stream;
@@ -850,9 +860,12 @@ ace_status run_chain_plane(ace_op *op, const float *phi, const DeviceTables *tab
   const ace_desc &d = op->desc;
   const long long N = op->N;
   cudaStream_t st = op->stream;
-  const int nstreams = std::min(kSide, std::max(1, cp.streams));
+  int nstreams = std::min(kSide, std::max(1, cp.streams));
   // few packs: smaller batches, so that every side stream has one
-  const int B = std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams));
+  int B = std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams));
+  // complex values of one pack in the scratch (16-byte units of two lines of axis 2)
+  const size_t pack_elems = (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2) * 2;
+  fit_scratch(sizeof(cpx<float>) * pack_elems, 0, &nstreams, &B);
   std::vector<int4> packs;
   form_packs(op->pairs_h, cp.RB, packs);
   void *tmp = nullptr;
@@ -860,8 +873,6 @@ ace_status run_chain_plane(ace_op *op, const float *phi, const DeviceTables *tab
   temps.push_back(tmp);
   int4 *packs_d = static_cast<int4 *>(tmp);
   ACE_CUDA(host_upload(op, packs_d, packs.data(), sizeof(int4) * packs.size(), st), "pack upload");
-  // complex values of one pack in the scratch (16-byte units of two lines of axis 2)
-  const size_t pack_elems = (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2) * 2;
   ACE_CUDA(cudaMallocAsync(&tmp, sizeof(cpx<float>) * pack_elems * B * nstreams, st), "alloc scratch");
   temps.push_back(tmp);
   cpx<float> *scratch_all = static_cast<cpx<float> *>(tmp);
