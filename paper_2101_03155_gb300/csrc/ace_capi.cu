@@ -955,15 +955,9 @@ ace_status run_chain_f64(ace_op *op, const double *phi, const DeviceTables *tab,
   cudaStream_t st = op->stream;
   int nstreams = std::min(kSide, std::max(1, cp.streams));
   int B = std::min(65535, std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams)));
-  // the pencil route keeps within ACE_SCRATCH_MB where it is set (one pack at least); W does not depend
-  // on the batches
-  const int budget_mb = pops ? 0 : env_int("ACE_SCRATCH_MB", 0);
-  if (budget_mb > 0) {
-    const double per = sizeof(cpx<double>) * (double)N;
-    const int slots = (int)std::min(65535.0, std::max(1.0, std::floor(budget_mb * 1048576.0 / per)));
-    nstreams = std::min(nstreams, slots);
-    B = std::min(B, slots / nstreams);
-  }
+  // the pencil route has a budget of 64 MB unless set (one pack at least; 16 orbitals on 160^3, one pack of 66 MB
+  // at a time, take 90 ms instead of 83); W does not depend on the batches
+  fit_scratch(sizeof(cpx<double>) * (size_t)N, pops ? 0 : 64, &nstreams, &B);
   std::vector<int4> packs;
   form_packs(op->pairs_h, cp.RB, packs);
   // only the side streams that get a batch: each of them is joined by its batches' events, and a stream

@@ -64,3 +64,21 @@ def test_budget_bounds_the_scratch(grid, prec, monkeypatch):
             assert torch.equal(W[mb], W[wide])
         else:
             assert rel_max(W[mb].cpu().numpy(), W[wide].cpu().numpy()) <= 2 * MIXED_W_RTOL
+
+
+@pytest.mark.parametrize("prec", [ace.ACE_MIXED, ace.ACE_FP64])
+def test_pencil_chain_has_64_mb_by_default(prec, monkeypatch):
+    """A grid of pencil passes whose pack takes 20 MB (mixed) or 40 MB: three packs or one at a time."""
+    import torch
+
+    monkeypatch.delenv("ACE_SCRATCH_MB", raising=False)
+    grid, n = (125, 125, 160), 4
+    fp64 = prec == ace.ACE_FP64
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    x = torch.rand((n,) + grid, generator=gen, device="cuda", dtype=torch.float64 if fp64 else torch.float32)
+    d = ace.make_desc(grid, np.diag([10.0, 10.0, 12.0]), n, prec=prec)
+    pairs = [(i, j) for i in range(n) for j in range(i, n)]
+    W, pool = torch.empty_like(x), _Pool()
+    abi.ace_exchange_w(d, x, pairs, W)
+    high = pool.high_of(lambda: abi.ace_exchange_w(d, x, pairs, W))
+    assert high <= x.numel() * x.element_size() + 64 * 2**20 + 4 * 2**20  # W, the scratch, small buffers
