@@ -294,16 +294,20 @@ ace_status ace_kernel_launches(const ace_op *op, long *launches);
 
 /* Autotuner of the pair chain; the paper has no counterpart (it is a property of this GPU code).
  * Screens `phi` as ace_build does, then times the pair chain on a sample of up to 480 of its packs
- * for each candidate setting of the stream-batched chain: packs per batch {1,2,3,4,6}, side streams
- * {2,4,8}, L2 set-aside for the scratch {0, 60 MB}, rows per block of the pack order {1,2,4,8};
- * then, on the best of those, the pencil tile of the axis-1 pass (FP32: 8 pairs of lines per warp in
+ * with the parameters that a build takes by the size of its grid, and for each candidate setting of the
+ * stream-batched chain: packs per batch {1,2,3,4,6} and half, once and twice what the size gives, side
+ * streams {2,4,8} (and 3 where the size gives 3), and, in the mixed form, L2 set-aside for the scratch
+ * {0, 60 MB} and rows per block of the pack order {1,2,4,8} (FP64 keeps the order, which decides the bits of
+ * W); then, on the best of those, the pencil tile of the axis-1 pass (FP32: 8 pairs of lines per warp in
  * blocks of two or four warps, or 4 pairs per warp); and the persistent chain (one launch walking the pack
  * list through a device task queue) with queue lags {2,3,4} where its grid is compiled.  The
- * fastest setting is kept for this grid and precision and used by later builds in the process;
+ * fastest setting is kept for this grid and precision and used by later builds in the process, the one by
+ * size where nothing beats it by 1%;
  * with the environment variable ACE_TUNE_FILE set, the table is also read from and written to that
  * file (one line per grid: n1 n2 n3 fp64 group batch streams l2_mb row_block persistent lag
  * pencil_tile; lines without the last field read as pencil tile 0).  params (optional, 7 ints)
  * receives {group, batch, streams, l2_mb, row_block, persistent lag or 0, pencil tile}.
+ * The packs per batch are the larger of group and batch (batch takes the listed values only).
  * Environment variables ACE_PLANE_BATCH, ACE_STREAMS, ACE_L2_PERSIST_MB, ACE_GROUP, ACE_ROW_BLOCK,
  * ACE_PERSISTENT, ACE_PERSIST_LAG, ACE_CONV_TILE override the table.  Grids without a plane-pass
  * plan keep the defaults.  Synchronous.  Errors as ace_build. */

@@ -513,7 +513,7 @@ bool find_plane_ops<double>(const ace_desc &d, ace::PlaneOps<double> *out) {
   return ace::conv_length_supported(d.n[0]) && ace::plane_ops_f64(d.n[1], d.n[2], out);
 }
 
-// Run-time parameters of the plane chain: packs per CTA group (G), packs per batch (B), side
+// Run-time parameters of the plane chain: packs per batch (the larger of G and B), side
 // streams, and the L2 set-aside for the scratch window (MB).  Defaults, or values found by
 // ace_autotune for the grid and precision; ACE_* environment variables override both.
 struct ChainParams {
@@ -578,7 +578,8 @@ void tune_store(const TuneKey &k, const ChainParams &c) {
   }
 }
 
-ChainParams chain_params(const ace_desc &d, bool fp64) {
+// Parameters by the size of the grid
+ChainParams size_params(const ace_desc &d, bool fp64) {
   ChainParams c;
   if (!fp64) {
     // Mixed form: packs per batch such that the scratch of all side streams takes about 60 MB (half
@@ -593,6 +594,11 @@ ChainParams chain_params(const ace_desc &d, bool fp64) {
     // GPU on small grids
     c.B = std::min(16, std::max(1, (int)std::lround(128e6 / (c.streams * 16.0 * d.n[0] * d.n[1] * d.n[2]))));
   }
+  return c;
+}
+
+ChainParams chain_params(const ace_desc &d, bool fp64) {
+  ChainParams c = size_params(d, fp64);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_file_load_locked();
@@ -600,8 +606,9 @@ ChainParams chain_params(const ace_desc &d, bool fp64) {
     for (const auto &e : g_tuned)
       if (e.first == k) c = e.second;
   }
-  c.G = std::max(1, env_int("ACE_GROUP", c.G));
-  c.B = std::max(c.G, env_int("ACE_PLANE_BATCH", c.B));
+  const int batch = env_int("ACE_PLANE_BATCH", 0);
+  c.G = std::max(1, env_int("ACE_GROUP", batch > 0 ? 1 : c.G));
+  c.B = std::max(c.G, batch > 0 ? batch : c.B);
   c.streams = std::min(kSide, std::max(1, env_int("ACE_STREAMS", c.streams)));
   c.persist_mb = std::max(0, env_int("ACE_L2_PERSIST_MB", c.persist_mb));
   c.RB = std::max(1, env_int("ACE_ROW_BLOCK", c.RB));
@@ -862,7 +869,7 @@ ace_status run_chain_plane(ace_op *op, const float *phi, const DeviceTables *tab
   cudaStream_t st = op->stream;
   int nstreams = std::min(kSide, std::max(1, cp.streams));
   // few packs: smaller batches, so that every side stream has one
-  int B = std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams));
+  int B = std::min(std::max(cp.G, cp.B), ((count + 1) / 2 + nstreams - 1) / nstreams);
   // complex values of one pack in the scratch (16-byte units of two lines of axis 2)
   const size_t pack_elems = (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2) * 2;
   fit_scratch(sizeof(cpx<float>) * pack_elems, 0, &nstreams, &B);
@@ -954,7 +961,7 @@ ace_status run_chain_f64(ace_op *op, const double *phi, const DeviceTables *tab,
   const long long N = op->N;
   cudaStream_t st = op->stream;
   int nstreams = std::min(kSide, std::max(1, cp.streams));
-  int B = std::min(65535, std::max(cp.G, std::min(cp.B, ((count + 1) / 2 + nstreams - 1) / nstreams)));
+  int B = std::min({65535, std::max(cp.G, cp.B), ((count + 1) / 2 + nstreams - 1) / nstreams});
   // the pencil route has a budget of 64 MB unless set (one pack at least; 16 orbitals on 160^3, one pack of 66 MB
   // at a time, take 90 ms instead of 83); W does not depend on the batches
   fit_scratch(sizeof(cpx<double>) * (size_t)N, pops ? 0 : 64, &nstreams, &B);
@@ -2266,96 +2273,110 @@ ace_status ace_autotune(const ace_desc *desc, const void *phi, ace_dtype dtype, 
     // a sample long enough (about 40% of a 128-orbital build on 96^3) for the L2 reuse of the
     // blocked pack order and of the persisting scratch window to show in the timing
     const int sample = std::min((count + 1) / 2, 480);
-    auto run_sample = [&](const ChainParams &c, std::vector<void *> &tmp) {
+    ace::PersistOps<T> qops{};
+    const bool has_persist = find_persist_ops<T>(desc->n[0], desc->n[1], desc->n[2], &qops);
+    auto run_sample = [&](const ChainParams &c, std::vector<void *> &tmp) -> ace_status {
+      if (c.persistent) {
+        std::vector<int4> packs;
+        form_packs(op->pairs_h, c.RB, packs);
+        packs.resize(std::min<size_t>(packs.size(), (size_t)sample));
+        const std::vector<ace::ChainBuild<T>> one{
+            {phi_w, static_cast<T *>(op->W), static_cast<const T *>(op->tab->Kperm), op->pmax, op->gmax}};
+        return run_chain_persistent<T>(op, op->stream, op->tab, qops, packs, {}, {}, 0, one, tmp, c);
+      }
       if constexpr (sizeof(T) == 8) return run_chain_f64(op, phi_w, op->tab, &pops, count, tmp, c, sample);
       else return run_chain_plane(op, phi_w, op->tab, pops, count, tmp, c, sample);
     };
     cudaEvent_t e0, e1;
     ACE_CUDA(cudaEventCreate(&e0), "event");
     ACE_CUDA(cudaEventCreate(&e1), "event");
-    float best_ms = 1e30f;
-    const int Bs[5] = {1, 2, 3, 4, 6}, Ss[3] = {2, 4, 8}, Ps[2] = {0, 60}, Rs[4] = {1, 2, 4, 8};
-    for (int ri = 0; ri < 4; ++ri)
-    for (int bi = 0; bi < 5; ++bi)
-      for (int si = 0; si < 3; ++si)
-        for (int pi = 0; pi < 2; ++pi) {
-          ChainParams c;
-          c.G = 1;
-          c.B = Bs[bi];
-          c.streams = Ss[si];
-          c.persist_mb = Ps[pi];
-          c.RB = Rs[ri];
-          float t[2];
-          for (int rep = 0; rep < 2; ++rep) {
-            std::vector<void *> tmp;
-            ACE_CUDA(cudaEventRecord(e0, op->stream), "event");
-            ace_status r = run_sample(c, tmp);
-            ACE_CUDA(cudaEventRecord(e1, op->stream), "event");
-            for (void *q : tmp) cudaFreeAsync(q, op->stream);
-            if (r != ACE_OK) return r;
-            ACE_CUDA(cudaEventSynchronize(e1), "tuning run");
-            cudaEventElapsedTime(&t[rep], e0, e1);
+    // the faster of `reps` runs (ms)
+    auto time_of = [&](const ChainParams &c, int reps, float *ms) -> ace_status {
+      *ms = 1e30f;
+      for (int rep = 0; rep < reps; ++rep) {
+        std::vector<void *> tmp;
+        float t = 0.f;
+        ACE_CUDA(cudaEventRecord(e0, op->stream), "event");
+        ace_status r = run_sample(c, tmp);
+        ACE_CUDA(cudaEventRecord(e1, op->stream), "event");
+        for (void *q : tmp) cudaFreeAsync(q, op->stream);
+        if (r != ACE_OK) return r;
+        ACE_CUDA(cudaEventSynchronize(e1), "tuning run");
+        cudaEventElapsedTime(&t, e0, e1);
+        *ms = std::min(*ms, t);
+      }
+      return ACE_OK;
+    };
+    float best_ms = 0.f;
+    auto consider = [&](const ChainParams &c) -> ace_status {
+      float ms = 0.f;
+      const ace_status r = time_of(c, 2, &ms);
+      if (r == ACE_OK && ms < best_ms) {
+        best_ms = ms;
+        best = c;
+      }
+      return r;
+    };
+    // packs per batch: `batch` takes the listed values, `group` what exceeds them or lies between
+    auto with_batch = [](ChainParams c, int b) {
+      const int listed[5] = {1, 2, 3, 4, 6};
+      c.G = c.B = 1;
+      for (int v : listed)
+        if (v <= b) c.B = v;
+      if (c.B != b) c.G = b;
+      return c;
+    };
+    // the parameters by size first: they are what a build without tuning uses
+    const ChainParams rule = size_params(*desc, op->fp64);
+    const ChainParams start = with_batch(rule, rule.B);
+    best = start;
+    ace_status r = time_of(start, 2, &best_ms);
+    if (r != ACE_OK) return r;
+    std::vector<int> Bs = {1, 2, 3, 4, 6}, Ss = {2, 4, 8}, Ps = {0, 60}, Rs = {1, 2, 4, 8};
+    for (int b : {rule.B / 2, rule.B, std::min(16, 2 * rule.B)})
+      if (b > 0 && std::find(Bs.begin(), Bs.end(), b) == Bs.end()) Bs.push_back(b);
+    if (rule.streams == 3) Ss.push_back(3);
+    if (op->fp64) {  // no L2 window, and the order of the packs decides the bits of W: both stay
+      Ps = {rule.persist_mb};
+      Rs = {rule.RB};
+    }
+    for (int rb : Rs)
+      for (int b : Bs)
+        for (int ns : Ss)
+          for (int mb : Ps) {
+            ChainParams c = with_batch(start, b);
+            c.streams = ns;
+            c.persist_mb = mb;
+            c.RB = rb;
+            if ((r = consider(c)) != ACE_OK) return r;
           }
-          const float ms = std::min(t[0], t[1]);
-          if (ms < best_ms) {
-            best_ms = ms;
-            best = c;
-          }
-        }
     // the pencil tile of the axis-1 pass (three compiled for the FP32 form) on the best settings
     if (sizeof(T) == 4) {
       const ChainParams base = best;
       for (int v : {1, 2}) {
         ChainParams c = base;
         c.conv = v;
-        float t[2];
-        for (int rep = 0; rep < 2; ++rep) {
-          std::vector<void *> tmp;
-          ACE_CUDA(cudaEventRecord(e0, op->stream), "event");
-          ace_status r = run_sample(c, tmp);
-          ACE_CUDA(cudaEventRecord(e1, op->stream), "event");
-          for (void *q : tmp) cudaFreeAsync(q, op->stream);
-          if (r != ACE_OK) return r;
-          ACE_CUDA(cudaEventSynchronize(e1), "tuning run");
-          cudaEventElapsedTime(&t[rep], e0, e1);
-        }
-        const float ms = std::min(t[0], t[1]);
-        if (ms < best_ms) {
-          best_ms = ms;
-          best = c;
-        }
+        if ((r = consider(c)) != ACE_OK) return r;
       }
     }
     // the persistent chain on the same sample, for a few queue lags
-    ace::PersistOps<T> qops{};
-    if (find_persist_ops<T>(desc->n[0], desc->n[1], desc->n[2], &qops)) {
-      std::vector<int4> packs;
-      form_packs(op->pairs_h, best.RB, packs);
-      packs.resize(std::min<size_t>(packs.size(), (size_t)sample));
-      const std::vector<ace::ChainBuild<T>> one{
-          {phi_w, static_cast<T *>(op->W), static_cast<const T *>(op->tab->Kperm), op->pmax, op->gmax}};
+    if (has_persist)
       for (int lag : {2, 3, 4}) {
         ChainParams c = best;
         c.persistent = 1;
         c.lag = lag;
-        float t[2];
-        for (int rep = 0; rep < 2; ++rep) {
-          std::vector<void *> tmp;
-          ACE_CUDA(cudaEventRecord(e0, op->stream), "event");
-          ace_status r = run_chain_persistent<T>(op, op->stream, op->tab, qops, packs, {}, {}, 0, one, tmp, c);
-          ACE_CUDA(cudaEventRecord(e1, op->stream), "event");
-          for (void *q : tmp) cudaFreeAsync(q, op->stream);
-          if (r != ACE_OK) return r;
-          ACE_CUDA(cudaEventSynchronize(e1), "tuning run");
-          cudaEventElapsedTime(&t[rep], e0, e1);
-        }
-        const float ms = std::min(t[0], t[1]);
-        if (ms < best_ms) {
-          best_ms = ms;
-          best = c;
-        }
+        if ((r = consider(c)) != ACE_OK) return r;
       }
+    // what won by less than 1% against the parameters by size, timed side by side, won by chance
+    float t_best = 1e30f, t_rule = 1e30f;
+    for (int rep = 0; rep < 4; ++rep) {
+      float ms = 0.f;
+      if ((r = time_of(best, 1, &ms)) != ACE_OK) return r;
+      t_best = std::min(t_best, ms);
+      if ((r = time_of(start, 1, &ms)) != ACE_OK) return r;
+      t_rule = std::min(t_rule, ms);
     }
+    if (t_best > 0.99f * t_rule) best = start;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     tune_store(TuneKey{desc->n[0], desc->n[1], desc->n[2], op->fp64 ? 1 : 0}, best);

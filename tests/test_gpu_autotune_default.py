@@ -1,0 +1,63 @@
+"""ace_autotune starts from the parameters that a build takes by the size of its grid: tuned builds are not slower than
+untuned ones where the size picks more packs per batch than the listed candidates, the environment still
+overrides the table, and the FP64 form keeps its pack order."""
+
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+# a fresh process, since the table lives as long as the process
+CODE = """
+import sys
+import numpy as np, torch
+sys.path.insert(0, {root!r})
+import paper_2101_03155_gb300 as ace
+from paper_2101_03155_gb300 import ace as abi
+from workloads.generators import water_like
+w = water_like(8, 11.74, {grid}, np.random.default_rng(1010), rho_cut=1e-3, dmin=4.0)
+fp64 = {fp64}
+phi = torch.from_numpy(w.phi if fp64 else w.phi.astype(np.float32)).cuda()
+d = ace.make_desc(w.grid, w.lattice, w.norb, rho_cut=w.rho_cut, prec=ace.ACE_FP64 if fp64 else ace.ACE_MIXED)
+st = torch.cuda.current_stream()
+def chain():
+    best, n, W = 1e30, 0, None
+    for _ in range(30):
+        op = ace.ace_build(d, phi, st)
+        best, n = min(best, abi.ace_stage_times(op)["pair_chain"]), abi.ace_kernel_launches(op)
+        W = abi.get_numpy(op, abi.ACE_GET_W)
+        op.close()
+    return best, n, W
+t0, n0, W0 = chain()
+p = abi.ace_autotune(d, phi, st)
+t1, n1, W1 = chain()
+import os
+os.environ["ACE_PLANE_BATCH"] = "1"
+n2 = chain()[1]
+print(t0, t1, n0, n1, n2, p["row_block"], int(np.array_equal(W0, W1)))
+"""
+
+
+def _run(grid, fp64):
+    r = subprocess.run([sys.executable, "-c", CODE.format(root=ROOT, grid=grid, fp64=fp64)], capture_output=True, text=True,
+                       cwd=ROOT, env={k: v for k, v in os.environ.items() if not k.startswith("ACE_")})
+    assert r.returncode == 0, r.stderr[-2000:]
+    return [float(x) for x in r.stdout.split()]
+
+
+@pytest.mark.parametrize("grid", [(32, 32, 32), (48, 48, 48)])
+def test_tuned_is_not_slower(grid):
+    t0, t1, n0, n1, n2, _, _ = _run(grid, False)
+    assert t1 <= 1.15 * t0  # chain times of separate runs differ by a few percent; batches of 6 took 1.9 times
+    assert n2 > max(n0, n1)  # one pack per batch from the environment
+
+
+def test_fp64_keeps_its_order():
+    t0, t1, n0, n1, n2, rb, same = _run((32, 32, 32), True)
+    assert rb == 4 and same
+    assert t1 <= 1.15 * t0 and n2 > n0
