@@ -1782,7 +1782,8 @@ ace_status checked_pairs(const ace_desc *desc, const int *pairs_host, long npair
 }
 
 // The pair chain of a begun build with a given pair list, into W_out (the caller's buffer when it
-// is device memory, else through a device buffer and a copy); no M, no Cholesky.
+// is device memory on a 16-byte boundary, else through a device buffer and a copy: the plane chain adds W in
+// pairs of points); no M, no Cholesky.
 template <typename T>
 ace_status exchange_w_impl(ace_op *op, void *W_out) {
   const int count = *static_cast<const int *>(op->readback);
@@ -1790,7 +1791,7 @@ ace_status exchange_w_impl(ace_op *op, void *W_out) {
   const int2 *ph = reinterpret_cast<const int2 *>(static_cast<const char *>(op->readback) + 32);
   op->pairs_h.assign(ph, ph + count);
   const size_t bytes = op->esz * (size_t)op->n * op->N;
-  const bool direct = is_device_pointer(W_out);
+  const bool direct = is_device_pointer(W_out) && (reinterpret_cast<uintptr_t>(W_out) & 15) == 0;
   if (direct)
     op->W = W_out;
   else
