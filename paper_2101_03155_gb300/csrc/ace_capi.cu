@@ -1940,14 +1940,18 @@ ace_status ace_m_partial(const ace_desc *desc, const void *phi_slab, const void 
   int *err_d = static_cast<int *>(tmp);
   ACE_CUDA(cudaMemsetAsync(err_d, 0, sizeof(int), st), "zero flag");
   long nl = 0;
-  if (dtype == ACE_F64)
-    ACE_CUDA(dense_gram<double>(static_cast<const double *>(phi_slab), n, static_cast<const double *>(W_slab), n, npts,
-                                -dV, M, err_d, temps, st, &nl),
-             "M partial");
-  else
-    ACE_CUDA(dense_gram<float>(static_cast<const float *>(phi_slab), n, static_cast<const float *>(W_slab), n, npts,
-                               -dV, M, err_d, temps, st, &nl),
-             "M partial");
+  ace_op tmpop;  // only for staging on `st`: slabs off a 16-byte boundary (they are read in 16-byte vectors)
+  tmpop.stream = st;
+  auto run = [&](auto tag) -> ace_status {
+    using T = decltype(tag);
+    const T *x = nullptr, *w = nullptr;
+    ace_status r = stage_input<T>(&tmpop, phi_slab, dtype, n * npts, &x, &temps);
+    if (r == ACE_OK) r = stage_input<T>(&tmpop, W_slab, dtype, n * npts, &w, &temps);
+    if (r != ACE_OK) return r;
+    ACE_CUDA(dense_gram<T>(x, n, w, n, npts, -dV, M, err_d, temps, st, &nl), "M partial");
+    return ACE_OK;
+  };
+  if ((s = dtype == ACE_F64 ? run(double{}) : run(float{})) != ACE_OK) return s;
   return finish_flag(err_d, st, "M partial");
 }
 

@@ -1,5 +1,6 @@
 """Device arrays of the multi-GPU steps that start off a 16-byte boundary go through aligned copies: W of
-ace_exchange_w (added in pairs of points) on every kind of grid."""
+ace_exchange_w (added in pairs of points) on every kind of grid, and the slabs of ace_m_partial (read in
+16-byte vectors) on every route of the Gram."""
 
 import numpy as np
 import pytest
@@ -44,3 +45,27 @@ def test_exchange_w(prec, grid, off):
     torch.cuda.synchronize()
     assert rel_max(got.cpu().numpy(), want.cpu().numpy()) <= (2 * MIXED_W_RTOL if prec == ace.ACE_MIXED else 0.0)
     assert bool((buf[:off] == 7.0).all()) and bool((buf[off + x.numel():] == 7.0).all())
+
+
+@pytest.mark.parametrize("prec", [ace.ACE_MIXED, ace.ACE_FP64])
+@pytest.mark.parametrize("n,npts", [(4, 132), (12, 4096), (12, 100), (40, 4097), (130, 2048)])
+@pytest.mark.parametrize("off", OFFSETS)
+def test_m_partial(prec, n, npts, off, monkeypatch):
+    import torch
+
+    gen = torch.Generator().manual_seed(n + npts)
+    dt = torch.float64 if prec == ace.ACE_FP64 else torch.float32
+    x = torch.randn((n, npts), generator=gen, dtype=dt).cuda()
+    y = torch.randn((n, npts), generator=gen, dtype=dt).cuda()
+    d = ace.make_desc((16, 16, 16), np.diag([8.0, 8.0, 8.0]), n, prec=prec)
+    for env in (None, "ACE_NO_TMA", "ACE_NO_TC"):
+        if env:
+            monkeypatch.setenv(env, "1")
+        M = [torch.empty((n, n), dtype=torch.float64, device="cuda") for _ in range(2)]
+        abi.ace_m_partial(d, x, y, M[0])
+        abi.ace_m_partial(d, _shifted(x, off)[0], _shifted(y, off)[0], M[1])
+        # the same kernels on the same values; FP64 atomics add the chunks of some routes in any order
+        tol = 2.0**-45 * (x.double().abs() @ y.double().abs().T) / 8.0
+        assert bool(((M[0] - M[1]).abs() <= tol).all())
+        if env:
+            monkeypatch.delenv(env)
