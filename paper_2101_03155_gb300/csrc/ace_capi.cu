@@ -838,11 +838,11 @@ ace_status run_chain_persistent(ace_op *op, cudaStream_t st, const DeviceTables 
   return ACE_OK;
 }
 
-// Side streams and packs per batch of a chain within ACE_SCRATCH_MB of scratch (unset: dflt_mb, 0 for no
-// bound), one pack at least.
+// Side streams and packs per batch of a chain within ACE_SCRATCH_MB of scratch (unset: dflt_mb, negative for
+// no bound), one pack at least.
 void fit_scratch(size_t pack_bytes, int dflt_mb, int *nstreams, int *B) {
   const int mb = env_int("ACE_SCRATCH_MB", dflt_mb);
-  if (mb <= 0) return;
+  if (mb < 0) return;
   const int slots = (int)std::min(65535.0, std::max(1.0, std::floor(mb * 1048576.0 / (double)pack_bytes)));
   *nstreams = std::min(*nstreams, slots);
   *B = std::min(*B, slots / *nstreams);
@@ -872,7 +872,7 @@ ace_status run_chain_plane(ace_op *op, const float *phi, const DeviceTables *tab
   int B = std::min(std::max(cp.G, cp.B), ((count + 1) / 2 + nstreams - 1) / nstreams);
   // complex values of one pack in the scratch (16-byte units of two lines of axis 2)
   const size_t pack_elems = (size_t)d.n[0] * d.n[2] * ((d.n[1] + 1) / 2) * 2;
-  fit_scratch(sizeof(cpx<float>) * pack_elems, 0, &nstreams, &B);
+  fit_scratch(sizeof(cpx<float>) * pack_elems, -1, &nstreams, &B);
   std::vector<int4> packs;
   form_packs(op->pairs_h, cp.RB, packs);
   void *tmp = nullptr;
@@ -964,7 +964,7 @@ ace_status run_chain_f64(ace_op *op, const double *phi, const DeviceTables *tab,
   int B = std::min({65535, std::max(cp.G, cp.B), ((count + 1) / 2 + nstreams - 1) / nstreams});
   // the pencil route has a budget of 64 MB unless set (one pack at least; 16 orbitals on 160^3, one pack of 66 MB
   // at a time, take 90 ms instead of 83); W does not depend on the batches
-  fit_scratch(sizeof(cpx<double>) * (size_t)N, pops ? 0 : 64, &nstreams, &B);
+  fit_scratch(sizeof(cpx<double>) * (size_t)N, pops ? -1 : 64, &nstreams, &B);
   std::vector<int4> packs;
   form_packs(op->pairs_h, cp.RB, packs);
   // only the side streams that get a batch: each of them is joined by its batches' events, and a stream

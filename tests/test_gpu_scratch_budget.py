@@ -59,6 +59,8 @@ def test_budget_bounds_the_scratch(grid, prec, monkeypatch):
     rest = high[one] - pack
     assert high[three] <= rest + three * 2**20 + 2**20
     assert high[wide] >= rest + 4 * pack
+    monkeypatch.setenv("ACE_SCRATCH_MB", "0")  # no budget at all: one pack
+    assert pool.high_of(lambda: abi.ace_exchange_w(d, x, pairs, W[one])) <= high[one] + 2**20
     for mb in (three, one):
         if fp64:
             assert torch.equal(W[mb], W[wide])
