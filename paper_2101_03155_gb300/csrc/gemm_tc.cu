@@ -754,7 +754,9 @@ __global__ void __launch_bounds__(LW_NT, 1) tc_left_mul_tma_kernel(const float *
   } else {
     // ---- split: team t takes the items of parity t; a thread splits column `col` of the box.  The
     // number of stages is even, so that each team meets only its own box barriers (a parity seen by
-    // neither team in between is ambiguous) ----
+    // neither team in between is ambiguous).  Three operand buffers are safe although the teams share them:
+    // a team that waits for op_empty of item q - 3 has waited for that of q - 5, and the one MMA lane's
+    // commits complete in order, so the buffer's use before (q - 6) is done and the parity is unambiguous ----
     const int team = warp >> 2, col = tid & 127;
     int stage = team, b = team;
     uint32_t sph = 0, bph = 0;
@@ -1006,7 +1008,9 @@ __global__ void __launch_bounds__(GW_NT, 1) tc_gram_tma_kernel(const __grid_cons
     // ---- split warps: team t (warps 8t - 8t + 7) takes the K-steps of parity t; its first 128
     // threads split the rows of the X box into the A tiles, the others those of the Y box into the
     // B tiles, a row of 32 K-values each; row `row` of a box holds its 16-byte chunk k4 at position
-    // k4 ^ (row & 7) ----
+    // k4 ^ (row & 7).  The teams share three operand buffers: a team that waits for op_empty of K-step q - 3 has
+    // waited for that of q - 5, and the one MMA lane's commits complete in order, so the buffer's use before
+    // (q - 6) is done and the parity is unambiguous ----
     const int team = warp >> 3, row = tid & 127, half = (tid >> 7) & 1;
     int stage = team, b = team;
     uint32_t sph = 0, bph = 0;

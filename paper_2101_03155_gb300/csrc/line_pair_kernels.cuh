@@ -67,7 +67,6 @@ __global__ void __launch_bounds__((PlaneOf<N2, N3>::NT), (lp_min_blocks<N2, N3>(
   if (!(a.skip_rel > 0.f && inv_plane_negligible(a.pmax, a.gmax, a.n1, i1, pk, a.skip_rel))) {
     lp_tables(N2, N3, G::NT, a.tw2, a.tw3, tw2, tw3);
     const PlanePtrs q = lp_ptrs(a, pk, (long long)i1 * (N2 * N3));
-    lp_prefetch(q, N2 * N3, a.hints);
     __syncthreads();
     lp_inv_rowsA<N3>(g, src, s, tw3);
     lp_sync(g);
@@ -118,7 +117,6 @@ struct LpConvShape {
   static constexpr int smem = 16 * (WARPS * T * L + L);
   static constexpr int fit = (228 * 1024) / (smem + 1024), thr = 640 / NT;
   static constexpr int minb = fit < thr ? fit : thr;
-  static constexpr bool fits = smem <= 227 * 1024;
 };
 
 template <int L, int V>

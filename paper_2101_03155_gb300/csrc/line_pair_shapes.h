@@ -3,7 +3,8 @@
 // shared memory.
 // Run-time shapes were tried (one kernel that selects the stages by length): twice the time per point
 // (80^3: 6.4 against 3.4 ms, 100 x 108 x 90: 20.7 against 10.7 ms).  Other grids take the five pencil
-// passes of pair_chain.cuh.
+// passes of pair_chain.cuh.  125 is not among the lengths: its plane passes have not been compiled or measured
+// (128 orbitals on 125^3 take 183 ms in pencil passes).  The shapes make 32 objects and most of a library of 90 MB.
 #pragma once
 
 #define ACE_LP_PLANE_LENGTHS(X)                                                                             \

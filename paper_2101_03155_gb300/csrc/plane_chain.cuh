@@ -246,15 +246,12 @@ __device__ __forceinline__ void plane_forward(const T *__restrict__ phi, long lo
 
 // Drops the 128-byte lines that lie wholly inside [base, base + bytes) from L2 without writing
 // them back (their contents become undefined); the CTA's threads share the lines.
-__device__ __forceinline__ void l2_discard_n(const void *base, size_t bytes, int nthreads) {
-  const unsigned long long b = reinterpret_cast<unsigned long long>(base);
-  const unsigned long long first = (b + 127) & ~127ull, end = (b + bytes) & ~127ull;
-  for (unsigned long long a = first + 128ull * threadIdx.x; a < end; a += 128ull * nthreads)
-    asm volatile("discard.global.L2 [%0], 128;" ::"l"(a) : "memory");
-}
 template <int NT>
 __device__ __forceinline__ void l2_discard(const void *base, size_t bytes) {
-  l2_discard_n(base, bytes, NT);
+  const unsigned long long b = reinterpret_cast<unsigned long long>(base);
+  const unsigned long long first = (b + 127) & ~127ull, end = (b + bytes) & ~127ull;
+  for (unsigned long long a = first + 128ull * threadIdx.x; a < end; a += 128ull * NT)
+    asm volatile("discard.global.L2 [%0], 128;" ::"l"(a) : "memory");
 }
 
 // Inverse transform of one permuted spectrum plane src (read through L2 only: it was written
