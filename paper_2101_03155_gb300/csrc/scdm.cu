@@ -28,6 +28,7 @@ constexpr int kNsMax = 64;          // Newton-Schulz iterations at most
 constexpr int kNsChunk = 16;        // iterations launched between host checks of convergence
 constexpr double kNsStop = 1e-12;   // max |T - I| below which the following iterations are skipped
 constexpr int kBlk = 8;             // points of a block of the FP32 selection
+constexpr long long kLeft = -1;
 constexpr int kSeedLag = 16;        // most vectors a threshold block may be behind
 constexpr int kChunk = 8;           // products summed in the working type before the FP64 add
 constexpr double kDependent = 1e-24;    // |residual|^2 / |psi(c)|^2 below which a column is dependent
@@ -84,7 +85,7 @@ struct SelArgs {
   long long *tval, *tidx;   // [gridDim.x]
   long long *bmax;       // [blocks]
   int *bcnt;             // [blocks]
-  long long *thr;        // [n + 1], from 0
+  long long *thr;        // [n + 1], from 0 (kLeft: the steps over bounds have been left)
   // clock cycles: the longest CTA of the current pass, and by how much the last passes have cost more than
   // passes over every point would have; then 0, or the step from which on every point is updated
   int *work;
@@ -120,7 +121,7 @@ struct __align__(16) ScdmSmem {
   double rv[kUpdNT / 32], rv0[kUpdNT / 32];
   long long rk[kUpdNT / 32], ri[kUpdNT / 32], tk[kUpdNT / 32], ti[kUpdNT / 32];
   long long chosen, top;
-  int last;
+  int last, leave;
 };
 
 __device__ __forceinline__ float dot4(float4 a, float4 b) {
@@ -230,8 +231,9 @@ __device__ __forceinline__ void stage_rows(const float *Ub, int nf, int j, int u
 // (u_j . psi(r))^2 in order of j.  With `stop` it ends early once every residual is below the largest
 // up-to-date one: the residuals only fall, so the block cannot hold the pivot.  A block that gets to k adds
 // its maximum to (best, bi) and to the threshold.  Returns the block's new bound.
-//   Up to 128 orbitals the rows of the basis come through the warp's staging buffers, eight ahead of their
-// use (loads from L2 one vector at a time took most of a long catch-up).
+//   Up to 128 orbitals (MANY = false) the rows of the basis come through the warp's staging buffers, eight ahead of
+// their use (loads from L2 one vector at a time took most of a long catch-up).
+template <bool MANY>
 __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ psi, int n, long long N, long long *d,
                                                     const SelArgs &s, long long blk, long long r0, int lim, int j, int k,
                                                     int upto, bool stop, long long dr, float (&x)[32],
@@ -241,7 +243,7 @@ __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ ps
   const long long thr = stop ? __ldcg(s.thr + k) : kNone;
   const float *Ub = static_cast<const float *>(s.Ub);
   long long mx = blk_max(dr);
-  if (n <= 128) {
+  if (!MANY) {
     const int c = threadIdx.x & 3, nf = (n + 3) / 4;
     int buf = 0;
     if (j < upto) stage_rows(Ub, nf, j, upto, stage);
@@ -270,9 +272,10 @@ __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ ps
         t += __shfl_xor_sync(0xffffffffu, t, 2);
         pm[q] = t + __shfl_xor_sync(0xffffffffu, t, 1);
       }
+      KeySquare sq[kRows];
 #pragma unroll
-      for (int q = 0; q < kRows; ++q)
-        if (q < m) dr = key_downdate(dr, __float_as_uint(pm[q]));
+      for (int q = 0; q < kRows; ++q) sq[q] = key_square(__float_as_uint(pm[q]));
+      dr = key_close(key_less_all<kRows>(key_open(dr), sq, m), dr);
       j += m;
       mx = blk_max(dr);
       buf ^= 1;
@@ -295,14 +298,15 @@ __device__ __forceinline__ long long refresh_loaded(const float *__restrict__ ps
   store_block(d, s, blk, r0, lim, j_in, j, k, dr, mx, best, bi);
   return mx;
 }
-__device__ long long refresh_block(const float *__restrict__ psi, int n, long long N, long long *d, const SelArgs &s,
-                                   long long blk, int k, int upto, bool stop, float4 *stage,
-                                   long long &best, long long &bi) {
+template <bool MANY>
+__device__ __forceinline__ long long refresh_block(const float *__restrict__ psi, int n, long long N, long long *d,
+                                                   const SelArgs &s, long long blk, int k, int upto, bool stop,
+                                                   float4 *stage, long long &best, long long &bi) {
   long long r0, dr;
   int lim, j;
   float x[32];
   load_state(psi, n, N, d, s, blk, r0, lim, j, dr, x);
-  return refresh_loaded(psi, n, N, d, s, blk, r0, lim, j, k, upto, stop, dr, x, stage, best, bi);
+  return refresh_loaded<MANY>(psi, n, N, d, s, blk, r0, lim, j, k, upto, stop, dr, x, stage, best, bi);
 }
 
 // Stored residuals: FP64 values, or the keys of the FP32 selection (residual_key.h)
@@ -321,7 +325,7 @@ struct Resid<float> {
 // choice of the pivots (U and Phi are computed from the pivots and Psi alone).  A column whose
 // residual is at the rounding level of T (|residual|^2 below kDependent(T) |psi(c_k)|^2) gives
 // u_k = 0 and sets *dependent.
-template <typename T, bool LAZY>
+template <typename T, bool LAZY, bool MANY>
 __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr, int n, long long N, int nblk,
                            typename Resid<T>::type *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm,
                            float4 *stage) {
@@ -470,7 +474,8 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
       __syncthreads();  // u_k for the CTA, in L2
       if (seed < N) {
         if (sr0 + (lane >> 2) == cr) seed_d = -1;
-        refresh_loaded(psi, n, N, d, s, seed, sr0, slim, sj, k + 1, k + 1, true, seed_d, sv, stage + warp * kStage, best, bi);
+        refresh_loaded<MANY>(psi, n, N, d, s, seed, sr0, slim, sj, k + 1, k + 1, true, seed_d, sv,
+                             stage + warp * kStage, best, bi);
       }
     }
   }
@@ -478,7 +483,7 @@ __device__ void pivot_step(const T *__restrict__ psi, long long si, long long sr
 
 // End of a pass for one block: publish the block maximum; the last block to publish takes the
 // pivot step and resets the counter for the next pass (true for that block).  Orbital i at point r is psi[i si + r sr].
-template <typename T, bool LAZY>
+template <typename T, bool LAZY, bool MANY = false>
 __device__ bool finish_pass(long long best, long long bi, long long top, long long ti, long long start,
                             const T *__restrict__ psi, long long si, long long sr, int n, long long N,
                             typename Resid<T>::type *__restrict__ d, const SelArgs &s, ScdmSmem<T> &sm, float4 *stage) {
@@ -518,15 +523,25 @@ __device__ bool finish_pass(long long best, long long bi, long long top, long lo
   __syncthreads();
   if (!sm.last) return false;
   __threadfence();
-  pivot_step<T, LAZY>(psi, si, sr, n, N, gridDim.x, d, s, sm, stage);
-  if (tid == 0) {
+  if (tid == kUpdNT - 1) {  // in the shadow of the pivot step's first loads
     *s.count = 0u;
     if constexpr (LAZY) {
+      sm.leave = 0;
       if (s.k > 0) {
-        *s.excess = max(0ll, *s.excess + __ldcg(s.work) - s.full_cost);
+        const long long x = max(0ll, __ldcg(s.excess) + __ldcg(s.work) - s.full_cost);
+        *s.excess = x;
         *s.work = 0;
-        if (*s.excess > s.leave_cost || s.k == s.leave_step) *s.left = s.k + 1;
+        // not past a quarter of the steps: what does not localise shows early, and the blocks' catch-up grows with k
+        sm.leave = (x > s.leave_cost && 4 * s.k < n) || s.k == s.leave_step;
       }
+    }
+  }
+  pivot_step<T, LAZY, MANY>(psi, si, sr, n, N, gridDim.x, d, s, sm, stage);
+  if constexpr (LAZY) {
+    if (sm.leave) {
+      __syncthreads();  // the pivot step's own entry of thr
+      for (int i = s.k + 1 + tid; i <= n; i += kUpdNT) s.thr[i] = kLeft;
+      if (tid == 0) *s.left = s.k + 1;
     }
   }
   return true;
@@ -571,7 +586,7 @@ __global__ void __launch_bounds__(kUpdNT) scdm_pass_kernel(const T *__restrict__
 // it was last brought up to date bounds its present one: a step has to look only at the blocks whose
 // bound reaches the largest up-to-date residual.  For 128 orbitals on 96^3 that is 27,000 block visits in
 // all 128 steps, a quarter of the blocks once, where passes over every point (the plain greedy selection)
-// read Psi 128 times: 12.3 ms per call, bound by HBM at 0.8 of its bandwidth; now 4.9 ms, most of it the
+// read Psi 128 times: 12.3 ms per call, bound by HBM at 0.8 of its bandwidth; now 4.1-4.9 ms, most of it the
 // chain of the 127 steps (launch, look at the bounds, visits, pivot step: about 30 us each).
 //   Orbitals that no rotation localises (plane waves of a metal) flatten the residuals, and the visits of a step
 // then cost more than a pass over every point: the steps measure themselves, and when the last ones have lost
@@ -582,7 +597,7 @@ __global__ void __launch_bounds__(kUpdNT) scdm_pass_kernel(const T *__restrict__
 
 // d[r] = |psi(r)|^2 (FP32), one point per thread; the sum has the order of refresh_block's (32 partial sums over
 // orbitals 4 l .. 4 l + 3 (+ 128 f), then the pairwise tree).
-template <bool LAZY>
+template <bool LAZY, bool MANY>
 __global__ void __launch_bounds__(kUpdNT) scdm_norm_kernel(const float *__restrict__ psi, int n, long long N,
                                                            long long *__restrict__ d, SelArgs s) {
   __shared__ __align__(16) ScdmSmem<float> sm;
@@ -627,7 +642,7 @@ __global__ void __launch_bounds__(kUpdNT) scdm_norm_kernel(const float *__restri
       s.bcnt[r / kBlk] = 0;
     }
   }
-  finish_pass<float, LAZY>(best, bi, best, bi < N ? bi / kBlk : N, 0, psi, N, 1, n, N, d, s, sm, stage_all);
+  finish_pass<float, LAZY, MANY>(best, bi, best, bi < N ? bi / kBlk : N, 0, psi, N, 1, n, N, d, s, sm, stage_all);
 }
 
 // Few points (see launch_scdm): step k >= 1 over every point, one per thread.  u_{k-1} . psi(r) is summed in the order
@@ -673,7 +688,8 @@ __global__ void __launch_bounds__(kUpdNT) scdm_full_kernel(const float *__restri
 }
 
 // Point-major copy pt[r][i] = psi[i][r] for i < n, zero for n <= i < ld: 32 points x 32 orbitals per block.
-__global__ void scdm_points_copy_kernel(const float *__restrict__ psi, int n, long long N, int ld, float *__restrict__ pt) {
+__global__ void scdm_points_copy_kernel(const float *__restrict__ psi, int n, long long N, int ld,
+                                        float *__restrict__ pt) {
   __shared__ float tile[32][33];
   const long long r0 = blockIdx.x * 32ll;
   const int i0 = blockIdx.y * 32;
@@ -687,6 +703,7 @@ __global__ void scdm_points_copy_kernel(const float *__restrict__ psi, int n, lo
 }
 
 // Every block up to date with u_0 .. u_{k-2}.
+template <bool MANY>
 __global__ void __launch_bounds__(kUpdNT, 2) scdm_catch_up_kernel(const float *__restrict__ psi, int n, long long N,
                                                                   long long *__restrict__ d, SelArgs s) {
   extern __shared__ float4 stage_all[];  // kStage per warp
@@ -694,7 +711,7 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_catch_up_kernel(const float *_
   long long best = kNone, bi = N;
   for (long long b = (long long)blockIdx.x * (kUpdNT / 32) + (threadIdx.x >> 5); b < nb; b += nwarps)
     if (s.bcnt[b] < s.k - 1)
-      refresh_block(psi, n, N, d, s, b, s.k, s.k - 1, false, stage_all + (threadIdx.x >> 5) * kStage, best, bi);
+      refresh_block<MANY>(psi, n, N, d, s, b, s.k, s.k - 1, false, stage_all + (threadIdx.x >> 5) * kStage, best, bi);
 }
 
 // Step k >= 1 over every point, from the point-major copy pt.  Every warp takes an equal share of the blocks, 32
@@ -703,8 +720,9 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_catch_up_kernel(const float *_
 // pairwise tree, and lane l keeps point l of the 32.  In the first such step (FIRST) the blocks that the last
 // pivot step looked at have u_{k-1} already.
 template <bool FIRST>
-__global__ void __launch_bounds__(kUpdNT, 3) scdm_points_kernel(const float *__restrict__ psi, const float *__restrict__ pt,
-                                                                int n, long long N, long long *__restrict__ d, SelArgs s) {
+__global__ void __launch_bounds__(kUpdNT, 3) scdm_points_kernel(const float *__restrict__ psi,
+                                                                const float *__restrict__ pt, int n, long long N,
+                                                                long long *__restrict__ d, SelArgs s) {
   __shared__ __align__(16) ScdmSmem<float> sm;
   const int tid = threadIdx.x, lane = tid & 31, nf = (n + 3) / 4, k = s.k;
   const unsigned full = 0xffffffffu;
@@ -767,9 +785,12 @@ __global__ void __launch_bounds__(kUpdNT, 3) scdm_points_kernel(const float *__r
 // threshold and which a later step will need: without it the longest catch-up of a step was 57 vectors on
 // average (128 orbitals on 96^3), a chain of dependent FP64 updates (8.0 ms per call).  A CTA leaves out the
 // block with its largest bound, which the pivot step may be working on.
+//   One CTA per SM: a step is a chain of latencies, and held to 128 registers for two it spills on it (ms per
+// call with two / one: 128 orbitals on 96^3 5.4 / 4.9, 256 on 64^3 17.4 / 14.5).
 constexpr int kAhead = 8;      // vectors per step and block
-constexpr int kAheadMost = 2;  // blocks per warp and step
-__global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__restrict__ psi, int n, long long N,
+constexpr int kAheadMost = 4;  // blocks per warp and step
+template <bool MANY>
+__global__ void __launch_bounds__(kUpdNT, 1) scdm_step_kernel(const float *__restrict__ psi, int n, long long N,
                                                               long long *__restrict__ d, SelArgs s) {
   __shared__ __align__(16) ScdmSmem<float> sm;
   extern __shared__ float4 stage_all[];  // kStage per warp
@@ -782,7 +803,7 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
   long long thr = __ldcg(s.thr + s.k);
   const long long soon = key_somewhat_below(thr);
   long long best = kNone, bi = N, top = kNone, ti = N;
-  if (*s.left) return;
+  if (thr == kLeft) return;
   for (long long b0 = w; b0 < nb; b0 += 32 * nwarps) {
     const long long b = b0 + lane * nwarps;
     long long bound = b < nb ? s.bmax[b] : kNone;
@@ -790,7 +811,8 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
     while (left) {
       const int src = __ffs(left) - 1;
       left &= left - 1;
-      const long long mx = refresh_block(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, s.k, true, stage, best, bi);
+      const long long blk = __shfl_sync(full, b, src);
+      const long long mx = refresh_block<MANY>(psi, n, N, d, s, blk, s.k, s.k, true, stage, best, bi);
       if (lane == src) bound = mx;
       if (left) {
         thr = __ldcg(s.thr + s.k);
@@ -799,7 +821,7 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
     }
     amax(top, ti, bound, b);
   }
-  if (finish_pass<float, true>(best, bi, top, ti, start, psi, N, 1, n, N, d, s, sm, stage_all)) return;
+  if (finish_pass<float, true, MANY>(best, bi, top, ti, start, psi, N, 1, n, N, d, s, sm, stage_all)) return;
   int most = kAheadMost;
   for (long long b0 = w; b0 < nb && most > 0; b0 += 32 * nwarps) {
     const long long b = b0 + lane * nwarps;
@@ -807,8 +829,8 @@ __global__ void __launch_bounds__(kUpdNT, 2) scdm_step_kernel(const float *__res
     const int cnt = bound >= 0 && bound >= soon && b != sm.top ? s.bcnt[b] : s.k;
     for (unsigned ahead = __ballot_sync(full, cnt < s.k); ahead && most > 0; ahead &= ahead - 1, --most) {
       const int src = __ffs(ahead) - 1;
-      refresh_block(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, min(s.k, __shfl_sync(full, cnt, src) + kAhead), false,
-                    stage, best, bi);
+      const int upto = min(s.k, __shfl_sync(full, cnt, src) + kAhead);
+      refresh_block<MANY>(psi, n, N, d, s, __shfl_sync(full, b, src), s.k, upto, false, stage, best, bi);
     }
   }
 }
@@ -942,7 +964,8 @@ __global__ void scdm_factor_kernel(const double *__restrict__ M, const double *_
 }
 
 struct Layout {
-  size_t d, bval, bidx, tval, tidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count, bmax, bcnt, thr, work, excess, left, total;
+  size_t d, bval, bidx, tval, tidx, Ub, M, S, Y0, Y1, Z0, Z1, Tm, U, Ut, f, dev, piv, dependent, count;
+  size_t bmax, bcnt, thr, work, excess, left, total;
 };
 
 Layout layout(int n, long long N, size_t elem) {
@@ -1035,7 +1058,8 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
   auto blocks = [&](auto kernel, size_t smem, long long least, unsigned *grid) {
     int per_sm = 0;
     // shared memory above 48 KB, asked for once per call (a driver call of a microsecond)
-    cudaError_t q = smem ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+    cudaError_t q = cudaSuccess;
+    if (smem) q = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (q == cudaSuccess) q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kUpdNT, smem);
     *grid = (unsigned)std::max<long long>(1, std::min({(long long)std::max(per_sm, 1) * sms, (long long)kUpdBlocks,
                                                        (N + least - 1) / least}));
@@ -1055,29 +1079,33 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
   } else if (4.0 * n * N < 1e6 * env_value("ACE_SCDM_BOUNDS_MB", 70)) {
     // Psi stays in L2 and a pass over every point is cheaper than the bounds (ms per call, with them / without:
     // 64 orbitals on 48^3 1.94 / 1.64, on 64^3 2.14 / 2.11; 32 on 64^3 1.35 / 1.10; on 72^3 64 take 2.2 / 3.2)
-    e = blocks(scdm_norm_kernel<false>, 0, kUpdNT, &first);
+    e = blocks(scdm_norm_kernel<false, false>, 0, kUpdNT, &first);
     if (e == cudaSuccess) e = blocks(scdm_full_kernel, 0, kUpdNT, &next);
     if (e != cudaSuccess) return e;
-    scdm_norm_kernel<false><<<first, kUpdNT, 0, st>>>(psi, n, N, d, sa);
+    scdm_norm_kernel<false, false><<<first, kUpdNT, 0, st>>>(psi, n, N, d, sa);
     e = steps(scdm_full_kernel, 0, 1, n);
   } else {
     // a pass over every point reads Psi at about 6.5 TB/s (at 1.9 GHz); leaving takes the point-major copy, the
-    // vectors that the blocks miss, about three passes' time
+    // vectors that the blocks miss: about three passes' time, and more where a block is read again for every four
+    // vectors
     sa.full_cost = (int)std::min(5e8, 4.0 * n * N / 3400.0);
-    sa.leave_cost = 3 * sa.full_cost + 114000;
+    sa.leave_cost = (n > 128 ? 16 : 3) * std::min(sa.full_cost, 100000000) + 114000;
     sa.leave_step = env_value("ACE_SCDM_LEAVE_STEP", 0);
     // thresholds, clocks and the step of leaving (neighbours in the workspace)
     e = cudaMemsetAsync(sa.thr, 0, L.total - L.thr, st);
-    if (e == cudaSuccess) e = blocks(scdm_norm_kernel<true>, kStageBytes, kUpdNT, &first);
-    if (e == cudaSuccess) e = blocks(scdm_catch_up_kernel, kStageBytes, kUpdNT, &next);
-    if (e == cudaSuccess) e = blocks(scdm_step_kernel, kStageBytes, kBlk * kUpdNT, &next);  // a block per lane
+    const auto catch_up = n > 128 ? scdm_catch_up_kernel<true> : scdm_catch_up_kernel<false>;
+    const auto norm = n > 128 ? scdm_norm_kernel<true, true> : scdm_norm_kernel<true, false>;
+    const auto step = n > 128 ? scdm_step_kernel<true> : scdm_step_kernel<false>;
+    if (e == cudaSuccess) e = blocks(norm, kStageBytes, kUpdNT, &first);
+    if (e == cudaSuccess) e = blocks(catch_up, kStageBytes, kUpdNT, &next);
+    if (e == cudaSuccess) e = blocks(step, kStageBytes, kBlk * kUpdNT, &next);  // a block per lane
     if (e != cudaSuccess) return e;
-    scdm_norm_kernel<true><<<first, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
+    norm<<<first, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
     // the host looks every 64 steps whether the steps over bounds were left (each look idles the device for
     // about 15 us, a step that returns at once takes 2.5)
     int left = 0;
     for (int k = 1; k < n && left == 0; k += 64) {
-      e = steps(scdm_step_kernel, kStageBytes, k, std::min(n, k + 64));
+      e = steps(step, kStageBytes, k, std::min(n, k + 64));
       if (e == cudaSuccess) e = cudaMemcpyAsync(&left, sa.left, sizeof(int), cudaMemcpyDeviceToHost, st);
       if (e == cudaSuccess) e = cudaStreamSynchronize(st);
       if (e != cudaSuccess) return e;
@@ -1087,9 +1115,10 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
       float *pt = nullptr;
       e = cudaMallocAsync(&pt, sizeof(float) * (size_t)N * ld, st);
       if (e != cudaSuccess) return e;
-      scdm_points_copy_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)((ld + 31) / 32)), dim3(32, 8), 0, st>>>(psi, n, N, ld, pt);
+      const dim3 tiles((unsigned)((N + 31) / 32), (unsigned)((ld + 31) / 32));
+      scdm_points_copy_kernel<<<tiles, dim3(32, 8), 0, st>>>(psi, n, N, ld, pt);
       sa.k = left;
-      scdm_catch_up_kernel<<<next, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
+      catch_up<<<next, kUpdNT, kStageBytes, st>>>(psi, n, N, d, sa);
       *launches += 2;
       e = blocks(scdm_points_kernel<false>, 0, kUpdNT, &next);
       for (sa.k = left; sa.k < n && e == cudaSuccess; ++sa.k) {

@@ -21,11 +21,16 @@ def lib(tmp_path_factory):
     src, so = d / "k.cpp", d / "k.so"
     src.write_text('#include "residual_key.h"\nextern "C" long long of_bits(unsigned b) { return ace::key_of_bits(b); }\n'
                    'extern "C" long long down(long long v, unsigned p) { return ace::key_downdate(v, p); }\n'
+                   'extern "C" long long down_all(long long v, const unsigned *p, int n) {\n'
+                   '  ace::KeySquare s[8];\n  for (int q = 0; q < 8; ++q) s[q] = ace::key_square(p[q]);\n'
+                   '  return ace::key_close(ace::key_less_all<8>(ace::key_open(v), s, n), v); }\n'
                    'extern "C" long long below(long long v) { return ace::key_somewhat_below(v); }\n')
     subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-o", str(so), str(src)], check=True)
     k = ctypes.CDLL(str(so))
     k.of_bits.argtypes, k.of_bits.restype = [ctypes.c_uint32], ctypes.c_longlong
     k.down.argtypes, k.down.restype = [ctypes.c_longlong, ctypes.c_uint32], ctypes.c_longlong
+    k.down_all.argtypes = [ctypes.c_longlong, ctypes.POINTER(ctypes.c_uint32), ctypes.c_int]
+    k.down_all.restype = ctypes.c_longlong
     k.below.argtypes, k.below.restype = [ctypes.c_longlong], ctypes.c_longlong
     return k
 
@@ -96,6 +101,29 @@ def test_marks(lib):
     for p in (0x7F800000, 0xFF800000, 0x7FC00000):
         assert lib.down(one, p) == 0 and lib.down(INF, p) == 0
     assert lib.down(INF, 0x7F7FFFFF) == INF
+
+
+def test_runs_equal_single_updates(lib):
+    """Eight updates at once give the bits of eight updates in turn, whether the leading bit stays or moves."""
+    rng = np.random.default_rng(4)
+    special = [lib.of_bits(b) for b in EDGES] + [-1, NONE, INF]
+    for trial in range(6000):
+        v = special[trial % len(special)] if trial < 300 else lib.of_bits(int(rng.integers(1, 0x7F800000)))
+        for _ in range(4):
+            root = float(_value(v)) ** 0.5 if 0 < v < INF else 1.0
+            scale = 2.0 ** -rng.integers(0, 40, 8) * rng.uniform(0, 1, 8) * rng.choice([1.0, 0.3, 0.02, 1.5])
+            p = np.minimum(root * scale, 3e38).astype(np.float32)
+            if rng.random() < 0.1:
+                p[rng.integers(0, 8)] = rng.choice(np.array([0, np.inf, np.nan, 1e-45, 3e38], dtype=np.float32))
+            bits = p.view(np.uint32)
+            n = int(rng.integers(0, 9))
+            want = v
+            for q in range(n):
+                want = lib.down(want, int(bits[q]))
+            assert lib.down_all(v, (ctypes.c_uint32 * 8)(*[int(b) for b in bits]), n) == want
+            if want <= 0:
+                break
+            v = want
 
 
 def test_look_ahead_mark(lib):
