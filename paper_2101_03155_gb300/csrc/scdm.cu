@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kUpdNT) scdm_pass_kernel(const T *__restrict__
 //   Orbitals that no rotation localises (plane waves of a metal) flatten the residuals, and the visits of a step
 // then cost more than a pass over every point: the steps measure themselves, and when the last ones have lost
 // about what changing over costs, the rest are passes over every point.  64 such orbitals on 72^3: 5.8 ms on
-// bounds alone, 3.4 with passes alone, 3.8 with the change; 200 on 64^3: 30, 13.4 and 14.2 ms.
+// bounds alone, 3.4 with passes alone, 3.8 with the change; 200 on 64^3: 32, 13.4 and 14.2 ms.
 //   Every residual goes through the same operations in the same order in all of these, so the pivots are the
 // same whichever way a step goes.
 
@@ -1086,10 +1086,9 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
     e = steps(scdm_full_kernel, 0, 1, n);
   } else {
     // a pass over every point reads Psi at about 6.5 TB/s (at 1.9 GHz); leaving takes the point-major copy, the
-    // vectors that the blocks miss: about three passes' time, and more where a block is read again for every four
-    // vectors
+    // vectors that the blocks miss, about three passes' time
     sa.full_cost = (int)std::min(5e8, 4.0 * n * N / 3400.0);
-    sa.leave_cost = (n > 128 ? 16 : 3) * std::min(sa.full_cost, 100000000) + 114000;
+    sa.leave_cost = 3 * sa.full_cost + 114000;
     sa.leave_step = env_value("ACE_SCDM_LEAVE_STEP", 0);
     // thresholds, clocks and the step of leaving (neighbours in the workspace)
     e = cudaMemsetAsync(sa.thr, 0, L.total - L.thr, st);
