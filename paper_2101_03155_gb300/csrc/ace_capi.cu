@@ -838,12 +838,13 @@ ace_status run_chain_persistent(ace_op *op, cudaStream_t st, const DeviceTables 
   return ACE_OK;
 }
 
-// Side streams and packs per batch of a chain within ACE_SCRATCH_MB of scratch (unset: dflt_mb, negative for
-// no bound), one pack at least.
+// Side streams and packs per batch of a chain within ACE_SCRATCH_MB of scratch, one pack at least; where it is
+// not set, within dflt_mb or two packs (negative: no bound).
 void fit_scratch(size_t pack_bytes, int dflt_mb, int *nstreams, int *B) {
-  const int mb = env_int("ACE_SCRATCH_MB", dflt_mb);
-  if (mb < 0) return;
-  const int slots = (int)std::min(65535.0, std::max(1.0, std::floor(mb * 1048576.0 / (double)pack_bytes)));
+  const int mb = env_int("ACE_SCRATCH_MB", -1), least = mb < 0 ? 2 : 1;
+  const double bytes = 1048576.0 * (mb < 0 ? dflt_mb : mb);
+  if (bytes < 0.0) return;
+  const int slots = (int)std::min(65535.0, std::max((double)least, std::floor(bytes / (double)pack_bytes)));
   *nstreams = std::min(*nstreams, slots);
   *B = std::min(*B, slots / *nstreams);
 }
@@ -962,8 +963,9 @@ ace_status run_chain_f64(ace_op *op, const double *phi, const DeviceTables *tab,
   cudaStream_t st = op->stream;
   int nstreams = std::min(kSide, std::max(1, cp.streams));
   int B = std::min({65535, std::max(cp.G, cp.B), ((count + 1) / 2 + nstreams - 1) / nstreams});
-  // the pencil route has a budget of 64 MB unless set (one pack at least; 16 orbitals on 160^3, one pack of 66 MB
-  // at a time, take 90 ms instead of 83); W does not depend on the batches
+  // the pencil route has a budget of 64 MB unless set, or two packs, so that one's additions run beside the
+  // other's transforms (16 orbitals on 160^3 in packs of 66 MB: 83 ms, one at a time 90); W does not depend on
+  // the batches
   fit_scratch(sizeof(cpx<double>) * (size_t)N, pops ? -1 : 64, &nstreams, &B);
   std::vector<int4> packs;
   form_packs(op->pairs_h, cp.RB, packs);
