@@ -51,7 +51,8 @@ struct PlaneArgs {
   const cpx<T> *tw3;   // [N3] e^{-2 pi i e / N3}
   long long N;
   int n1, n2, n3;
-  int hints;           // bit 0: drop each consumed scratch plane from L2 without writing it back
+  int hints;           // bit 0: drop each consumed scratch plane from L2 without writing it back; bits 1 and 2:
+                       // fetch the orbital / W planes into L2 ahead of the accumulation
   const float *pmax;   // plane maxima [norb][n1] and orbital maxima [norb] for the plane skip
   const float *gmax;
   float skip_rel;      // > 0: planes below this fraction of the orbitals' maxima are skipped

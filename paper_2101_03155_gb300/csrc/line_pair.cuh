@@ -560,6 +560,23 @@ __device__ __forceinline__ void lp_inv_acc(const G &g, const unit *s, const Plan
   });
 }
 
+// Asks L2 for the 16-byte lines wholly inside [base, base + bytes) (one thread; no wait).
+__device__ __forceinline__ void l2_prefetch(const void *base, int bytes) {
+  const unsigned long long b = reinterpret_cast<unsigned long long>(base);
+  const unsigned long long first = (b + 15) & ~15ull;
+  const unsigned n = (unsigned)(((b + bytes) & ~15ull) - first);
+  if (n) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(first), "r"(n) : "memory");
+}
+// The orbital and W planes that the accumulation will touch, fetched while the transforms run (ACE_L2_HINTS bits 1
+// and 2, off by default: within 2% either way).  Taking the call out changes the inverse kernel's schedule: 128
+// orbitals on 96^3 11.63 -> 11.80 ms, 96 on 100x108x90 10.75 -> 10.86.
+__device__ __forceinline__ void lp_prefetch(const PlanePtrs &q, int npts, int mode) {
+  const int t = threadIdx.x;
+  if ((mode & 2) && t < 4 && !(t == 2 && q.same_a)) l2_prefetch(t == 0 ? q.fa : t == 1 ? q.fb : t == 2 ? q.fc : q.fd, 4 * npts);
+  if ((mode & 4) && t >= 4 && t < 8 && !(t == 6 && q.same_a))
+    l2_prefetch(t == 4 ? q.wa : t == 5 ? q.wb : t == 6 ? q.wc : q.wd, 4 * npts);
+}
+
 // Twiddle tables of both axes in shared memory as {c, c, s, s} units (shared when N2 = N3).
 __device__ __forceinline__ void lp_tables(int n2, int n3, int nt, const cpx<float> *t2, const cpx<float> *t3, unit *tw2,
                                           unit *tw3) {

@@ -67,6 +67,7 @@ __global__ void __launch_bounds__((PlaneOf<N2, N3>::NT), (lp_min_blocks<N2, N3>(
   if (!(a.skip_rel > 0.f && inv_plane_negligible(a.pmax, a.gmax, a.n1, i1, pk, a.skip_rel))) {
     lp_tables(N2, N3, G::NT, a.tw2, a.tw3, tw2, tw3);
     const PlanePtrs q = lp_ptrs(a, pk, (long long)i1 * (N2 * N3));
+    lp_prefetch(q, N2 * N3, a.hints);
     __syncthreads();
     lp_inv_rowsA<N3>(g, src, s, tw3);
     lp_sync(g);
