@@ -43,7 +43,7 @@ CHAIN_DRAM_BYTES_PER_BUILD = 11.03e9 * 2346 / 2666
 # changes
 DENSE_DRAM_BYTES = {"screen": 458.3e6, "M": 936.0e6, "xi": 888.3e6}
 # DRAM bytes per SCDM localisation of the 128-orbital 96^3 set (ncu, profiles/scdm_water32_96c.md)
-SCDM_DRAM_BYTES = 2649e6
+SCDM_DRAM_BYTES = 2286e6
 
 
 def _peaks():
