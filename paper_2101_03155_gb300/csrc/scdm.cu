@@ -1076,9 +1076,10 @@ cudaError_t launch_scdm(const T *psi, int n, long long N, void *ws, cudaStream_t
     if (e != cudaSuccess) return e;
     scdm_pass_kernel<T, true><<<first, kUpdNT, 0, st>>>(psi, n, N, d, sa);
     e = steps(scdm_pass_kernel<T, false>, 0, 1, n);
-  } else if (4.0 * n * N < 1e6 * env_value("ACE_SCDM_BOUNDS_MB", 70)) {
+  } else if (4.0 * n * N < 1e6 * env_value("ACE_SCDM_BOUNDS_MB", 60)) {
     // Psi stays in L2 and a pass over every point is cheaper than the bounds (ms per call, with them / without:
-    // 64 orbitals on 48^3 1.94 / 1.64, on 64^3 2.14 / 2.11; 32 on 64^3 1.35 / 1.10; on 72^3 64 take 2.2 / 3.2)
+    // 64 orbitals on 48^3 1.9 / 1.65, 32 on 64^3 1.35 / 1.09; from 60 MB on the bounds win: 64 on 64^3 2.01 / 2.10,
+    // on 72^3 1.97 / 3.2)
     e = blocks(scdm_norm_kernel<false, false>, 0, kUpdNT, &first);
     if (e == cudaSuccess) e = blocks(scdm_full_kernel, 0, kUpdNT, &next);
     if (e != cudaSuccess) return e;
