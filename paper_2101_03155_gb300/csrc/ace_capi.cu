@@ -606,9 +606,9 @@ ChainParams chain_params(const ace_desc &d, bool fp64) {
     for (const auto &e : g_tuned)
       if (e.first == k) c = e.second;
   }
-  const int batch = env_int("ACE_PLANE_BATCH", 0);
-  c.G = std::max(1, env_int("ACE_GROUP", batch > 0 ? 1 : c.G));
-  c.B = std::max(c.G, batch > 0 ? batch : c.B);
+  const int batch = env_int("ACE_PLANE_BATCH", -1);  // overrides both fields of the table
+  c.G = std::max(1, env_int("ACE_GROUP", batch >= 0 ? 1 : c.G));
+  c.B = std::max(c.G, batch >= 0 ? batch : c.B);
   c.streams = std::min(kSide, std::max(1, env_int("ACE_STREAMS", c.streams)));
   c.persist_mb = std::max(0, env_int("ACE_L2_PERSIST_MB", c.persist_mb));
   c.RB = std::max(1, env_int("ACE_ROW_BLOCK", c.RB));

@@ -39,6 +39,8 @@ t1, n1, W1 = chain()
 import os
 os.environ["ACE_PLANE_BATCH"] = "1"
 n2 = chain()[1]
+os.environ["ACE_PLANE_BATCH"] = "0"
+assert chain()[1] == n2  # at least one pack
 print(t0, t1, n0, n1, n2, p["row_block"], int(np.array_equal(W0, W1)))
 """
 
